@@ -315,7 +315,8 @@ cudaError_t launch_rhs(const Geom &g, const double *f, const double *u0, const d
 cudaError_t launch_grad_rhs(const Geom &g, const double *lam, double *gf, double *gu0,
                             double *gup, cudaStream_t st);
 cudaError_t launch_grad_a(const Geom &g, const double *lam, const double *u, const double *u0,
-                          double *gface_x, double *gface_y, double *grad, cudaStream_t st);
+                          double *gface_x, double *gface_y, double *scratch, long long cap,
+                          double *grad, cudaStream_t st);
 
 // preconditioner pipeline: z = P^-1 v (v may be double, z double or float)
 struct PrecPlan {

@@ -1733,7 +1733,9 @@ int st_grad_a(st_handle *h, const double *lam_dev, const double *u_dev, const do
   if (h->g.dim == 3) return ST_ERR_ARG;  // the face gradient is written for 1D and 2D grids
   ProfScope prof_scope(h);
   ST_ENTER(h);
-  ST_TRY(launch_grad_a(h->g, lam_dev, u_dev, u0_dev, h->gfx, h->gfy, grad_dev, h->stream));
+  // the stencil-output vector is free between solves: the partial face sums go there
+  ST_TRY(launch_grad_a(h->g, lam_dev, u_dev, u0_dev, h->gfx, h->gfy, h->q, h->g.N, grad_dev,
+                       h->stream));
   return ST_OK;
 }
 

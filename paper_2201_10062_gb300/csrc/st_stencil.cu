@@ -485,18 +485,44 @@ __global__ void __launch_bounds__(kNT, D3 ? 3 : 4) k_stencil_df(Geom g, const fl
   }
 }
 
+// Time levels per thread of the right-hand-side and gradient kernels: a thread keeps one node and
+// walks this many levels, so a level's plane is read once per chunk (and not once as f^(k) and once
+// as f^(k-1)), and no index is recovered by a division (assembly, its adjoint and the face
+// gradients at 255^2 x 128: 369 -> 250 us for the three calls; one element per thread with a 64-bit
+// division each, and one unchunked walk for the faces, before).
+constexpr int kRhsLevels = 16;
+
 // f_H (Sec. 1 for theta, Sec. 4 with the start-up history moved into blocks 1-2 for BDF2).
-__global__ void k_rhs(Geom g, const double *__restrict__ f, const double *__restrict__ u0,
-                      const double *__restrict__ uprev, const double *__restrict__ extra,
-                      double *__restrict__ fH) {
-  const long long N = g.N, m = g.m;
-  const double tau = g.tau;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < N;
-       e += (long long)gridDim.x * blockDim.x) {
-    const long long k = e / m, p = e - k * m;
-    double r;
-    if (g.scheme == ST_THETA) {
-      r = g.theta * tau * f[(k + 1) * m + p] + (1.0 - g.theta) * tau * f[k * m + p];
+// Bound by memory (24 bytes per unknown with an extra term) and, close behind, by the float64
+// pipe: two fused multiply-adds per unknown, one where 1 - theta = 0.  Nodes by the first grid
+// axis, chunks of kRhsLevels levels by the second.
+template <bool EXTRA>
+__global__ void __launch_bounds__(256)
+    k_rhs(Geom g, const double *__restrict__ f, const double *__restrict__ u0,
+          const double *__restrict__ uprev, const double *__restrict__ extra,
+          double *__restrict__ fH) {
+  const long long m = g.m;
+  const long long p = blockIdx.x * 256LL + threadIdx.x;
+  if (p >= m) return;
+  const int k0 = blockIdx.y * kRhsLevels, k1 = min(g.n, k0 + kRhsLevels);
+  const bool theta = g.scheme == ST_THETA;
+  const double a = theta ? g.theta * g.tau : g.tau;
+  const double b = theta ? (1.0 - g.theta) * g.tau : 0.0;
+  const bool two = theta && g.theta != 1.0;  // f^(k-1) enters block k
+  const double *fp = f + (long long)k0 * m + p;
+  const double *ep = EXTRA ? extra + (long long)k0 * m + p : nullptr;
+  double *op = fH + (long long)k0 * m + p;
+  double f0 = two ? __ldg(fp) : 0.0;
+#pragma unroll 4
+  for (int k = k0; k < k1; ++k, op += m) {
+    fp += m;
+    const double f1 = __ldg(fp);
+    double r = EXTRA ? __ldg(ep) : 0.0;
+    if (EXTRA) ep += m;
+    if (two) r = EXTRA ? fma(b, f0, r) : b * f0;
+    r = (two || EXTRA) ? fma(a, f1, r) : a * f1;
+    f0 = f1;
+    if (theta) {
       if (k == 0) {
         const int i = (int)(p % g.mx), row = (int)(p / g.mx);
         const int jz = row / g.my, jy = row - jz * g.my;
@@ -505,12 +531,10 @@ __global__ void k_rhs(Geom g, const double *__restrict__ f, const double *__rest
         r += c - (1.0 - g.theta) * Kc;
       }
     } else {
-      r = tau * f[(k + 1) * m + p];
       if (k == 0) r += 2.0 * u0[p] - 0.5 * (uprev ? uprev[p] : u0[p]);
       if (k == 1) r -= 0.5 * u0[p];
     }
-    if (extra) r += extra[e];
-    fH[e] = r;
+    *op = r;
   }
 }
 
@@ -518,25 +542,31 @@ __global__ void k_rhs(Geom g, const double *__restrict__ f, const double *__rest
 // f (at t_0..t_n), u0 and (BDF2) u^(-1).
 //   theta: f_H block k = theta tau f^(k) + (1-theta) tau f^(k-1), block 1 += (I - (1-theta) tau K) u0
 //   BDF2:  f_H block k = tau f^(k), block 1 += 2 u0 - u^(-1)/2, block 2 += -u0/2
-__global__ void k_grad_rhs(Geom g, const double *__restrict__ lam, double *__restrict__ gf,
-                           double *__restrict__ gu0, double *__restrict__ gup) {
-  const long long m = g.m, total = (long long)(g.n + 1) * m;
+// Same walk as k_rhs, over the n + 1 levels of f.
+__global__ void __launch_bounds__(256)
+    k_grad_rhs(Geom g, const double *__restrict__ lam, double *__restrict__ gf,
+               double *__restrict__ gu0, double *__restrict__ gup) {
+  const long long m = g.m;
+  const long long p = blockIdx.x * 256LL + threadIdx.x;
+  if (p >= m) return;
   const int n = g.n;
-  const double tau = g.tau;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const long long k = e / m, p = e - k * m;  // f^(k), k = 0..n
-    double r = 0.0;
-    if (g.scheme == ST_THETA) {
-      if (k >= 1) r += g.theta * tau * lam[(k - 1) * m + p];
-      if (k <= n - 1) r += (1.0 - g.theta) * tau * lam[k * m + p];
-    } else {
-      if (k >= 1) r = tau * lam[(k - 1) * m + p];
-    }
-    gf[e] = r;
+  const int k0 = blockIdx.y * kRhsLevels, k1 = min(n + 1, k0 + kRhsLevels);
+  const bool theta = g.scheme == ST_THETA;
+  const double a = theta ? g.theta * g.tau : g.tau;
+  const double b = theta ? (1.0 - g.theta) * g.tau : 0.0;
+  const bool two = theta && g.theta != 1.0;
+  const double *lp = lam + (long long)k0 * m + p;
+  double *op = gf + (long long)k0 * m + p;
+  double l0 = k0 > 0 ? __ldg(lp - m) : 0.0;  // block k - 1 (0-based), paired with theta tau
+#pragma unroll 4
+  for (int k = k0; k < k1; ++k, lp += m, op += m) {
+    const double l1 = k < n ? __ldg(lp) : 0.0;
+    double r = a * l0;
+    if (two) r = fma(b, l1, r);
+    *op = r;
+    l0 = l1;
     if (k == 0) {
-      const double l1 = lam[p];
-      if (g.scheme == ST_THETA) {
+      if (theta) {
         if (gu0) {
           const int i = (int)(p % g.mx), row = (int)(p / g.mx);
           const int jz = row / g.my, jy = row - jz * g.my;
@@ -559,9 +589,18 @@ __global__ void k_grad_rhs(Geom g, const double *__restrict__ lam, double *__res
 // (j,i)] when j < my and y-face (j, i) [between (j-1,i) and (j,i)] when i < mx.
 // cx/cy already hold tau*a/h^2; a_face enters linearly, so tau/h^2 = c/a_face is recovered from
 // the unit-coefficient spacing passed in sx, sy.
-__global__ void k_grad_faces(Geom g, const double *__restrict__ lam, const double *__restrict__ u,
-                             const double *__restrict__ u0, double sx, double sy,
-                             double *__restrict__ gx, double *__restrict__ gy) {
+//
+// Bound by the float64 pipe: with E = lam_p - lam_q and D = u_p - u_q the sum over k is
+// theta sum E_k D_k + (1 - theta) sum E_k D_{k-1}, so a face takes two differences and two fused
+// multiply-adds per level (one where theta = 1 or BDF2) and w is never formed.  The levels are
+// cut into chunks over the grid's third axis (a 255^2 grid alone has fewer threads than the chip
+// holds); every chunk writes its own partial face sums, [chunk][face], added in order by
+// k_grad_nodes.
+template <bool TWO>
+__global__ void __launch_bounds__(256)
+    k_grad_faces(Geom g, const double *__restrict__ lam, const double *__restrict__ u,
+                 const double *__restrict__ u0, double sx, double sy, int kc,
+                 double *__restrict__ gx, double *__restrict__ gy) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int mx = g.mx, my = g.my;
@@ -571,49 +610,62 @@ __global__ void k_grad_faces(Geom g, const double *__restrict__ lam, const doubl
   const bool doY = (g.dim == 2) && (i < mx);
   if (!doX && !doY) return;
   const double th = (g.scheme == ST_THETA) ? g.theta : 1.0;
-  // node indices (or -1 for a boundary node)
-  const long long pc = (i < mx && j < my) ? (long long)j * mx + i : -1;
-  const long long pl = (i > 0 && j < my) ? (long long)j * mx + i - 1 : -1;
-  const long long pd = (j > 0 && i < mx) ? (long long)(j - 1) * mx + i : -1;
-  double ax = 0.0, ay = 0.0;
-  double uc_prev = pc >= 0 ? u0[pc] : 0.0, ul_prev = pl >= 0 ? u0[pl] : 0.0,
-         ud_prev = pd >= 0 ? u0[pd] : 0.0;
-  for (int k = 0; k < g.n; ++k) {
-    const double *L = lam + (long long)k * m;
-    const double *U = u + (long long)k * m;
-    const double uc = pc >= 0 ? U[pc] : 0.0;
-    const double ul = pl >= 0 ? U[pl] : 0.0;
-    const double ud = pd >= 0 ? U[pd] : 0.0;
-    const double wc = th * uc + (1.0 - th) * uc_prev;
-    const double wl = th * ul + (1.0 - th) * ul_prev;
-    const double wd = th * ud + (1.0 - th) * ud_prev;
-    const double lc = pc >= 0 ? L[pc] : 0.0;
+  // a node outside the grid has value zero; pc, pl, pd: the face's own node and its west and
+  // south neighbours
+  const bool hc = i < mx && j < my, hl = i > 0 && j < my, hd = j > 0 && i < mx;
+  const long long pc = (long long)j * mx + i, pl = pc - 1, pd = pc - mx;
+  const int k0 = blockIdx.z * kc, k1 = min(g.n, k0 + kc);
+  double dx = 0.0, dy = 0.0;  // D of the level before
+  if (TWO) {
+    const double *U = k0 > 0 ? u + (long long)(k0 - 1) * m : u0;
+    const double uc = hc ? U[pc] : 0.0;
+    dx = uc - (hl ? U[pl] : 0.0);
+    dy = uc - (hd ? U[pd] : 0.0);
+  }
+  double ax = 0.0, ay = 0.0, bx = 0.0, by = 0.0;
+  const double *L = lam + (long long)k0 * m, *U = u + (long long)k0 * m;
+#pragma unroll 2
+  for (int k = k0; k < k1; ++k, L += m, U += m) {
+    const double uc = hc ? __ldg(U + pc) : 0.0, lc = hc ? __ldg(L + pc) : 0.0;
     if (doX) {
-      const double ll = pl >= 0 ? L[pl] : 0.0;
-      ax += (lc - ll) * (wc - wl);
+      const double e = lc - (hl ? __ldg(L + pl) : 0.0), d = uc - (hl ? __ldg(U + pl) : 0.0);
+      ax = fma(e, d, ax);
+      if (TWO) bx = fma(e, dx, bx);
+      dx = d;
     }
     if (doY) {
-      const double ld_ = pd >= 0 ? L[pd] : 0.0;
-      ay += (lc - ld_) * (wc - wd);
+      const double e = lc - (hd ? __ldg(L + pd) : 0.0), d = uc - (hd ? __ldg(U + pd) : 0.0);
+      ay = fma(e, d, ay);
+      if (TWO) by = fma(e, dy, by);
+      dy = d;
     }
-    uc_prev = uc;
-    ul_prev = ul;
-    ud_prev = ud;
   }
-  if (doX) gx[(long long)j * (mx + 1) + i] = -sx * ax;
-  if (doY) gy[(long long)j * mx + i] = -sy * ay;
+  if (TWO) {
+    ax = th * ax + (1.0 - th) * bx;
+    ay = th * ay + (1.0 - th) * by;
+  }
+  const long long fx = (long long)(mx + 1) * my, fy = (long long)mx * (my + 1);
+  if (doX) gx[blockIdx.z * fx + (long long)j * (mx + 1) + i] = -sx * ax;
+  if (doY) gy[blockIdx.z * fy + (long long)j * mx + i] = -sy * ay;
 }
 
-// Nodal gradient: each face gradient is split half/half between its two nodes.
-__global__ void k_grad_nodes(int dim, int mx, int my, const double *__restrict__ gx,
+// Nodal gradient: each face gradient (the sum of its chunks' partial sums, in order) is split
+// half/half between its two nodes.
+__global__ void k_grad_nodes(int dim, int mx, int my, int nchunk, const double *__restrict__ gx,
                              const double *__restrict__ gy, double *__restrict__ grad) {
+  const long long nfx = (long long)(mx + 1) * my, nfy = (long long)mx * (my + 1);
+  auto sum = [&](const double *p, long long stride) -> double {
+    double s = p[0];
+    for (int c = 1; c < nchunk; ++c) s += p[c * stride];
+    return s;
+  };
   const int I = blockIdx.x * blockDim.x + threadIdx.x;  // 0..mx+1
   const int J = blockIdx.y * blockDim.y + threadIdx.y;  // 0..my+1 (0 in 1D)
   if (dim == 1) {
     if (I > mx + 1 || J > 0) return;
     double s = 0.0;
-    if (I <= mx) s += 0.5 * gx[I];      // face I: between nodes I and I+1
-    if (I >= 1) s += 0.5 * gx[I - 1];   // face I-1: between nodes I-1 and I
+    if (I <= mx) s += 0.5 * sum(gx + I, nfx);      // face I: between nodes I and I+1
+    if (I >= 1) s += 0.5 * sum(gx + I - 1, nfx);   // face I-1: between nodes I-1 and I
     grad[I] = s;
     return;
   }
@@ -622,14 +674,14 @@ __global__ void k_grad_nodes(int dim, int mx, int my, const double *__restrict__
   // x-faces lie on interior rows j = J-1; face (j, i) joins nodal columns i and i+1
   if (J >= 1 && J <= my) {
     const int j = J - 1;
-    if (I <= mx) s += 0.5 * gx[(long long)j * (mx + 1) + I];
-    if (I >= 1) s += 0.5 * gx[(long long)j * (mx + 1) + I - 1];
+    if (I <= mx) s += 0.5 * sum(gx + (long long)j * (mx + 1) + I, nfx);
+    if (I >= 1) s += 0.5 * sum(gx + (long long)j * (mx + 1) + I - 1, nfx);
   }
   // y-faces lie on interior columns i = I-1; face (j, i) joins nodal rows j and j+1
   if (I >= 1 && I <= mx) {
     const int i = I - 1;
-    if (J <= my) s += 0.5 * gy[(long long)J * mx + i];
-    if (J >= 1) s += 0.5 * gy[(long long)(J - 1) * mx + i];
+    if (J <= my) s += 0.5 * sum(gy + (long long)J * mx + i, nfy);
+    if (J >= 1) s += 0.5 * sum(gy + (long long)(J - 1) * mx + i, nfy);
   }
   grad[(long long)J * (mx + 2) + I] = s;
 }
@@ -715,40 +767,57 @@ template cudaError_t launch_stencil<float>(const Geom &, int, const float *, dou
 
 cudaError_t launch_rhs(const Geom &g, const double *f, const double *u0, const double *uprev,
                        const double *extra, double *fH, cudaStream_t st) {
-  long long blocks = (g.N + 255) / 256;
-  if (blocks > 152LL * 16) blocks = 152LL * 16;
+  const dim3 gr((unsigned)((g.m + 255) / 256), (unsigned)((g.n + kRhsLevels - 1) / kRhsLevels));
   prof_begin(KC_AUX, st);
-  k_rhs<<<(unsigned)blocks, 256, 0, st>>>(g, f, u0, uprev, extra, fH);
+  if (extra)
+    k_rhs<true><<<gr, 256, 0, st>>>(g, f, u0, uprev, extra, fH);
+  else
+    k_rhs<false><<<gr, 256, 0, st>>>(g, f, u0, uprev, extra, fH);
   prof_end(st);
   return cudaGetLastError();
 }
 
 cudaError_t launch_grad_rhs(const Geom &g, const double *lam, double *gf, double *gu0,
                             double *gup, cudaStream_t st) {
-  long long blocks = ((long long)(g.n + 1) * g.m + 255) / 256;
-  if (blocks > 152LL * 16) blocks = 152LL * 16;
+  const dim3 gr((unsigned)((g.m + 255) / 256), (unsigned)(g.n / kRhsLevels + 1));
   prof_begin(KC_AUX, st);
-  k_grad_rhs<<<(unsigned)blocks, 256, 0, st>>>(g, lam, gf, gu0, gup);
+  k_grad_rhs<<<gr, 256, 0, st>>>(g, lam, gf, gu0, gup);
   prof_end(st);
   return cudaGetLastError();
 }
 
+// scratch: room for cap doubles, used for the chunks' partial face sums when there is more than one
 cudaError_t launch_grad_a(const Geom &g, const double *lam, const double *u, const double *u0,
-                          double *gface_x, double *gface_y, double *grad, cudaStream_t st) {
+                          double *gface_x, double *gface_y, double *scratch, long long cap,
+                          double *grad, cudaStream_t st) {
   const double hx = 1.0 / (g.mx + 1), hy = 1.0 / (g.my + 1);
   const double sx = g.tau / (hx * hx), sy = g.tau / (hy * hy);
   dim3 b(32, 8);
   const int fy = (g.dim == 2) ? g.my + 1 : 1;
-  dim3 gr((g.mx + 1 + 31) / 32, (fy + 7) / 8);
+  const long long nfx = (long long)(g.mx + 1) * g.my, nfy = (long long)g.mx * (g.my + 1);
+  const long long tiles = ((g.mx + 1 + 31) / 32) * (long long)((fy + 7) / 8);
+  // chunks of levels: enough blocks for eight per SM, at least eight levels each (a chunk rereads
+  // one level), and no more than the scratch holds
+  long long nc = (152LL * 8 + tiles - 1) / tiles;
+  if (nc > (g.n + 7) / 8) nc = (g.n + 7) / 8;
+  if (nc > cap / (nfx + nfy)) nc = cap / (nfx + nfy);
+  if (nc < 1) nc = 1;
+  const int kc = (int)((g.n + nc - 1) / nc);
+  nc = (g.n + kc - 1) / kc;
+  double *gx = nc > 1 ? scratch : gface_x, *gy = nc > 1 ? scratch + nc * nfx : gface_y;
+  dim3 gr((g.mx + 1 + 31) / 32, (fy + 7) / 8, (unsigned)nc);
   prof_begin(KC_AUX, st);
-  k_grad_faces<<<gr, b, 0, st>>>(g, lam, u, u0, sx, sy, gface_x, gface_y);
+  if (g.scheme == ST_THETA && g.theta != 1.0)
+    k_grad_faces<true><<<gr, b, 0, st>>>(g, lam, u, u0, sx, sy, kc, gx, gy);
+  else
+    k_grad_faces<false><<<gr, b, 0, st>>>(g, lam, u, u0, sx, sy, kc, gx, gy);
   prof_end(st);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int ny = (g.dim == 2) ? g.my + 2 : 1;
   dim3 gn((g.mx + 2 + 31) / 32, (ny + 7) / 8);
   prof_begin(KC_AUX, st);
-  k_grad_nodes<<<gn, b, 0, st>>>(g.dim, g.mx, g.my, gface_x, gface_y, grad);
+  k_grad_nodes<<<gn, b, 0, st>>>(g.dim, g.mx, g.my, (int)nc, gx, gy, grad);
   prof_end(st);
   return cudaGetLastError();
 }
