@@ -38,12 +38,15 @@ __global__ void k_zero3_gated(long long N, df *a, df *b, df *c, const State *S) 
   }
 }
 
-__global__ void k_df_to_double_gated(long long N, const df *__restrict__ src,
+// padded double-float x into the caller's contiguous float64 vector
+__global__ void k_df_to_double_gated(unsigned total, int mx, int px, const df *__restrict__ src,
                                      double *__restrict__ dst, const State *S) {
   if (!(S->finish && !S->done)) return;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < N;
-       e += (long long)gridDim.x * blockDim.x)
-    dst[e] = df_to_double(src[e]);
+  for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < total;
+       e += gridDim.x * blockDim.x) {
+    const unsigned l = e / (unsigned)mx, i = e - l * (unsigned)mx;
+    dst[e] = df_to_double(src[(long long)l * px + i]);
+  }
 }
 
 // End of one trip of an instance's loop: continue while the instance is not done and the trip
@@ -106,11 +109,12 @@ cudaError_t iteration(st_handle *h, int b, cudaStream_t st) {
 cudaError_t refine(st_handle *h, const double *fH, double *u, cudaStream_t st) {
   const Geom &g = h->g;
   cudaError_t e;
-  k_df_to_double_gated<<<kStreamBlocks, kNT, 0, st>>>(g.N, h->Xdf, u, h->S);
+  k_df_to_double_gated<<<kStreamBlocks, kNT, 0, st>>>((unsigned)g.N, g.mx, g.px, h->Xdf, u,
+                                                      h->S);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = launch_resid_outer(g, u, (df *)h->V[0], fH, h->S, h->partials, st)) != cudaSuccess)
     return e;
-  k_zero3_gated<<<kStreamBlocks, kNT, 0, st>>>(g.N, (df *)h->D[0], (df *)h->D[1], (df *)h->V[1],
+  k_zero3_gated<<<kStreamBlocks, kNT, 0, st>>>(g.Np, (df *)h->D[0], (df *)h->D[1], (df *)h->V[1],
                                               h->S);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   return launch_prec<float, df, float>(g, h->pp, (const df *)h->V[0], (float *)h->Z[0], h->S,
@@ -317,11 +321,11 @@ int st_solve_batch(st_batch *b, const double *const *fH_devs, double *const *u_d
     S.inner_floor = inner_floor();
     S.target = std::max(0.5 * tol, S.inner_floor);
     BT_TRY(cudaMemcpyAsync(h->S, h->hS, kStatePushBytes, cudaMemcpyHostToDevice, s));
-    BT_TRY(cudaMemsetAsync(h->Xdf, 0, g.N * sizeof(df), s));
+    BT_TRY(cudaMemsetAsync(h->Xdf, 0, g.Np * sizeof(df), s));
     BT_TRY(cudaMemsetAsync(u_devs[i], 0, g.N * sizeof(double), s));
-    BT_TRY(cudaMemsetAsync(h->D[0], 0, g.N * sizeof(df), s));
-    BT_TRY(cudaMemsetAsync(h->D[1], 0, g.N * sizeof(df), s));
-    BT_TRY(cudaMemsetAsync(h->V[1], 0, g.N * sizeof(df), s));
+    BT_TRY(cudaMemsetAsync(h->D[0], 0, g.Np * sizeof(df), s));
+    BT_TRY(cudaMemsetAsync(h->D[1], 0, g.Np * sizeof(df), s));
+    BT_TRY(cudaMemsetAsync(h->V[1], 0, g.Np * sizeof(df), s));
     BT_TRY(launch_flip_to_df(g, fH_devs[i], (df *)h->V[0], s));
     BT_TRY(launch_norm2(g.N, fH_devs[i], h->S, h->partials, s));
     BT_TRY((launch_prec<float, df, float>(g, h->pp, (const df *)h->V[0], (float *)h->Z[0], h->S,

@@ -29,6 +29,12 @@ struct Geom {
   const df *czd;
   int c_uniform;        // every face coefficient equals c_uni (constant a, equal spacing)
   df c_uni;             // that coefficient as a double-float pair
+  // float32 and double-float vectors of the mixed path are stored with one padding slot after each
+  // x line: px = mx + 1 (a power of two) slots a line, mp = px*my*mz a time level, Np = n*mp in
+  // all.  Lines, planes and levels then start on 16-byte boundaries (tensor copies need that),
+  // and the padding holds zeros: the Dirichlet values the stencil reads on either side of a line.
+  int px;
+  long long mp, Np;
 };
 
 // The six face coefficients (tau a / h^2) around interior node (i, jy, jz): west/east along x,
@@ -381,13 +387,27 @@ int setup_handle(const st_problem *prob, st_handle **out, int ugroup);
 void close_device(int dev);
 bool device_closed(int dev);
 
-bool time_tc_supported(int n);
-size_t time_tc_sop_halves(int n);
-void time_tc_build_sop(int n, unsigned short *out);
-cudaError_t launch_time_tc(float *data, const Geom &g, const Spec<float> &sp,
-                           const unsigned short *sop, State *S, int tmode, double *partials,
-                           int gk, cudaStream_t st);
-bool dst_tc_supported(int len);
+// Tensor-core DSTs on padded float32 vectors (st_dst_tma.cu).  dst_tma_supported: the axis length
+// has a tile shape (16..256); images: the fp16 operand image of S_len the kernels load into tensor
+// memory, in halves, and its host builder.
+bool dst_tma_supported(int len);
+size_t dst_tma_image_halves(int len);
+void dst_tma_build_image(int len, unsigned short *out);
+// time DST, 1/p scaling with <v, P^-1 v> (and the MINRES scalar step of tmode), time DST, in place
+cudaError_t launch_time_tma(float *data, const Geom &g, const Spec<float> &sp,
+                            const unsigned short *img, State *S, int tmode, double *partials,
+                            int gk, cudaStream_t st);
+// one DST-I along x (in place, or into a caller's contiguous vector), y or z (in place), and along
+// time alone (in -> out)
+cudaError_t launch_dst_tma_x(float *data, const Geom &g, const unsigned short *img, State *S,
+                             int gk, cudaStream_t st, float *user = nullptr);
+cudaError_t launch_dst_tma_y(float *data, const Geom &g, const unsigned short *img, State *S,
+                             int gk, cudaStream_t st);
+cudaError_t launch_dst_tma_z(float *data, const Geom &g, const unsigned short *img, State *S,
+                             int gk, cudaStream_t st);
+cudaError_t launch_time_tma_single(const float *in, float *out, const Geom &g,
+                                   const unsigned short *img, State *S, int gk, cudaStream_t st);
+int time_tc_grid();
 // float64-accurate time stage on the tensor cores (integer digits of S_n and of the double-float
 // data, exact float32 accumulation per digit group; k_time_tcd)
 bool time_tcd_supported(int n);
@@ -403,15 +423,6 @@ void time_tc_long_build(int n, unsigned short *out);
 cudaError_t launch_time_tc_long(float *data, const Geom &g, const Spec<float> &sp,
                                 const unsigned short *A, State *S, int tmode, double *partials,
                                 int gk, cudaStream_t st);
-cudaError_t launch_dst_tc_y(float *data, const Geom &g, const unsigned short *sop, State *S,
-                            int gk, cudaStream_t st);
-cudaError_t launch_dst_tc_z(float *data, const Geom &g, const unsigned short *sop, State *S,
-                            int gk, cudaStream_t st);
-cudaError_t launch_dst_tc_x(float *data, const Geom &g, const unsigned short *sop, State *S,
-                            int gk, cudaStream_t st);
-bool dst_tc_len_supported(int len);
-cudaError_t launch_time_tc_single(const float *in, float *out, const Geom &g,
-                                  const unsigned short *sop, State *S, int gk, cudaStream_t st);
 
 // energy mode of the time kernel's last block
 enum { TM_NONE = 0, TM_INIT = 1, TM_ITER = 2, TM_RESTART = 3 };
@@ -436,6 +447,8 @@ cudaError_t launch_prec_lanczos(const Geom &g, const PrecPlan &pp, const Tin *q,
 template <class Tc, class Tin, class Tout>
 cudaError_t launch_prec(const Geom &g, const PrecPlan &pp, const Tin *v, Tout *z, State *S,
                         int tmode, double *partials, cudaStream_t st);
+cudaError_t launch_prec_user(const Geom &g, const PrecPlan &pp, const double *v, float *scratch,
+                             float *out, State *S, double *partials, cudaStream_t st);
 int time_blocks_for(const Geom &g, const PrecPlan &pp, bool fp32);
 int time_J_default(int n, bool fp32);
 // the spatial DST passes alone, ungated: float32 (fp32), else the float64 path's engine
@@ -466,7 +479,7 @@ cudaError_t launch_resid_outer(const Geom &g, const double *x, df *r_out, const 
 cudaError_t launch_update_group(st_handle *h, cudaStream_t st);
 float *zslot(st_handle *h, int s);
 cudaError_t launch_flip_to_df(const Geom &g, const double *src, df *dst, cudaStream_t st);
-cudaError_t launch_df_to_double(long long N, const df *src, double *dst, cudaStream_t st);
+cudaError_t launch_df_to_double(const Geom &g, const df *src, double *dst, cudaStream_t st);
 
 // real part used when a transform reads its input in the compute type
 template <class Tc>
@@ -592,7 +605,9 @@ struct st_handle {
   st::df *Xdf;           // ST_MIXED: double-float solution accumulator
   double *partials;      // per-block partial sums
   st::State *S;          // device scalars
-  double *hbuf_in, *hbuf_out;  // device staging for st_solve_host
+  // device staging for st_solve_host and st_solve_transpose; hbuf_out is q in ST_MIXED (the float64
+  // iterate is only needed between inner runs, when q is free)
+  double *hbuf_in, *hbuf_out;
   double *gfx, *gfy;     // face-gradient scratch for st_grad_a
   void *cheb;            // P_theta, 2D/3D varying a: Chebyshev scalars and scratch vectors
   // the tensor-core operand images the handle was built with (the autotuner may switch a stage
@@ -608,6 +623,9 @@ struct st_handle {
   // z_j lives in slot (j - 1) % (ugroup + 1) of Z[0], Z[1], Zx[0], ...
   int ugroup;
   float *Zx[st::kUpdRing - 1];
+  // ST_MIXED: the one allocation behind Z[0], Z[1] and Zx (zero slots before the first line, then the
+  // padded vectors); zscratch: a padded float32 vector for st_apply_prec_f32
+  float *zslab, *zscratch;
 };
 
 

@@ -213,20 +213,26 @@ __global__ void __launch_bounds__(kNT, ILP == 1 ? 4 : 3)
   }
 }
 
-__global__ void k_flip_to_df(long long m, int n, const double *__restrict__ src,
-                             df *__restrict__ dst) {
-  const long long total = (long long)n * m;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const long long k = e / m, p = e - k * m;
-    dst[(long long)(n - 1 - k) * m + p] = df_of_double(src[e]);
+// between a caller's contiguous float64 vector and a padded double-float one: element e of the
+// float64 vector is element i of x line l
+__global__ void k_flip_to_df(unsigned total, int mx, int px, unsigned rows, int n,
+                             const double *__restrict__ src, df *__restrict__ dst) {
+  for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < total;
+       e += gridDim.x * blockDim.x) {
+    const unsigned l = e / (unsigned)mx, i = e - l * (unsigned)mx;
+    const unsigned k = l / rows, r = l - k * rows;
+    dst[(long long)((unsigned)(n - 1) - k) * rows * px + (long long)r * px + i] =
+        df_of_double(src[e]);
   }
 }
 
-__global__ void k_df_to_double(long long N, const df *__restrict__ src, double *__restrict__ dst) {
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < N;
-       e += (long long)gridDim.x * blockDim.x)
-    dst[e] = df_to_double(src[e]);
+__global__ void k_df_to_double(unsigned total, int mx, int px, const df *__restrict__ src,
+                               double *__restrict__ dst) {
+  for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < total;
+       e += gridDim.x * blockDim.x) {
+    const unsigned l = e / (unsigned)mx, i = e - l * (unsigned)mx;
+    dst[e] = df_to_double(src[(long long)l * px + i]);
+  }
 }
 }  // namespace
 
@@ -325,10 +331,10 @@ cudaError_t launch_update_group(st_handle *h, cudaStream_t st) {
   for (int s = 0; s < zr.len; ++s) zr.p[s] = zslot(h, s);
   prof_begin(KC_UPDATE, st);
   if (update_ilp() == 2)
-    k_update_group_df<2><<<kStreamBlocks, kNT, 0, st>>>(h->g.N, zr, (df *)h->D[0],
+    k_update_group_df<2><<<kStreamBlocks, kNT, 0, st>>>(h->g.Np, zr, (df *)h->D[0],
                                                         (df *)h->D[1], h->Xdf, h->S);
   else
-    k_update_group_df<1><<<kStreamBlocks, kNT, 0, st>>>(h->g.N, zr, (df *)h->D[0],
+    k_update_group_df<1><<<kStreamBlocks, kNT, 0, st>>>(h->g.Np, zr, (df *)h->D[0],
                                                         (df *)h->D[1], h->Xdf, h->S);
   prof_end(st);
   return cudaGetLastError();
@@ -336,14 +342,15 @@ cudaError_t launch_update_group(st_handle *h, cudaStream_t st) {
 
 cudaError_t launch_flip_to_df(const Geom &g, const double *src, df *dst, cudaStream_t st) {
   prof_begin(KC_AUX, st);
-  k_flip_to_df<<<kStreamBlocks, kNT, 0, st>>>(g.m, g.n, src, dst);
+  k_flip_to_df<<<kStreamBlocks, kNT, 0, st>>>((unsigned)g.N, g.mx, g.px, (unsigned)(g.my * g.mz),
+                                              g.n, src, dst);
   prof_end(st);
   return cudaGetLastError();
 }
 
-cudaError_t launch_df_to_double(long long N, const df *src, double *dst, cudaStream_t st) {
+cudaError_t launch_df_to_double(const Geom &g, const df *src, double *dst, cudaStream_t st) {
   prof_begin(KC_AUX, st);
-  k_df_to_double<<<kStreamBlocks, kNT, 0, st>>>(N, src, dst);
+  k_df_to_double<<<kStreamBlocks, kNT, 0, st>>>((unsigned)g.N, g.mx, g.px, src, dst);
   prof_end(st);
   return cudaGetLastError();
 }
@@ -473,7 +480,7 @@ int partials_needed(const Geom &g) {
   if (a > r) r = a;
   const int b = time_blocks_for(g, PrecPlan{}, false);
   const int c = time_blocks_for(g, PrecPlan{}, true);
-  const int d = (int)((g.m + 15) / 16);
+  const int d = (int)((g.mp + 15) / 16);
   if (b > r) r = b;
   if (c > r) r = c;
   if (d > r) r = d;
@@ -490,6 +497,9 @@ Geom geom_of(const st_problem *p) {
   g.n = p->n;
   g.m = (long long)g.mx * g.my * g.mz;
   g.N = g.m * g.n;
+  g.px = g.mx + 1;
+  g.mp = (long long)g.px * g.my * g.mz;
+  g.Np = g.mp * g.n;
   g.scheme = p->scheme;
   g.tau = p->T / p->n;
   g.theta = (p->scheme == ST_THETA) ? p->theta : 1.0;
@@ -525,29 +535,50 @@ size_t cheb_coef_bytes(const Geom &g, int deg) {
   return ((size_t)deg * g.n * 2 * (sizeof(double) + sizeof(float)) + 255) / 256 * 256;
 }
 
+// zero slots in front of the first z vector of the mixed path (the stencil reads one slot to the
+// left of a line; 256 bytes keep the vectors aligned)
+constexpr size_t kZGuard = 64;
+
+// The z vectors of a mixed handle: one allocation for the whole ring.  Each takes Np slots; the
+// padding of a full ring is counted whatever the group, so every further pending z costs N floats.
+size_t zslab_floats(const Geom &g, int ugroup) {
+  return kZGuard + (size_t)(ugroup + 1) * (size_t)g.N +
+         (size_t)(kUpdRing + 1) * (size_t)(g.Np - g.N);
+}
+
+// the axes of a mixed handle that the tensor-core transforms take (st_dst_tma.cu): 32-column
+// tiles and, along x, whole 32-element chunks
+bool tc_time_ok(const Geom &g) { return dst_tma_supported(g.n) && g.mp >= 32; }
+bool tc_x_ok(const Geom &g) { return g.mx >= 31 && dst_tma_supported(g.mx); }
+bool tc_y_ok(const Geom &g) {
+  return g.dim >= 2 && g.my >= 31 && g.px >= 32 && dst_tma_supported(g.my);
+}
+bool tc_z_ok(const Geom &g) {
+  return g.dim == 3 && g.mz >= 31 && (long long)g.px * g.my >= 32 && dst_tma_supported(g.mz);
+}
+
 size_t workspace_bytes(const Geom &g, bool mixed, int cheb, int ugroup) {
   const size_t N = (size_t)g.N;
+  const size_t Nv = mixed ? (size_t)g.Np : N;  // the mixed path's own vectors are padded
   size_t b = 0;
-  if (mixed) b += (size_t)(ugroup - 1) * N * sizeof(float);  // grouped update: pending z_j
   if (cheb) b += cheb_coef_bytes(g, cheb) + 5 * N * sizeof(double);
-  b += 2 * N * sizeof(double);                             // V
-  b += 2 * N * (mixed ? sizeof(float) : sizeof(double));   // Z
-  b += 2 * N * sizeof(double);                             // D
-  b += N * sizeof(double);                                 // q
-  if (mixed) b += N * sizeof(df);                          // x accumulator
-  b += 2 * N * sizeof(double);                             // host staging
+  b += 2 * Nv * sizeof(double);                            // V
+  b += mixed ? zslab_floats(g, ugroup) * sizeof(float) : 2 * N * sizeof(double);  // Z
+  b += 2 * Nv * sizeof(double);                            // D
+  b += Nv * sizeof(double);                                // q
+  if (mixed) b += Nv * sizeof(df);                         // x accumulator
+  b += (mixed ? 1 : 2) * N * sizeof(double);               // host staging
   b += (size_t)partials_needed(g) * sizeof(double);
   b += sizeof(State);
   b += ((size_t)g.my * (g.mx + 1) + (size_t)(g.my + 1) * g.mx) * sizeof(double);  // grad faces
   b += table_doubles(g) * sizeof(double) + table_floats(g) * sizeof(float) + 256;
   b += table_floats(g) * sizeof(dd) + 256;  // double-float copies of the spectral tables
   b += (faces_x(g) + faces_y(g) + faces_z(g)) * sizeof(df) + 256;  // df faces
-  if (mixed && time_tc_supported(g.n)) b += time_tc_sop_halves(g.n) * 2;
-  if (mixed && !time_tc_supported(g.n) && time_tc_long_supported(g.n))
-    b += time_tc_long_bytes(g.n) + 256;
-  if (mixed && g.dim >= 2 && dst_tc_supported(g.my)) b += time_tc_sop_halves(g.my) * 2 + 256;
-  if (mixed && g.dim == 3 && dst_tc_supported(g.mz)) b += time_tc_sop_halves(g.mz) * 2 + 256;
-  if (mixed && dst_tc_supported(g.mx)) b += time_tc_sop_halves(g.mx) * 2 + 256;
+  if (mixed && tc_time_ok(g)) b += dst_tma_image_halves(g.n) * 2;
+  if (mixed && !tc_time_ok(g) && time_tc_long_supported(g.n)) b += time_tc_long_bytes(g.n) + 256;
+  if (mixed && tc_y_ok(g)) b += dst_tma_image_halves(g.my) * 2 + 256;
+  if (mixed && tc_z_ok(g)) b += dst_tma_image_halves(g.mz) * 2 + 256;
+  if (mixed && tc_x_ok(g)) b += dst_tma_image_halves(g.mx) * 2 + 256;
   if (!mixed && time_tcd_supported(g.n)) b += time_tcd_bytes(g.n) + 256;  // digits of S_n
   b += 256;  // alignment of the z image
   return b;
@@ -773,9 +804,9 @@ int build_tables(st_handle *h) {
   const char *no_tc = std::getenv("ST_DISABLE_TENSOR_CORES");
   const bool use_tc = p.precision == ST_MIXED && !(no_tc && no_tc[0] == '1');
   bool long_tc = false;
-  if (use_tc && time_tc_supported(n)) {
-    sop.resize(time_tc_sop_halves(n));
-    time_tc_build_sop(n, sop.data());
+  if (use_tc && tc_time_ok(g)) {
+    sop.resize(dst_tma_image_halves(n));
+    dst_tma_build_image(n, sop.data());
   } else if (use_tc && time_tc_long_supported(n)) {
     // streamed chunks for 256 < n <= 512, in the same slot of the table allocation
     sop.resize(time_tc_long_bytes(n) / 2);
@@ -791,20 +822,18 @@ int build_tables(st_handle *h) {
   const size_t o_cdf = (o_sop + sop.size() * sizeof(unsigned short) + 255) / 256 * 256;
   // fp16 S_my / S_mz images for the tensor-core y- and z-DSTs (mixed precision, supported lengths)
   std::vector<unsigned short> sopy, sopz, sopx;
-  if (p.precision == ST_MIXED && g.dim >= 2 && dst_tc_supported(g.my) &&
-      !(no_tc && no_tc[0] == '1')) {
-    sopy.resize(time_tc_sop_halves(g.my));
-    time_tc_build_sop(g.my, sopy.data());
+  if (use_tc && tc_y_ok(g)) {
+    sopy.resize(dst_tma_image_halves(g.my));
+    dst_tma_build_image(g.my, sopy.data());
   }
-  if (p.precision == ST_MIXED && g.dim == 3 && dst_tc_supported(g.mz) &&
-      !(no_tc && no_tc[0] == '1')) {
-    sopz.resize(time_tc_sop_halves(g.mz));
-    time_tc_build_sop(g.mz, sopz.data());
+  if (use_tc && tc_z_ok(g)) {
+    sopz.resize(dst_tma_image_halves(g.mz));
+    dst_tma_build_image(g.mz, sopz.data());
   }
   // and S_mx for the tensor-core x-DST of the last spatial pass
-  if (p.precision == ST_MIXED && dst_tc_supported(g.mx) && !(no_tc && no_tc[0] == '1')) {
-    sopx.resize(time_tc_sop_halves(g.mx));
-    time_tc_build_sop(g.mx, sopx.data());
+  if (use_tc && tc_x_ok(g)) {
+    sopx.resize(dst_tma_image_halves(g.mx));
+    dst_tma_build_image(g.mx, sopx.data());
   }
   const size_t o_sopy = (o_cdf + cdf.size() * sizeof(df) + 255) / 256 * 256;
   const size_t o_sopz = (o_sopy + sopy.size() * sizeof(unsigned short) + 255) / 256 * 256;
@@ -876,6 +905,8 @@ int build_tables(st_handle *h) {
   if (cheb) {
     const size_t cb = cheb_coef_bytes(g, cheb);
     ST_TRY(cudaMalloc(&h->cheb, cb + 5 * (size_t)g.N * sizeof(double)));
+    // the scratch vectors' padding slots hold zeros
+    ST_TRY(cudaMemset((char *)h->cheb + cb, 0, 5 * (size_t)g.N * sizeof(double)));
     const size_t cnt = (size_t)cheb * n;
     std::vector<float> af(cnt), sf(cnt);
     for (size_t i = 0; i < cnt; ++i) {
@@ -900,7 +931,7 @@ int build_tables(st_handle *h) {
       (sop.empty() || pp.pcr || pp.cheb) ? nullptr
                               : reinterpret_cast<const unsigned short *>((const char *)h->tables + o_sop);
   // the P_theta paths with varying a transform time alone (no scaling) on the tensor cores
-  pp.sop_t1 = (!sop.empty() && !long_tc && (pp.pcr || pp.cheb) && dst_tc_len_supported(n))
+  pp.sop_t1 = (!sop.empty() && !long_tc && (pp.pcr || pp.cheb))
                   ? reinterpret_cast<const unsigned short *>((const char *)h->tables + o_sop)
                   : nullptr;
   pp.sop = long_tc ? nullptr : sop_img;
@@ -961,7 +992,7 @@ void free_handle(st_handle *h) {
   cudaFree(h->tables);
   for (int i = 0; i < 2; ++i) {
     cudaFree(h->V[i]);
-    cudaFree(h->Z[i]);
+    if (!h->mixed) cudaFree(h->Z[i]);
     cudaFree(h->D[i]);
   }
   cudaFree(h->q);
@@ -969,12 +1000,12 @@ void free_handle(st_handle *h) {
   cudaFree(h->partials);
   cudaFree(h->S);
   cudaFree(h->hbuf_in);
-  cudaFree(h->hbuf_out);
+  if (!h->mixed) cudaFree(h->hbuf_out);
   cudaFree(h->gfx);
   cudaFree(h->gfy);
   cudaFree(h->cheb);
   if (h->hS) cudaFreeHost(h->hS);
-  for (int i = 0; i < kUpdRing - 1; ++i) cudaFree(h->Zx[i]);
+  cudaFree(h->zslab);
   prof_free(h->prof);
   delete h;
 }
@@ -1170,9 +1201,9 @@ int solve_fp64(st_handle *h, const double *fH, double *x, double tol, int maxit,
 // recomputed in float64 (iterative refinement) until ||r||/||b|| <= tol.
 int mixed_start(st_handle *h, double target, int maxit) {
   const Geom &g = h->g;
-  ST_TRY(cudaMemsetAsync(h->D[0], 0, g.N * sizeof(df), h->stream));
-  ST_TRY(cudaMemsetAsync(h->D[1], 0, g.N * sizeof(df), h->stream));
-  ST_TRY(cudaMemsetAsync(h->V[1], 0, g.N * sizeof(df), h->stream));
+  ST_TRY(cudaMemsetAsync(h->D[0], 0, g.Np * sizeof(df), h->stream));
+  ST_TRY(cudaMemsetAsync(h->D[1], 0, g.Np * sizeof(df), h->stream));
+  ST_TRY(cudaMemsetAsync(h->V[1], 0, g.Np * sizeof(df), h->stream));
   State &s = *h->hS;
   const double bn = s.bnorm2;
   std::memset(&s, 0, sizeof(State));
@@ -1207,7 +1238,7 @@ int solve_mixed(st_handle *h, const double *fH, double *x, double tol, int maxit
                 st_stats *stats) {
   const Geom &g = h->g;
   cudaStream_t st = h->stream;
-  ST_TRY(cudaMemsetAsync(h->Xdf, 0, g.N * sizeof(df), st));
+  ST_TRY(cudaMemsetAsync(h->Xdf, 0, g.Np * sizeof(df), st));
   ST_TRY(cudaMemsetAsync(x, 0, g.N * sizeof(double), st));
   std::memset(h->hS, 0, sizeof(State));
   int r = push_state(h);
@@ -1236,7 +1267,7 @@ int solve_mixed(st_handle *h, const double *fH, double *x, double tol, int maxit
     last_est = s.est;
     status = s.status;
     ST_TRY(launch_update_group(h, st));  // the inner run's pending updates
-    ST_TRY(launch_df_to_double(g.N, h->Xdf, x, st));
+    ST_TRY(launch_df_to_double(g, h->Xdf, x, st));
     // r = Y f_H - Y T x (float64), stored as the next step's double-float right-hand side
     ST_TRY(launch_resid_df(g, x, (df *)h->V[0], fH, h->S, h->partials, st));
     r = sync_state(h);
@@ -1298,29 +1329,43 @@ int st::setup_handle(const st_problem *prob, st_handle **out, int ugroup) {
   };
   r = build_tables(h);
   if (r) return fail(r);
-  const size_t zsz = h->mixed ? sizeof(float) : sizeof(double);
+  const size_t Nv = h->mixed ? (size_t)g.Np : N;
   cudaError_t e = cudaSuccess;
   for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
-    e = cudaMalloc(&h->V[i], N * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&h->Z[i], N * zsz);
-    if (e == cudaSuccess) e = cudaMalloc(&h->D[i], N * sizeof(double));
+    e = cudaMalloc(&h->V[i], Nv * sizeof(double));
+    if (e == cudaSuccess && !h->mixed) e = cudaMalloc(&h->Z[i], N * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc(&h->D[i], Nv * sizeof(double));
   }
-  if (e == cudaSuccess) e = cudaMalloc(&h->q, N * sizeof(double));
+  // z vectors of a mixed handle, with those of the iterations a grouped update keeps pending; their
+  // padding stays zero from here on
+  h->ugroup = h->mixed ? ugroup : 1;
+  if (e == cudaSuccess && h->mixed) {
+    const size_t zf = zslab_floats(g, ugroup);
+    e = cudaMalloc(&h->zslab, zf * sizeof(float));
+    if (e == cudaSuccess) e = cudaMemset(h->zslab, 0, zf * sizeof(float));
+    float *z0 = h->zslab + kZGuard;
+    h->Z[0] = z0;
+    h->Z[1] = z0 + g.Np;
+    for (int i = 0; i < ugroup - 1; ++i) h->Zx[i] = z0 + (size_t)(i + 2) * g.Np;
+  }
+  h->zscratch = (float *)h->Z[0];
+  if (e == cudaSuccess) e = cudaMalloc(&h->q, Nv * sizeof(double));
   h->pp.tscratch = reinterpret_cast<dd *>(h->q);  // free during a preconditioner pass
-  if (e == cudaSuccess && h->mixed) e = cudaMalloc(&h->Xdf, N * sizeof(df));
+  if (e == cudaSuccess && h->mixed) e = cudaMalloc(&h->Xdf, Nv * sizeof(df));
   h->partials_len = partials_needed(g);
   if (e == cudaSuccess) e = cudaMalloc(&h->partials, (size_t)h->partials_len * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&h->S, sizeof(State));
   if (e == cudaSuccess) e = cudaMalloc(&h->hbuf_in, N * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&h->hbuf_out, N * sizeof(double));
+  if (e == cudaSuccess) {
+    if (h->mixed)
+      h->hbuf_out = h->q;
+    else
+      e = cudaMalloc(&h->hbuf_out, N * sizeof(double));
+  }
   if (e == cudaSuccess) e = cudaMalloc(&h->gfx, (size_t)g.my * (g.mx + 1) * sizeof(double));
   if (e == cudaSuccess)
     e = cudaMalloc(&h->gfy, ((size_t)g.my + 1) * g.mx * sizeof(double));
   if (e == cudaSuccess) e = cudaMallocHost(&h->hS, sizeof(State));
-  // z vectors of the iterations a grouped update keeps pending (mixed single solves)
-  h->ugroup = h->mixed ? ugroup : 1;
-  for (int i = 0; i < h->ugroup - 1 && e == cudaSuccess; ++i)
-    e = cudaMalloc(&h->Zx[i], N * sizeof(float));
   if (e == cudaSuccess) e = cudaMemset(h->S, 0, sizeof(State));
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) return fail(map_cuda(e));
@@ -1453,7 +1498,7 @@ int st_autotune(st_handle *h, int reps) {
     return best;
   };
   cudaMemsetAsync(h->V[0], 0, g.N * sizeof(double), st);
-  cudaMemsetAsync(h->Z[0], 0, g.N * (fp32 ? sizeof(float) : sizeof(double)), st);
+  cudaMemsetAsync(h->Z[0], 0, fp32 ? g.Np * sizeof(float) : g.N * sizeof(double), st);
   // 1. stencil: blocks per launch (time-chunk length)
   {
     const int cand[] = {608, 1216, 2432, 4864};
@@ -1516,8 +1561,8 @@ int st_autotune(st_handle *h, int reps) {
     if (fp32) h->pp.time_J_f = bj; else h->pp.time_J_d = bj;
     if (fp32 && h->tc_time_img && !h->pp.pcr && !h->pp.cheb) {
       const float ms_tc = timed([&]() {
-        return launch_time_tc((float *)h->Z[0], h->g, h->pp.spec_f, h->tc_time_img, h->S,
-                              TM_NONE, h->partials, GK_NONE, st);
+        return launch_time_tma((float *)h->Z[0], h->g, h->pp.spec_f, h->tc_time_img, h->S,
+                               TM_NONE, h->partials, GK_NONE, st);
       });
       tc_time = (ms_tc <= best) ? 1 : 0;
     }
@@ -1652,6 +1697,9 @@ int st_apply_prec(st_handle *h, const double *v_dev, double *z_dev) {
   ST_ENTER(h);
   ST_TRY((launch_prec<double, double, double>(h->g, h->pp, v_dev, z_dev, h->S, TM_NONE,
                                               h->partials, h->stream)));
+  // the float64 pass used the Chebyshev scratch unpadded: the mixed path wants its padding zero
+  if (h->mixed && h->pp.cheb)
+    ST_TRY(cudaMemsetAsync(h->pp.cheb_work, 0, 5 * (size_t)h->g.N * sizeof(double), h->stream));
   return ST_OK;
 }
 
@@ -1659,8 +1707,14 @@ int st_apply_prec_f32(st_handle *h, const double *v_dev, float *z_dev) {
   if (!h || !v_dev || !z_dev) return ST_ERR_ARG;
   ProfScope prof_scope(h);
   ST_ENTER(h);
-  ST_TRY((launch_prec<float, double, float>(h->g, h->pp, v_dev, z_dev, h->S, TM_NONE,
-                                            h->partials, h->stream)));
+  // the passes work on a padded vector of the handle (Z[0], free between solves); on a float64
+  // handle, whose vectors are not padded, its slots (and the Chebyshev scratch) are zeroed first
+  if (!h->mixed) {
+    ST_TRY(cudaMemsetAsync(h->zscratch, 0, (size_t)h->g.Np * sizeof(float), h->stream));
+    if (h->pp.cheb)
+      ST_TRY(cudaMemsetAsync(h->pp.cheb_work, 0, 5 * (size_t)h->g.N * sizeof(double), h->stream));
+  }
+  ST_TRY(launch_prec_user(h->g, h->pp, v_dev, h->zscratch, z_dev, h->S, h->partials, h->stream));
   return ST_OK;
 }
 

@@ -34,9 +34,11 @@ constexpr int kNT = 256;
 // still completes z_{k+1} (needed if the stopping rule later decides to continue).
 
 // ------------------------------------------------------------------------------ spatial DST
-// XL = true: lines are rows (contiguous, line l starts at l*len).
-// XL = false: lines are columns of the (my x mx) planes: line l = k*mx + i starts at k*m + i and
-// its elements are mx apart.  A block owns 2*PB consecutive lines (PB complex sequences, line
+// XL = true: lines are rows (contiguous; line l starts at l*pin in the source and at l*pout in the
+// output: the line length len, or len + 1 in the padded layout).
+// XL = false: lines are columns of planes: line l = k*mx + i starts at k*m + i and its elements are
+// `ld` apart; columns i with i mod pin >= pout are left alone (the padding columns of z lines: the
+// two lines of a packed pair leave rounding in each other, and the padding stays exactly zero).  A block owns 2*PB consecutive lines (PB complex sequences, line
 // 2p in the real part and line 2p+1 in the imaginary part), loads them coalesced into shared
 // memory as odd extensions, runs in-place Stockham passes and writes the sine coefficients.
 constexpr int kNTD = 512;  // threads per spatial-DST block
@@ -60,8 +62,8 @@ struct StockhamPasses {
 // and the fused Lanczos source (its loads held in registers ahead of the stores): two
 template <class Tc, class Src, class Tout, bool XL, int LOGL>
 __global__ void __launch_bounds__(kNTD, (sizeof(Tc) == 4 && !has_fetch<Src>::value) ? 3 : 2)
-    k_dst_space(Src src, Tout *out, int len, long long nlines, int mx, long long m,
-                const Tc *tw, int PB, const State *S, int gk) {
+    k_dst_space(Src src, Tout *out, int len, long long nlines, int mx, long long ld, long long m,
+                int pin, int pout, const Tc *tw, int PB, const State *S, int gk) {
   if (gate_closed(S, gk)) return;
   src.prepare(S);
   constexpr int logL = LOGL;
@@ -96,10 +98,10 @@ __global__ void __launch_bounds__(kNTD, (sizeof(Tc) == 4 && !has_fetch<Src>::val
       const int idx = tid + u * kNTD;
       const int pp = idx >> logH, e = idx & (half - 1);
       const int la = 2 * pp, lb = la + 1;
-      const long long i0 = (line0 + la) * len + e;
+      const long long i0 = (line0 + la) * pin + e;
       if (idx < (PB << logH) && e < len) {
         if (la < nl) ra[u] = src.fetch(i0);
-        if (lb < nl) rb[u] = src.fetch(i0 + len);
+        if (lb < nl) rb[u] = src.fetch(i0 + pin);
       }
     }
 #pragma unroll
@@ -108,9 +110,9 @@ __global__ void __launch_bounds__(kNTD, (sizeof(Tc) == 4 && !has_fetch<Src>::val
       const int pp = idx >> logH, e = idx & (half - 1);
       if (idx >= (PB << logH) || e >= len) continue;
       const int la = 2 * pp, lb = la + 1;
-      const long long i0 = (line0 + la) * len + e;
+      const long long i0 = (line0 + la) * pin + e;
       const Tc a = (la < nl) ? src.finish(i0, ra[u]) : Tc(0);
-      const Tc b = (lb < nl) ? src.finish(i0 + len, rb[u]) : Tc(0);
+      const Tc b = (lb < nl) ? src.finish(i0 + pin, rb[u]) : Tc(0);
       cpx<Tc> *bq = buf + pp * Ls;
       bq[fft_pad<Tc>(e + 1)] = cpx<Tc>{a, b};
       bq[fft_pad<Tc>(L - 1 - e)] = cpx<Tc>{-a, -b};
@@ -121,9 +123,9 @@ __global__ void __launch_bounds__(kNTD, (sizeof(Tc) == 4 && !has_fetch<Src>::val
       const int pp = idx >> logH, e = idx & (half - 1);
       if (e >= len) continue;
       const int la = 2 * pp, lb = la + 1;
-      const long long i0 = (line0 + la) * len + e;
+      const long long i0 = (line0 + la) * pin + e;
       const Tc a = (la < nl) ? src(i0) : Tc(0);
-      const Tc b = (lb < nl) ? src(i0 + len) : Tc(0);
+      const Tc b = (lb < nl) ? src(i0 + pin) : Tc(0);
       cpx<Tc> *bq = buf + pp * Ls;
       bq[fft_pad<Tc>(e + 1)] = cpx<Tc>{a, b};
       bq[fft_pad<Tc>(L - 1 - e)] = cpx<Tc>{-a, -b};
@@ -137,16 +139,16 @@ __global__ void __launch_bounds__(kNTD, (sizeof(Tc) == 4 && !has_fetch<Src>::val
     if (la < nl) {
       const int l = (int)line0 + la;
       const int k = l / mx, i = l - k * mx;
-      ia = (long long)k * m + i;
+      if (pin == pout || i % pin < pout) ia = (long long)k * m + i;
     }
     if (lb < nl) {
       const int l = (int)line0 + lb;
       const int k = l / mx, i = l - k * mx;
-      ib = (long long)k * m + i;
+      if (pin == pout || i % pin < pout) ib = (long long)k * m + i;
     }
     cpx<Tc> *bq = buf + pp * Ls;
     for (int e = tid >> logPB; e < len; e += estep) {
-      const long long off = (long long)e * mx;
+      const long long off = (long long)e * ld;
       const Tc a = (ia >= 0) ? src(ia + off) : Tc(0);
       const Tc b = (ib >= 0) ? src(ib + off) : Tc(0);
       bq[fft_pad<Tc>(e + 1)] = cpx<Tc>{a, b};
@@ -162,9 +164,9 @@ __global__ void __launch_bounds__(kNTD, (sizeof(Tc) == 4 && !has_fetch<Src>::val
       if (e >= len) continue;
       const cpx<Tc> Z = buf[pp * Ls + fft_pad<Tc>(e + 1)];
       const int la = 2 * pp, lb = la + 1;
-      Tout *p = out + (line0 + la) * len + e;
+      Tout *p = out + (line0 + la) * pout + e;
       if (la < nl) p[0] = (Tout)(-Z.y * sc);
-      if (lb < nl) p[len] = (Tout)(Z.x * sc);
+      if (lb < nl) p[pout] = (Tout)(Z.x * sc);
     }
   } else {
     const int pp = tid & (PB - 1), estep = kNTD >> logPB;
@@ -173,17 +175,17 @@ __global__ void __launch_bounds__(kNTD, (sizeof(Tc) == 4 && !has_fetch<Src>::val
     if (la < nl) {
       const int l = (int)line0 + la;
       const int k = l / mx, i = l - k * mx;
-      pa = out + (long long)k * m + i;
+      if (pin == pout || i % pin < pout) pa = out + (long long)k * m + i;
     }
     if (lb < nl) {
       const int l = (int)line0 + lb;
       const int k = l / mx, i = l - k * mx;
-      pb = out + (long long)k * m + i;
+      if (pin == pout || i % pin < pout) pb = out + (long long)k * m + i;
     }
     const cpx<Tc> *bq = buf + pp * Ls;
     for (int e = tid >> logPB; e < len; e += estep) {
       const cpx<Tc> Z = bq[fft_pad<Tc>(e + 1)];
-      const long long off = (long long)e * mx;
+      const long long off = (long long)e * ld;
       if (pa) pa[off] = (Tout)(-Z.y * sc);
       if (pb) pb[off] = (Tout)(Z.x * sc);
     }
@@ -270,8 +272,8 @@ __device__ void time_dst_tile(Tc *X, Tc *Y, const Tc *sintab, int n, int J) {
 
 template <class Tc, int KT, int JT>
 __global__ void __launch_bounds__(kNT)
-    k_time(const Tc *data, Tc *out, int n, long long m, int mx, int J, Spec<Tc> sp, State *S,
-           int tmode, int tkind, double *__restrict__ partials, int gk) {
+    k_time(const Tc *data, Tc *out, int n, long long m, int mx, int px, int J, Spec<Tc> sp,
+           State *S, int tmode, int tkind, double *__restrict__ partials, int gk) {
   __shared__ double red[32];
   if (gate_closed(S, gk)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -284,11 +286,13 @@ __global__ void __launch_bounds__(kNT)
   const int Je = (int)min((long long)J, m - j0);
   for (int r = tid; r < 2 * (n + 1); r += kNT) sintab[r] = sp.sintab[r];
   for (int c = tid; c < J; c += kNT) {
-    Tc v = Tc(0);
+    // px = mx, or mx + 1 in the padded layout, whose padding columns hold zeros (and keep them
+    // with any positive factor)
+    Tc v = Tc(1);
     if (c < Je) {
       const long long j = j0 + c;
-      const long long jy = j / mx, jx = j - jy * mx;
-      v = sp.mux[jx] + sp.muy[jy];
+      const long long jy = j / px, jx = j - jy * px;
+      if (jx < mx) v = sp.mux[jx] + sp.muy[jy];
     }
     tmu[c] = v;
   }
@@ -349,7 +353,7 @@ __global__ void __launch_bounds__(kNT)
 // <v_k, z_k>, whose sum over k is <v, P_theta^-1 v> (the time DST is orthogonal).
 template <class Tc>
 __global__ void __launch_bounds__(kNT)
-    k_pcr_ptheta(Tc *data, int n, int mx, const double *__restrict__ cx, Spec<Tc> sp, State *S,
+    k_pcr_ptheta(Tc *data, int n, int mx, int px, const double *__restrict__ cx, Spec<Tc> sp, State *S,
                  int tmode, double *__restrict__ partials, int gk) {
   __shared__ double red[32];
   if (gate_closed(S, gk)) return;
@@ -360,7 +364,7 @@ __global__ void __launch_bounds__(kNT)
   const int k = blockIdx.x;  // 0-based frequency
   const int tid = threadIdx.x;
   const Tc lh = sp.lh[k], lt = sp.lht[k];
-  Tc *row = data + (long long)k * mx;
+  Tc *row = data + (long long)k * px;
   for (int i = tid; i < mx; i += kNT) {
     const Tc w = (Tc)cx[i], e = (Tc)cx[i + 1];  // tau a/h^2 at the faces of node i
     b[i] = lh + lt * (w + e);
@@ -465,7 +469,7 @@ constexpr int kChebBX = 32, kChebBY = 8;
 
 template <class Tc>
 __global__ void __launch_bounds__(kChebBX * kChebBY)
-    k_cheb_resid(Geom g, const Tc *__restrict__ dprev, const Tc *__restrict__ w,
+    k_cheb_resid(Geom g, int px, const Tc *__restrict__ dprev, const Tc *__restrict__ w,
                  Tc *__restrict__ dnext, const Tc *rsrc, Tc *r, Tc *__restrict__ x,
                  const Tc *__restrict__ acoef, const Tc *__restrict__ lh,
                  const Tc *__restrict__ lht, int first, const State *S, int gk) {
@@ -475,9 +479,10 @@ __global__ void __launch_bounds__(kChebBX * kChebBY)
   const int row = blockIdx.x * kChebBY + threadIdx.y;
   const int k = blockIdx.z;
   if (ix >= mx || row >= my * mz) return;
-  const long long pl = (long long)mx * my;
+  // px slots a line (mx, or mx + 1 in the padded layout): planes of px * my
+  const long long pl = (long long)px * my;
   {
-    const long long e = (long long)k * g.m + (long long)row * mx + ix;
+    const long long e = (long long)k * (pl * mz) + (long long)row * px + ix;
     const int jz = row / my, jy = row - jz * my;
     const Tc ak = first ? Tc(0) : acoef[k];
     auto dv = [&](long long q) -> Tc { return first ? w[q] : ak * dprev[q] + w[q]; };
@@ -489,13 +494,13 @@ __global__ void __launch_bounds__(kChebBX * kChebBY)
     Tc cd = Tc(0), cu = Tc(0);
     if (g.dim == 3) {
       cd = face_c<Tc>(g.cz, g.czd, (long long)row * mx + ix);
-      cu = face_c<Tc>(g.cz, g.czd, (long long)row * mx + ix + pl);
+      cu = face_c<Tc>(g.cz, g.czd, (long long)row * mx + ix + (long long)mx * my);
     }
     Tc kd = (cw + ce + cs + cn + cd + cu) * dc;
     if (ix > 0) kd -= cw * dv(e - 1);
     if (ix < mx - 1) kd -= ce * dv(e + 1);
-    if (jy > 0) kd -= cs * dv(e - mx);
-    if (jy < my - 1) kd -= cn * dv(e + mx);
+    if (jy > 0) kd -= cs * dv(e - px);
+    if (jy < my - 1) kd -= cn * dv(e + px);
     if (jz > 0) kd -= cd * dv(e - pl);
     if (jz < mz - 1) kd -= cu * dv(e + pl);
     r[e] = rsrc[e] - (lh[k] * dc + lht[k] * kd);
@@ -545,14 +550,30 @@ __global__ void __launch_bounds__(kNT)
   }
 }
 
-// z = source elements in the transform type (a conversion, or the fused Lanczos step)
+// z = source elements in the transform type (a conversion, or the fused Lanczos step), line by
+// line: pin slots a line in the source, pout in z.  The padding slots of z keep their zeros.
 template <class Tc, class Src>
-__global__ void k_copy_to(long long N, Src src, Tc *z, const State *S, int gk) {
+__global__ void k_copy_to(unsigned nlines, int mx, int pin, int pout, Src src, Tc *z,
+                          const State *S, int gk) {
   if (gate_closed(S, gk)) return;
   src.prepare(S);
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < N;
-       e += (long long)gridDim.x * blockDim.x)
-    z[e] = src(e);
+  const unsigned total = nlines * (unsigned)mx;  // = N < 2^31
+  for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < total;
+       e += gridDim.x * blockDim.x) {
+    const unsigned l = e / (unsigned)mx, i = e - l * (unsigned)mx;
+    z[(long long)l * pout + i] = src((long long)l * pin + i);
+  }
+}
+
+// padded float32 vector into a caller's contiguous one
+__global__ void k_unpad(unsigned nlines, int mx, int px, const float *__restrict__ z,
+                        float *__restrict__ out) {
+  const unsigned total = nlines * (unsigned)mx;
+  for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < total;
+       e += gridDim.x * blockDim.x) {
+    const unsigned l = e / (unsigned)mx, i = e - l * (unsigned)mx;
+    out[e] = z[(long long)l * px + i];
+  }
 }
 
 // the x pass that carries the fused Lanczos step is timed as its own kernel class
@@ -585,8 +606,9 @@ size_t time_smem(int n, int J) {
 }
 
 template <class Tc, class Src, class Tout, bool XL, int LOGL>
-cudaError_t launch_dst_l(Src in, Tout *out, int len, long long nlines, int mx, long long m,
-                         const Tc *tw, const State *S, int gk, int pbshift, cudaStream_t st) {
+cudaError_t launch_dst_l(Src in, Tout *out, int len, long long nlines, int mx, long long ld,
+                         long long m, int pin, int pout, const Tc *tw, const State *S, int gk,
+                         int pbshift, cudaStream_t st) {
   constexpr int L = 1 << LOGL;
   int PB = dst_pairs<Tc>(L) >> pbshift;
   if (PB < 1) PB = 1;
@@ -596,27 +618,68 @@ cudaError_t launch_dst_l(Src in, Tout *out, int len, long long nlines, int mx, l
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   prof_begin(XL ? (is_lanczos_src<Src>::value ? KC_LANCZOS : KC_DSTX) : KC_DSTY, st);
-  kern<<<(unsigned)blocks, kNTD, sm, st>>>(in, out, len, nlines, mx, m, tw, PB, S, gk);
+  kern<<<(unsigned)blocks, kNTD, sm, st>>>(in, out, len, nlines, mx, ld, m, pin, pout, tw, PB, S,
+                                           gk);
   prof_end(st);
   return cudaGetLastError();
 }
 
 template <class Tc, class Src, class Tout, bool XL>
-cudaError_t launch_dst(Src in, Tout *out, int len, int L, long long nlines, int mx,
-                       long long m, const Tc *tw, const State *S, int gk, int pbshift,
-                       cudaStream_t st) {
+cudaError_t launch_dst(Src in, Tout *out, int len, int L, long long nlines, int mx, long long ld,
+                       long long m, int pin, int pout, const Tc *tw, const State *S, int gk,
+                       int pbshift, cudaStream_t st) {
   switch (L) {
-    case 8: return launch_dst_l<Tc, Src, Tout, XL, 3>(in, out, len, nlines, mx, m, tw, S, gk, pbshift, st);
-    case 16: return launch_dst_l<Tc, Src, Tout, XL, 4>(in, out, len, nlines, mx, m, tw, S, gk, pbshift, st);
-    case 32: return launch_dst_l<Tc, Src, Tout, XL, 5>(in, out, len, nlines, mx, m, tw, S, gk, pbshift, st);
-    case 64: return launch_dst_l<Tc, Src, Tout, XL, 6>(in, out, len, nlines, mx, m, tw, S, gk, pbshift, st);
-    case 128: return launch_dst_l<Tc, Src, Tout, XL, 7>(in, out, len, nlines, mx, m, tw, S, gk, pbshift, st);
-    case 256: return launch_dst_l<Tc, Src, Tout, XL, 8>(in, out, len, nlines, mx, m, tw, S, gk, pbshift, st);
-    case 512: return launch_dst_l<Tc, Src, Tout, XL, 9>(in, out, len, nlines, mx, m, tw, S, gk, pbshift, st);
-    case 1024: return launch_dst_l<Tc, Src, Tout, XL, 10>(in, out, len, nlines, mx, m, tw, S, gk, pbshift, st);
-    case 2048: return launch_dst_l<Tc, Src, Tout, XL, 11>(in, out, len, nlines, mx, m, tw, S, gk, pbshift, st);
+    case 8: return launch_dst_l<Tc, Src, Tout, XL, 3>(in, out, len, nlines, mx, ld, m, pin, pout, tw, S, gk, pbshift, st);
+    case 16: return launch_dst_l<Tc, Src, Tout, XL, 4>(in, out, len, nlines, mx, ld, m, pin, pout, tw, S, gk, pbshift, st);
+    case 32: return launch_dst_l<Tc, Src, Tout, XL, 5>(in, out, len, nlines, mx, ld, m, pin, pout, tw, S, gk, pbshift, st);
+    case 64: return launch_dst_l<Tc, Src, Tout, XL, 6>(in, out, len, nlines, mx, ld, m, pin, pout, tw, S, gk, pbshift, st);
+    case 128: return launch_dst_l<Tc, Src, Tout, XL, 7>(in, out, len, nlines, mx, ld, m, pin, pout, tw, S, gk, pbshift, st);
+    case 256: return launch_dst_l<Tc, Src, Tout, XL, 8>(in, out, len, nlines, mx, ld, m, pin, pout, tw, S, gk, pbshift, st);
+    case 512: return launch_dst_l<Tc, Src, Tout, XL, 9>(in, out, len, nlines, mx, ld, m, pin, pout, tw, S, gk, pbshift, st);
+    case 1024: return launch_dst_l<Tc, Src, Tout, XL, 10>(in, out, len, nlines, mx, ld, m, pin, pout, tw, S, gk, pbshift, st);
+    case 2048: return launch_dst_l<Tc, Src, Tout, XL, 11>(in, out, len, nlines, mx, ld, m, pin, pout, tw, S, gk, pbshift, st);
     default: return cudaErrorInvalidValue;
   }
+}
+
+// Slots of an x line, a plane of x lines and a time level of the vectors of transform type Tc:
+// float32 vectors are padded (Geom::px), float64 and double-float ones are not.
+struct Lay {
+  int px;
+  long long pl, mp, Np;
+};
+template <class Tc>
+Lay lay(const Geom &g) {
+  if (sizeof(Tc) == sizeof(float)) return Lay{g.px, (long long)g.px * g.my, g.mp, g.Np};
+  return Lay{g.mx, (long long)g.mx * g.my, g.m, g.N};
+}
+// slots of an x line of a source: a caller's float64 vector is contiguous, the mixed path's own
+// vectors are padded
+template <class Src>
+struct src_elem;
+template <class Tc, class Tin>
+struct src_elem<SrcArray<Tc, Tin>> {
+  using type = Tin;
+};
+template <class Tc, class Tv>
+struct src_elem<SrcLanczos<Tc, Tv>> {
+  using type = Tv;
+};
+template <class T>
+struct is_padded {
+  static constexpr bool value = false;
+};
+template <>
+struct is_padded<float> {
+  static constexpr bool value = true;
+};
+template <>
+struct is_padded<df> {
+  static constexpr bool value = true;
+};
+template <class Src>
+int src_px(const Geom &g) {
+  return is_padded<typename src_elem<Src>::type>::value ? g.px : g.mx;
 }
 
 template <class Tc>
@@ -660,13 +723,14 @@ cudaError_t launch_time(Tc *data, const Geom &g, const Spec<Tc> &sp, State *S, i
                         Tc *out = nullptr) {
   const int J = Jover > 0 ? Jover : time_J<Tc>(g.n);
   const size_t sm = time_smem<Tc>(g.n, J);
-  const long long blocks = (g.m + J - 1) / J;
+  const Lay y = lay<Tc>(g);
+  const long long blocks = (y.mp + J - 1) / J;
   constexpr int KT = TimeTile<Tc>::KT, JT = TimeTile<Tc>::JT;
   auto kern = k_time<Tc, KT, JT>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   prof_begin(KC_TIME, st);
-  kern<<<(unsigned)blocks, kNT, sm, st>>>(data, out ? out : data, g.n, g.m, g.mx, J, sp, S, tmode,
+  kern<<<(unsigned)blocks, kNT, sm, st>>>(data, out ? out : data, g.n, y.mp, g.mx, y.px, J, sp, S, tmode,
                                           tkind, partials, gk);
   prof_end(st);
   return cudaGetLastError();
@@ -677,7 +741,7 @@ cudaError_t launch_time(Tc *data, const Geom &g, const Spec<Tc> &sp, State *S, i
 int time_blocks_for(const Geom &g, const PrecPlan &pp, bool fp32) {
   int J = fp32 ? pp.time_J_f : pp.time_J_d;
   if (J <= 0) J = fp32 ? time_J<float>(g.n) : time_J<double>(g.n);
-  return (int)((g.m + J - 1) / J);
+  return (int)(((fp32 ? g.mp : g.m) + J - 1) / J);
 }
 
 int time_J_default(int n, bool fp32) { return fp32 ? time_J<float>(n) : time_J<double>(n); }
@@ -748,10 +812,11 @@ template <class Tc, class Src>
 cudaError_t dst_y_pass(Src src, Tc *out, const Geom &g, const PrecPlan &pp, State *S, int gk,
                        cudaStream_t st) {
   if (sizeof(Tc) == sizeof(float) && pp.sop_y != nullptr)
-    return launch_dst_tc_y(reinterpret_cast<float *>(out), g, pp.sop_y, S, gk, st);
+    return launch_dst_tma_y(reinterpret_cast<float *>(out), g, pp.sop_y, S, gk, st);
   const long long ny = (long long)g.n * g.mz * g.mx;
-  return launch_dst<Tc, Src, Tc, false>(src, out, g.my, pp.Ly, ny, g.mx, (long long)g.mx * g.my,
-                                        tw_of<Tc>(pp, false), S, gk, pp.dst_shift, st);
+  const Lay y = lay<Tc>(g);
+  return launch_dst<Tc, Src, Tc, false>(src, out, g.my, pp.Ly, ny, g.mx, y.px, y.pl, g.mx,
+                                        g.mx, tw_of<Tc>(pp, false), S, gk, pp.dst_shift, st);
 }
 
 // The last spatial pass, DST-I along x in place: the tensor cores in float32 when the plan has
@@ -760,11 +825,13 @@ template <class Tc, class Tout>
 cudaError_t dst_x_last_pass(Tout *z, const Geom &g, const PrecPlan &pp, State *S, int gk,
                             cudaStream_t st) {
   if (sizeof(Tc) == sizeof(float) && pp.sop_x != nullptr)
-    return launch_dst_tc_x(reinterpret_cast<float *>(z), g, pp.sop_x, S, gk, st);
+    return launch_dst_tma_x(reinterpret_cast<float *>(z), g, pp.sop_x, S, gk, st);
   const long long nx = (long long)g.n * g.my * g.mz;
+  const int px = lay<Tc>(g).px;
   return launch_dst<Tc, SrcArray<Tc, Tout>, Tout, true>(SrcArray<Tc, Tout>{z}, z, g.mx, pp.Lx,
-                                                        nx, g.mx, g.m, tw_of<Tc>(pp, true), S,
-                                                        gk, pp.dst_shift, st);
+                                                        nx, g.mx, 0, 0, px, px,
+                                                        tw_of<Tc>(pp, true), S, gk,
+                                                        pp.dst_shift, st);
 }
 
 template <class Tc>
@@ -786,10 +853,11 @@ template <class Tc, class Src>
 cudaError_t dst_z_pass(Src src, Tc *out, const Geom &g, const PrecPlan &pp, State *S, int gk,
                        cudaStream_t st) {
   if (sizeof(Tc) == sizeof(float) && pp.sop_z != nullptr)
-    return launch_dst_tc_z(reinterpret_cast<float *>(out), g, pp.sop_z, S, gk, st);
-  const long long nz = (long long)g.n * g.mx * g.my;
-  return launch_dst<Tc, Src, Tc, false>(src, out, g.mz, pp.Lz, nz, g.mx * g.my, g.m,
-                                        twz_of<Tc>(pp), S, gk, pp.dst_shift, st);
+    return launch_dst_tma_z(reinterpret_cast<float *>(out), g, pp.sop_z, S, gk, st);
+  const Lay y = lay<Tc>(g);
+  return launch_dst<Tc, Src, Tc, false>(src, out, g.mz, pp.Lz, (long long)g.n * y.pl, (int)y.pl,
+                                        y.pl, y.mp, y.px, g.mx, twz_of<Tc>(pp), S, gk,
+                                        pp.dst_shift, st);
 }
 
 // The time DST alone (the P_theta paths with varying a): tensor cores in float32 when the plan has
@@ -799,8 +867,8 @@ template <class Tc>
 cudaError_t time_single(Tc *in, Tc *out, const Geom &g, const PrecPlan &pp, State *S,
                         double *partials, int gk, int Jo, cudaStream_t st) {
   if (sizeof(Tc) == sizeof(float) && pp.sop_t1 != nullptr)
-    return launch_time_tc_single(reinterpret_cast<const float *>(in),
-                                 reinterpret_cast<float *>(out), g, pp.sop_t1, S, gk, st);
+    return launch_time_tma_single(reinterpret_cast<const float *>(in),
+                                  reinterpret_cast<float *>(out), g, pp.sop_t1, S, gk, st);
   return launch_time<Tc>(in, g, spec_of<Tc>(pp), S, TM_NONE, 1, partials, gk, Jo, st, out);
 }
 
@@ -813,7 +881,8 @@ cudaError_t cheb_stages(const Geom &g, const PrecPlan &pp, Src src, Tc *zc, Stat
   using Arr = SrcArray<Tc, Tc>;
   const int gk = gate_kind_of(tmode);
   const Spec<Tc> &sp = spec_of<Tc>(pp);
-  const long long N = g.N;
+  const Lay y = lay<Tc>(g);
+  const long long N = y.Np;
   Tc *R = reinterpret_cast<Tc *>(pp.cheb_work);
   Tc *W = R + N, *X = R + 2 * N;
   Tc *Dd[2] = {R + 3 * N, R + 4 * N};
@@ -829,7 +898,8 @@ cudaError_t cheb_stages(const Geom &g, const PrecPlan &pp, Src src, Tc *zc, Stat
     return r;
   };
   prof_begin(KC_AUX, st);
-  k_copy_to<Tc, Src><<<kChebBlocks, kNT, 0, st>>>(N, src, zc, S, gk);
+  k_copy_to<Tc, Src><<<kChebBlocks, kNT, 0, st>>>((unsigned)nx, g.mx, src_px<Src>(g), y.px, src,
+                                                  zc, S, gk);
   prof_end(st);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   e = time_single<Tc>(zc, zc, g, pp, S, partials, gk, Jo, st);
@@ -838,14 +908,14 @@ cudaError_t cheb_stages(const Geom &g, const PrecPlan &pp, Src src, Tc *zc, Stat
   for (int j = 0; j < pp.cheb; ++j) {
     // the axes commute: x, y (z), then x with the scaling fused into its loads, then y (z); the
     // y and z passes take the tensor cores in float32 when the plan has the S_my / S_mz image
-    e = launch_dst<Tc, Arr, Tc, true>(Arr{j == 0 ? zc : R}, W, g.mx, pp.Lx, nx, g.mx, g.m, twx, S,
-                                      gk, pp.dst_shift, st);
+    e = launch_dst<Tc, Arr, Tc, true>(Arr{j == 0 ? zc : R}, W, g.mx, pp.Lx, nx, g.mx, 0, 0, y.px,
+                                      y.px, twx, S, gk, pp.dst_shift, st);
     if (e != cudaSuccess) return e;
     if ((e = yz_pass(W)) != cudaSuccess) return e;
     const SrcChebScale<Tc> sc{W, scoef + (size_t)j * g.n, sp.lh, sp.lht, sp.mux, sp.muy,
-                              (unsigned)g.m, (unsigned)g.mx};
-    e = launch_dst<Tc, SrcChebScale<Tc>, Tc, true>(sc, W, g.mx, pp.Lx, nx, g.mx, g.m, twx, S, gk,
-                                                   pp.dst_shift, st);
+                              (unsigned)y.mp, (unsigned)y.px};
+    e = launch_dst<Tc, SrcChebScale<Tc>, Tc, true>(sc, W, g.mx, pp.Lx, nx, g.mx, 0, 0, y.px, y.px,
+                                                   twx, S, gk, pp.dst_shift, st);
     if (e != cudaSuccess) return e;
     if ((e = yz_pass(W)) != cudaSuccess) return e;
     const Tc *aj = acoef + (size_t)j * g.n;
@@ -854,13 +924,13 @@ cudaError_t cheb_stages(const Geom &g, const PrecPlan &pp, Src src, Tc *zc, Stat
       const dim3 rg((unsigned)((g.my * g.mz + kChebBY - 1) / kChebBY),
                     (unsigned)((g.mx + kChebBX - 1) / kChebBX), (unsigned)g.n);
       prof_begin(KC_TIME, st);
-      k_cheb_resid<Tc><<<rg, rb, 0, st>>>(g, Dd[cur], W, Dd[cur ^ 1], j == 0 ? zc : R, R, X, aj,
+      k_cheb_resid<Tc><<<rg, rb, 0, st>>>(g, y.px, Dd[cur], W, Dd[cur ^ 1], j == 0 ? zc : R, R, X, aj,
                                           sp.lh, sp.lht, j == 0 ? 1 : 0, S, gk);
       prof_end(st);
       cur ^= 1;
     } else {
       prof_begin(KC_TIME, st);
-      k_cheb_final<Tc><<<kChebBlocks, kNT, 0, st>>>(N, g.m, Dd[cur], W, X, zc, R, aj,
+      k_cheb_final<Tc><<<kChebBlocks, kNT, 0, st>>>(N, y.mp, Dd[cur], W, X, zc, R, aj,
                                                     j == 0 ? 1 : 0, S, tmode, partials, gk);
       prof_end(st);
     }
@@ -901,8 +971,8 @@ cudaError_t prec_stages_dd(const Geom &g, const PrecPlan &pp, Src src, double *z
   const long long nx = (long long)g.n * g.my * g.mz;
   cudaError_t e;
   e = launch_dst<dd, decltype(AsDd<Src>::of(src)), dd, true>(AsDd<Src>::of(src), zd, g.mx, pp.Lx,
-                                                             nx, g.mx, g.m, pp.twx_dd, S, gk,
-                                                             pp.dst_shift, st);
+                                                             nx, g.mx, 0, 0, g.mx, g.mx,
+                                                             pp.twx_dd, S, gk, pp.dst_shift, st);
   if (e != cudaSuccess) return e;
   if (g.dim >= 2 && (e = dst_y_pass<dd>(Inner{zd}, zd, g, pp, S, gk, st)) != cudaSuccess) return e;
   if (g.dim == 3 && (e = dst_z_pass<dd>(Inner{zd}, zd, g, pp, S, gk, st)) != cudaSuccess) return e;
@@ -915,8 +985,8 @@ cudaError_t prec_stages_dd(const Geom &g, const PrecPlan &pp, Src src, double *z
   if (after_time && (e = cudaEventRecord(after_time, st)) != cudaSuccess) return e;
   if (g.dim == 3 && (e = dst_z_pass<dd>(Inner{zd}, zd, g, pp, S, gk, st)) != cudaSuccess) return e;
   if (g.dim >= 2 && (e = dst_y_pass<dd>(Inner{zd}, zd, g, pp, S, gk, st)) != cudaSuccess) return e;
-  return launch_dst<dd, Inner, double, true>(Inner{zd}, z, g.mx, pp.Lx, nx, g.mx, g.m, pp.twx_dd,
-                                             S, gk, pp.dst_shift, st);
+  return launch_dst<dd, Inner, double, true>(Inner{zd}, z, g.mx, pp.Lx, nx, g.mx, 0, 0, g.mx, g.mx,
+                                             pp.twx_dd, S, gk, pp.dst_shift, st);
 }
 
 // The stages of one preconditioner pass; `src` feeds the first one.
@@ -924,7 +994,8 @@ cudaError_t prec_stages_dd(const Geom &g, const PrecPlan &pp, Src src, double *z
 // has been enqueued.
 template <class Tc, class Src, class Tout>
 cudaError_t prec_stages(const Geom &g, const PrecPlan &pp, Src src, Tout *z, State *S, int tmode,
-                        double *partials, cudaStream_t st, cudaEvent_t after_time = nullptr) {
+                        double *partials, cudaStream_t st, cudaEvent_t after_time = nullptr,
+                        Tout *user = nullptr) {
   static_assert(sizeof(Tc) == sizeof(Tout), "in-place stages need Tout == Tc");
   using Inner = SrcArray<Tc, Tout>;
   const int gk = gate_kind_of(tmode);
@@ -941,7 +1012,9 @@ cudaError_t prec_stages(const Geom &g, const PrecPlan &pp, Src src, Tout *z, Sta
     // P_theta with a varying 1D coefficient: time DST, tridiagonal solves, time DST
     Tc *zc = reinterpret_cast<Tc *>(z);
     prof_begin(KC_AUX, st);
-    k_copy_to<Tc, Src><<<152 * 8, kNT, 0, st>>>(g.N, src, zc, S, gk);
+    const int px = lay<Tc>(g).px;
+    k_copy_to<Tc, Src><<<152 * 8, kNT, 0, st>>>((unsigned)((long long)g.n * g.my * g.mz), g.mx,
+                                                src_px<Src>(g), px, src, zc, S, gk);
     prof_end(st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int Jo = sizeof(Tc) == sizeof(float) ? pp.time_J_f : pp.time_J_d;
@@ -952,7 +1025,7 @@ cudaError_t prec_stages(const Geom &g, const PrecPlan &pp, Src src, Tout *z, Sta
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     prof_begin(KC_TIME, st);
-    kern<<<g.n, kNT, sm, st>>>(zc, g.n, g.mx, g.cx, spec_of<Tc>(pp), S, tmode, partials, gk);
+    kern<<<g.n, kNT, sm, st>>>(zc, g.n, g.mx, px, g.cx, spec_of<Tc>(pp), S, tmode, partials, gk);
     prof_end(st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (after_time && (e = cudaEventRecord(after_time, st)) != cudaSuccess) return e;
@@ -960,14 +1033,15 @@ cudaError_t prec_stages(const Geom &g, const PrecPlan &pp, Src src, Tout *z, Sta
   }
   const long long nx = (long long)g.n * g.my * g.mz;
   Tc *zt = reinterpret_cast<Tc *>(z);
-  e = launch_dst<Tc, Src, Tout, true>(src, z, g.mx, pp.Lx, nx, g.mx, g.m, tw_of<Tc>(pp, true), S,
-                                      gk, pp.dst_shift, st);
+  e = launch_dst<Tc, Src, Tout, true>(src, z, g.mx, pp.Lx, nx, g.mx, 0, 0, src_px<Src>(g),
+                                      lay<Tc>(g).px, tw_of<Tc>(pp, true), S, gk, pp.dst_shift,
+                                      st);
   if (e != cudaSuccess) return e;
   if (g.dim >= 2 && (e = dst_y_pass<Tc>(Inner{z}, zt, g, pp, S, gk, st)) != cudaSuccess) return e;
   if (g.dim == 3 && (e = dst_z_pass<Tc>(Inner{z}, zt, g, pp, S, gk, st)) != cudaSuccess) return e;
   if (sizeof(Tc) == sizeof(float) && pp.sop != nullptr)
-    e = launch_time_tc(reinterpret_cast<float *>(z), g, pp.spec_f, pp.sop, S, tmode, partials, gk,
-                       st);
+    e = launch_time_tma(reinterpret_cast<float *>(z), g, pp.spec_f, pp.sop, S, tmode, partials, gk,
+                        st);
   else if (sizeof(Tc) == sizeof(float) && pp.sop_long != nullptr)
     e = launch_time_tc_long(reinterpret_cast<float *>(z), g, pp.spec_f, pp.sop_long, S, tmode,
                             partials, gk, st);
@@ -978,6 +1052,16 @@ cudaError_t prec_stages(const Geom &g, const PrecPlan &pp, Src src, Tout *z, Sta
   if (after_time && (e = cudaEventRecord(after_time, st)) != cudaSuccess) return e;
   if (g.dim == 3 && (e = dst_z_pass<Tc>(Inner{z}, zt, g, pp, S, gk, st)) != cudaSuccess) return e;
   if (g.dim >= 2 && (e = dst_y_pass<Tc>(Inner{z}, zt, g, pp, S, gk, st)) != cudaSuccess) return e;
+  // a caller's contiguous output: the last pass leaves the padding out
+  if (user) {
+    if (sizeof(Tc) == sizeof(float) && pp.sop_x != nullptr)
+      return launch_dst_tma_x(reinterpret_cast<float *>(z), g, pp.sop_x, S, gk, st,
+                              reinterpret_cast<float *>(user));
+    return launch_dst<Tc, SrcArray<Tc, Tout>, Tout, true>(SrcArray<Tc, Tout>{z}, user, g.mx, pp.Lx,
+                                                          nx, g.mx, 0, 0, lay<Tc>(g).px, g.mx,
+                                                          tw_of<Tc>(pp, true), S, gk,
+                                                          pp.dst_shift, st);
+  }
   return dst_x_last_pass<Tc>(z, g, pp, S, gk, st);
 }
 
@@ -985,6 +1069,21 @@ template <class Tc, class Tin, class Tout>
 cudaError_t launch_prec(const Geom &g, const PrecPlan &pp, const Tin *v, Tout *z, State *S,
                         int tmode, double *partials, cudaStream_t st) {
   return prec_stages<Tc>(g, pp, SrcArray<Tc, Tin>{v}, z, S, tmode, partials, st);
+}
+
+// z = P^-1 v in float32 into a caller's contiguous vector, by way of the padded scratch: the last x
+// pass writes it, or (the P_theta paths that end with a time transform) a copy.
+cudaError_t launch_prec_user(const Geom &g, const PrecPlan &pp, const double *v, float *scratch,
+                             float *out, State *S, double *partials, cudaStream_t st) {
+  const bool direct = !pp.cheb && !pp.pcr;
+  cudaError_t e = prec_stages<float>(g, pp, SrcArray<float, double>{v}, scratch, S, TM_NONE,
+                                     partials, st, nullptr, direct ? out : nullptr);
+  if (e != cudaSuccess || direct) return e;
+  prof_begin(KC_AUX, st);
+  k_unpad<<<152 * 8, kNT, 0, st>>>((unsigned)((long long)g.n * g.my * g.mz), g.mx, g.px, scratch,
+                                   out);
+  prof_end(st);
+  return cudaGetLastError();
 }
 
 // One MINRES iteration's preconditioner pass with the Lanczos step fused into its first stage:
@@ -1002,49 +1101,29 @@ cudaError_t launch_prec_lanczos(const Geom &g, const PrecPlan &pp, const Tin *q,
 
 // Autotuning helpers: the spatial DSTs (x then y, in place) and the FFMA time kernel alone,
 // ungated, with the knobs currently in pp.
+template <class T>
+static cudaError_t run_dsts(const Geom &g, const PrecPlan &pp, T *z, cudaStream_t st) {
+  using A = SrcArray<T, T>;
+  const Lay y = lay<T>(g);
+  const long long nx = (long long)g.n * g.my * g.mz, ny = (long long)g.n * g.mz * g.mx;
+  cudaError_t e = launch_dst<T, A, T, true>(A{z}, z, g.mx, pp.Lx, nx, g.mx, 0, 0, y.px, y.px,
+                                            tw_of<T>(pp, true), nullptr, GK_NONE, pp.dst_shift,
+                                            st);
+  if (e == cudaSuccess && g.dim >= 2)
+    e = launch_dst<T, A, T, false>(A{z}, z, g.my, pp.Ly, ny, g.mx, y.px, y.pl, g.mx, g.mx,
+                                   tw_of<T>(pp, false), nullptr, GK_NONE, pp.dst_shift, st);
+  if (e == cudaSuccess && g.dim == 3)
+    e = launch_dst<T, A, T, false>(A{z}, z, g.mz, pp.Lz, (long long)g.n * y.pl, (int)y.pl, y.pl,
+                                   y.mp, y.px, g.mx, twz_of<T>(pp), nullptr, GK_NONE, pp.dst_shift, st);
+  return e;
+}
+
 cudaError_t tune_run_dsts(const Geom &g, const PrecPlan &pp, bool fp32, void *data,
                           cudaStream_t st) {
-  const long long nx = (long long)g.n * g.my * g.mz, ny = (long long)g.n * g.mz * g.mx;
-  const long long nz = (long long)g.n * g.mx * g.my;
-  cudaError_t e;
-  if (fp32) {
-    float *z = (float *)data;
-    using A = SrcArray<float, float>;
-    e = launch_dst<float, A, float, true>(A{z}, z, g.mx, pp.Lx, nx, g.mx, g.m, pp.twx_f, nullptr,
-                                          GK_NONE, pp.dst_shift, st);
-    if (e == cudaSuccess && g.dim >= 2)
-      e = launch_dst<float, A, float, false>(A{z}, z, g.my, pp.Ly, ny, g.mx,
-                                             (long long)g.mx * g.my, pp.twy_f, nullptr, GK_NONE,
-                                             pp.dst_shift, st);
-    if (e == cudaSuccess && g.dim == 3)
-      e = launch_dst<float, A, float, false>(A{z}, z, g.mz, pp.Lz, nz, g.mx * g.my, g.m,
-                                             pp.twz_f, nullptr, GK_NONE, pp.dst_shift, st);
-  } else if (pp.fp64_dd) {
-    // the float64 path's double-float engine: its own FFT kernels (double-float data in place)
-    dd *z = (dd *)data;
-    using A = SrcArray<dd, dd>;
-    e = launch_dst<dd, A, dd, true>(A{z}, z, g.mx, pp.Lx, nx, g.mx, g.m, pp.twx_dd, nullptr,
-                                    GK_NONE, pp.dst_shift, st);
-    if (e == cudaSuccess && g.dim >= 2)
-      e = launch_dst<dd, A, dd, false>(A{z}, z, g.my, pp.Ly, ny, g.mx, (long long)g.mx * g.my,
-                                       pp.twy_dd, nullptr, GK_NONE, pp.dst_shift, st);
-    if (e == cudaSuccess && g.dim == 3)
-      e = launch_dst<dd, A, dd, false>(A{z}, z, g.mz, pp.Lz, nz, g.mx * g.my, g.m, pp.twz_dd,
-                                       nullptr, GK_NONE, pp.dst_shift, st);
-  } else {
-    double *z = (double *)data;
-    using A = SrcArray<double, double>;
-    e = launch_dst<double, A, double, true>(A{z}, z, g.mx, pp.Lx, nx, g.mx, g.m, pp.twx_d,
-                                            nullptr, GK_NONE, pp.dst_shift, st);
-    if (e == cudaSuccess && g.dim >= 2)
-      e = launch_dst<double, A, double, false>(A{z}, z, g.my, pp.Ly, ny, g.mx,
-                                               (long long)g.mx * g.my, pp.twy_d, nullptr,
-                                               GK_NONE, pp.dst_shift, st);
-    if (e == cudaSuccess && g.dim == 3)
-      e = launch_dst<double, A, double, false>(A{z}, z, g.mz, pp.Lz, nz, g.mx * g.my, g.m,
-                                               pp.twz_d, nullptr, GK_NONE, pp.dst_shift, st);
-  }
-  return e;
+  if (fp32) return run_dsts<float>(g, pp, (float *)data, st);
+  // the float64 path's double-float engine has its own FFT kernels (double-float data in place)
+  if (pp.fp64_dd) return run_dsts<dd>(g, pp, (dd *)data, st);
+  return run_dsts<double>(g, pp, (double *)data, st);
 }
 
 cudaError_t tune_run_pass(const Geom &g, const PrecPlan &pp, int axis,
@@ -1080,9 +1159,6 @@ cudaError_t tune_run_time(const Geom &g, const PrecPlan &pp, bool fp32, void *da
 template cudaError_t launch_prec<double, double, double>(const Geom &, const PrecPlan &,
                                                          const double *, double *, State *, int,
                                                          double *, cudaStream_t);
-template cudaError_t launch_prec<float, double, float>(const Geom &, const PrecPlan &,
-                                                       const double *, float *, State *, int,
-                                                       double *, cudaStream_t);
 template cudaError_t launch_prec<float, df, float>(const Geom &, const PrecPlan &, const df *,
                                                    float *, State *, int, double *, cudaStream_t);
 template cudaError_t launch_prec_lanczos<double, double, double>(const Geom &, const PrecPlan &,
@@ -1090,11 +1166,6 @@ template cudaError_t launch_prec_lanczos<double, double, double>(const Geom &, c
                                                                  double *, double *, State *,
                                                                  double *, cudaStream_t,
                                                                  cudaEvent_t);
-template cudaError_t launch_prec_lanczos<float, double, float>(const Geom &, const PrecPlan &,
-                                                               const double *, const double *,
-                                                               double *, float *, State *,
-                                                               double *, cudaStream_t,
-                                                               cudaEvent_t);
 template cudaError_t launch_prec_lanczos<float, df, float>(const Geom &, const PrecPlan &,
                                                            const df *, const df *, df *, float *,
                                                            State *, double *, cudaStream_t,

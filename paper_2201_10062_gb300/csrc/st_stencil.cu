@@ -8,6 +8,8 @@
 // and Y only reverses the block order, so row k of T v is written to block n-1-k.
 // One thread owns one spatial node and walks a chunk of consecutive time levels (and their
 // mirror images), carrying neighbouring planes in registers so that each plane of v is read once.
+#include <type_traits>
+
 #include "st_internal.cuh"
 
 namespace st {
@@ -106,6 +108,7 @@ __global__ void __launch_bounds__(kNT) k_stencil(Geom g, const Tz *__restrict__ 
   if (valid) {
     const int jz = j / g.my, jy = j - jz * g.my;
     const long long p = (long long)j * mx + i;
+    const long long po = std::is_same<TO, df>::value ? (long long)j * g.px + i : p;
     const Faces6<double> fc = faces_at(g, i, jy, jz);
     const double th = g.theta, omth = 1.0 - g.theta;
     auto center = [&](int k) -> double { return ld(z + (long long)k * m + p); };
@@ -163,8 +166,10 @@ __global__ void __launch_bounds__(kNT) k_stencil(Geom g, const Tz *__restrict__ 
           b1 = nb2;
         }
       }
-      const long long oA = (long long)kB * m + p;  // block n-1-kA receives row kA
-      const long long oB = (long long)kA * m + p;  // block n-1-kB = kA receives row kB
+      // block n-1-kA receives row kA, block n-1-kB = kA row kB (double-float output is padded)
+      const long long mo = std::is_same<TO, df>::value ? g.mp : m;
+      const long long oA = (long long)kB * mo + po;
+      const long long oB = (long long)kA * mo + po;
       if (MODE == SM_MINRES) {
         yA *= s;
         put(out + oA, yA);
@@ -298,8 +303,9 @@ __global__ void __launch_bounds__(kNT, D3 ? 3 : 4) k_stencil_df(Geom g, const fl
   if (lead && S->restart) S->restart = 0;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;  // row jz*my + jy
-  const int mx = g.mx, my = g.my, dim = g.dim, n = g.n;
-  const long long m = g.m, pl = (long long)mx * my;
+  // z and out are padded: px slots a line, m a level
+  const int mx = g.mx, my = g.my, dim = g.dim, n = g.n, px = g.px;
+  const long long m = g.mp, pl = (long long)px * my;
   const bool valid = (i < mx) && (j < my * g.mz);
   const int half = (n + 1) >> 1;
   const int k0 = blockIdx.z * kc;
@@ -307,7 +313,7 @@ __global__ void __launch_bounds__(kNT, D3 ? 3 : 4) k_stencil_df(Geom g, const fl
   acc_df D{0.f, 0.f};
   if (valid) {
     const int jz = D3 ? j / my : 0, jy = j - jz * my;
-    const long long p = (long long)j * mx + i;
+    const long long p = (long long)j * px + i;
     const df zero_f{0.f, 0.f};
     const Faces6<df> fc = UNI ? Faces6<df>{zero_f, zero_f, zero_f, zero_f, zero_f, zero_f}
                               : faces_df_at(g, i, jy, jz);
@@ -348,10 +354,10 @@ __global__ void __launch_bounds__(kNT, D3 ? 3 : 4) k_stencil_df(Geom g, const fl
       const float *b = z + (long long)k * m + p;
       P5 r;
       r.c = __ldg(b);
-      r.w = i > 0 ? __ldg(b - 1) : 0.f;
-      r.e = i < mx - 1 ? __ldg(b + 1) : 0.f;
-      r.s = (dim >= 2 && jy > 0) ? __ldg(b - mx) : 0.f;
-      r.n = (dim >= 2 && jy < my - 1) ? __ldg(b + mx) : 0.f;
+      r.w = __ldg(b - 1);  // the padding slots on either side of a line hold the boundary's zeros
+      r.e = __ldg(b + 1);
+      r.s = (dim >= 2 && jy > 0) ? __ldg(b - px) : 0.f;
+      r.n = (dim >= 2 && jy < my - 1) ? __ldg(b + px) : 0.f;
       r.d = (D3 && jz > 0) ? __ldg(b - pl) : 0.f;
       r.u = (D3 && jz < g.mz - 1) ? __ldg(b + pl) : 0.f;
       return r;
