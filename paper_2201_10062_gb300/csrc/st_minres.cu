@@ -546,15 +546,22 @@ size_t zslab_floats(const Geom &g, int ugroup) {
          (size_t)(kUpdRing + 1) * (size_t)(g.Np - g.N);
 }
 
-// the axes of a mixed handle that the tensor-core transforms take (st_dst_tma.cu): 32-column
-// tiles and, along x, whole 32-element chunks
-bool tc_time_ok(const Geom &g) { return dst_tma_supported(g.n) && g.mp >= 32; }
+// The axes of a mixed handle that the tensor-core transforms take (st_dst_tma.cu): 32-column tiles
+// and, along x, whole 32-element chunks.  A launch of theirs takes 9 (one axis) or 19 us (time) however
+// small the vector, so small ones stay on the CUDA cores: along y and z below 3 2^18 unknowns (127^2 x
+// 48: 11.2 us either way; 63^2 x 96: 11.7 against 9.7 by FFT; 255^2 x 48: 14.1 against 20.2), along
+// time below 2^19 where n < 64 (127^2 x 31: 19.4 either way; 63^2 x 48: 23.8 against 22.0 by FFMA;
+// 255^2 x 16: 24.3 against 33.4; from n = 64 on the tensor cores win at every size).
+bool tc_time_ok(const Geom &g) {
+  return dst_tma_supported(g.n) && g.mp >= 32 && (g.n >= 64 || g.N >= (1LL << 19));
+}
 bool tc_x_ok(const Geom &g) { return g.mx >= 31 && dst_tma_supported(g.mx); }
 bool tc_y_ok(const Geom &g) {
-  return g.dim >= 2 && g.my >= 31 && g.px >= 32 && dst_tma_supported(g.my);
+  return g.dim >= 2 && g.my >= 31 && g.px >= 32 && dst_tma_supported(g.my) && g.N >= (3LL << 18);
 }
 bool tc_z_ok(const Geom &g) {
-  return g.dim == 3 && g.mz >= 31 && (long long)g.px * g.my >= 32 && dst_tma_supported(g.mz);
+  return g.dim == 3 && g.mz >= 31 && (long long)g.px * g.my >= 32 && dst_tma_supported(g.mz) &&
+         g.N >= (3LL << 18);
 }
 
 size_t workspace_bytes(const Geom &g, bool mixed, int cheb, int ugroup) {

@@ -461,12 +461,15 @@ struct TcdSmem {
   uint32_t bdig, ytile, part, cdown, tmu, mbar, tmem, total;
 };
 
+// folded rows padded to the MMA's K step (rows past the fold are zero digits)
+__host__ __device__ inline int tcd_hk(int n) { return ((n + 1) / 2 + 15) & ~15; }
+
 __host__ __device__ inline TcdSmem tcd_layout(int n) {
-  const int h = n / 2;
+  const int h = (n + 1) / 2, hK = tcd_hk(n);
   TcdSmem L{};
   uint32_t o = 0;
-  L.bdig = o;  // two buffers of [digit][32][h] fp16
-  o += 2u * kDg * kTN * (uint32_t)h * 2u;
+  L.bdig = o;  // two buffers of [digit][32][hK] fp16
+  o += 2u * kDg * kTN * (uint32_t)hK * 2u;
   L.ytile = o;  // the drain warps' staged rows: hi floats then lo floats, [h][kYS]
   o += 2u * (uint32_t)h * kYS * 4u;
   L.part = o;  // 8 build warps x 32 per-column partial maxima
@@ -560,10 +563,10 @@ __global__ void __launch_bounds__(kNTG, 1)
   __shared__ double red[32];
   if (gate_closed(S, gk)) return;
   extern __shared__ __align__(1024) unsigned char smem[];
-  const int h = n >> 1, hb = h >> 3;
+  const int h = (n + 1) >> 1, hK = tcd_hk(n), hb = hK >> 3;
   const TcdSmem L = tcd_layout(n);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const uint32_t bop = (uint32_t)kTN * h * 2u;   // one digit's B operand
+  const uint32_t bop = (uint32_t)kTN * hK * 2u;  // one digit's B operand
   const uint32_t bbytes = (uint32_t)kDg * bop;   // one B buffer
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + L.tmem);
   float *yhi = reinterpret_cast<float *>(smem + L.ytile);
@@ -601,7 +604,7 @@ __global__ void __launch_bounds__(kNTG, 1)
     }
   }
   const uint32_t tmem = *tmem_slot;
-  const uint32_t acol = (uint32_t)(h / 2);            // tensor-memory columns of one S digit
+  const uint32_t acol = (uint32_t)(hK / 2);           // tensor-memory columns of one S digit
   const uint32_t dcol = tmem + (uint32_t)kDg * acol;  // the two accumulators follow S
   bool ok = true;
   // phases of bfull, bempty, afull and aempty as this thread's role waits on them
@@ -619,11 +622,11 @@ __global__ void __launch_bounds__(kNTG, 1)
       const int q = warp & 3, nq = (kNTG / 32 - q + 3) / 4, r = (q << 5) + lane;
       const uint32_t tl = (uint32_t)(q * 32) << 16;
       for (int pc = warp >> 2; pc < kDg; pc += nq) {
-        const unsigned char *img = A_g + (size_t)(P * kDg + pc) * kM * h * 2u;
-        for (int ks = 0; ks < h / 16; ++ks) {
+        const unsigned char *img = A_g + (size_t)(P * kDg + pc) * kM * hK * 2u;
+        for (int ks = 0; ks < hK / 16; ++ks) {
           uint32_t w[8];
-          const uint4 a0 = *reinterpret_cast<const uint4 *>(img + canon_off(r, ks * 16, h));
-          const uint4 a1 = *reinterpret_cast<const uint4 *>(img + canon_off(r, ks * 16 + 8, h));
+          const uint4 a0 = *reinterpret_cast<const uint4 *>(img + canon_off(r, ks * 16, hK));
+          const uint4 a1 = *reinterpret_cast<const uint4 *>(img + canon_off(r, ks * 16 + 8, hK));
           w[0] = a0.x; w[1] = a0.y; w[2] = a0.z; w[3] = a0.w;
           w[4] = a1.x; w[5] = a1.y; w[6] = a1.z; w[7] = a1.w;
           tmem_st8(tmem + tl + (uint32_t)pc * acol + (uint32_t)ks * 8u, w);
@@ -648,8 +651,8 @@ __global__ void __launch_bounds__(kNTG, 1)
           pbf ^= 1u << b;
           // descriptors differ only in their start-address field (address / 16), so each MMA
           // takes one add on a descriptor built once per tile
-          const uint64_t bdesc = make_desc(smem_u32(smem + L.bdig) + (uint32_t)b * bbytes, h);
-          const int ksteps = h / 16;
+          const uint64_t bdesc = make_desc(smem_u32(smem + L.bdig) + (uint32_t)b * bbytes, hK);
+          const int ksteps = hK / 16;
           for (int g = 0; g < kDg; ++g) {
             const int a = (int)(G & 1u);
             if (!mbar_wait(aempty + 8u * a, ((pae >> a) & 1u))) {
@@ -696,11 +699,16 @@ __global__ void __launch_bounds__(kNTG, 1)
 #pragma unroll
           for (int q = 0; q < 8; ++q) {
             f[it][q] = dd(0.f, 0.f);
-            if (tb < hb && bc < je) {
-              const int t = tb * 8 + q;
+            const int t = tb * 8 + q, tm = n - 1 - t;
+            if (t <= tm && bc < je) {
               const dd x1 = ld_dd(in + (long long)t * m + j0 + bc);
-              const dd x2 = ld_dd(in + (long long)(n - 1 - t) * m + j0 + bc);
-              f[it][q] = P == 0 ? x1 + x2 : x1 - x2;
+              if (t == tm) {
+                // the middle row of an odd n: only odd k see it
+                if (P == 0) f[it][q] = x1;
+              } else {
+                const dd x2 = ld_dd(in + (long long)tm * m + j0 + bc);
+                f[it][q] = P == 0 ? x1 + x2 : x1 - x2;
+              }
               mxv = fmaxf(mxv, fabsf(f[it][q].hi));
             }
           }
@@ -726,7 +734,7 @@ __global__ void __launch_bounds__(kNTG, 1)
           int dq[8][kDg];
 #pragma unroll
           for (int q = 0; q < 8; ++q) digits7(f[it][q], up21, dq[q]);
-          const uint32_t off = canon_off(bc, tb * 8, h);
+          const uint32_t off = canon_off(bc, tb * 8, hK);
 #pragma unroll
           for (int dg = 0; dg < kDg; ++dg) {
             uint32_t pk[4];
@@ -855,23 +863,27 @@ __global__ void __launch_bounds__(kNTG, 1)
 
 }  // namespace
 
-// n a multiple of 32 up to 256 (h = n/2 folded rows, a multiple of the MMA K step; seven S
-// digits of h/2 columns plus two 32-column accumulators within the 512 tensor-memory columns),
-// and the layout within the 227 KB a block may opt into (with 1 KB of static shared memory)
+// Multiples of 32 up to 256, and every n from 129 to 256 (ceil(n/2) folded rows, padded to the MMA K
+// step; seven S digits of half as many columns plus two 32-column accumulators within the 512
+// tensor-memory columns; the layout within the 227 KB a block may opt into, with 1 KB of static
+// shared memory).  At 127 x 255 spatial points, one P_H pass with this stage against the
+// double-float CUDA-core one: n = 243 923 against 1751 us, n = 200 813 against 1270 (errors against
+// float64 equal to 0.2%), but n = 100 521 against 531 and n = 50 377 against 236: between the
+// multiples of 32 below 128 the CUDA cores stay.
 bool time_tcd_supported(int n) {
-  if (n < 32 || n > 256 || (n % 32) != 0) return false;
-  if (kDg * (n / 4) + 2 * kTN > 512) return false;
+  if (n < 32 || n > 256 || (n <= 128 && n % 32 != 0)) return false;
+  if (kDg * (tcd_hk(n) / 2) + 2 * kTN > 512) return false;
   return tcd_layout(n).total + 1024u <= 227u * 1024u;
 }
 
-size_t time_tcd_bytes(int n) { return (size_t)2 * kDg * kM * (size_t)(n / 2) * 2; }
+size_t time_tcd_bytes(int n) { return (size_t)2 * kDg * kM * (size_t)tcd_hk(n) * 2; }
 
 // Host: the digit image of S_n for k_time_tcd: piece (parity P, digit i) at index P * 7 + i, the
-// rows r of parity P (k = 2r+1 or 2r+2) by K = h folded columns, canonical K-major fp16; the
+// rows r of parity P (k = 2r+1 or 2r+2) by K = hK folded columns, canonical K-major fp16; the
 // digits of S 2^eS (integers, |.| <= 2^7) are taken in float64, where they are exact.
 // Returns eS.
 int time_tcd_build(int n, unsigned char *out) {
-  const int h = n / 2;
+  const int h = (n + 1) / 2, hK = tcd_hk(n);
   const double PI = 3.14159265358979323846;
   const double sn = std::sqrt(2.0 / (n + 1));
   double smax = 0.0;
@@ -882,7 +894,7 @@ int time_tcd_build(int n, unsigned char *out) {
   std::frexp(smax, &E);
   const int eS = 7 - E;  // smax 2^eS in [2^6, 2^7)
   unsigned short *o = reinterpret_cast<unsigned short *>(out);
-  const size_t piece = (size_t)kM * h;  // halves
+  const size_t piece = (size_t)kM * hK;  // halves
   for (size_t i = 0; i < time_tcd_bytes(n) / 2; ++i) o[i] = 0;
   for (int P = 0; P < 2; ++P)
     for (int r = 0; r < h; ++r) {
@@ -895,7 +907,7 @@ int time_tcd_build(int n, unsigned char *out) {
           v = (v - q) * 128.0;
           const __half hq = __float2half_rn((float)q);
           __half_raw raw = hq;
-          o[(size_t)(P * kDg + dg) * piece + canon_off(r, t, h) / 2] = raw.x;
+          o[(size_t)(P * kDg + dg) * piece + canon_off(r, t, hK) / 2] = raw.x;
         }
       }
     }

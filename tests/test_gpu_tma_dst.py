@@ -30,6 +30,12 @@ CASES += [(1, 31, 1, 1, 100), (2, 31, 63, 1, 65), (2, 63, 31, 1, 30), (2, 127, 1
           (2, 255, 31, 1, 129), (2, 31, 255, 1, 21), (2, 255, 255, 1, 24), (2, 15, 63, 1, 50),
           (3, 31, 31, 31, 20), (3, 15, 63, 31, 18), (3, 63, 15, 127, 16)]
 
+# sizes at which every axis takes the tensor cores by default (small vectors keep the CUDA cores along
+# y, z and, for n < 64, time)
+CASES += [(2, 255, 255, 1, n) for n in (16, 17, 31, 33, 48, 63)]
+CASES += [(2, 127, 127, 1, 64), (2, 255, 63, 1, 65), (2, 511, 31, 1, 60), (2, 255, 127, 1, 40),
+          (3, 31, 31, 31, 32), (3, 31, 63, 127, 16)]
+
 
 # 2e-5: float32 transforms, 22-bit operand split with float32 accumulation.  (Against float64 the
 # symbol's float32 tables add their own error on anisotropic grids, the same in both engines.)
