@@ -31,13 +31,11 @@
 // tiles with its warps in separate roles that hand off through mbarriers, every wait bounded.  On a
 // timeout the block records ST_ERR_TIMEOUT and stops; before it frees its tensor memory every MMA
 // must be known to be complete, else it keeps it and sets State::tmem_held (see tc_release_cols).
-#include <cuda.h>
-
 #include <cmath>
 #include <cstdlib>
 #include <type_traits>
 
-#include "st_tc.cuh"
+#include "st_tma.cuh"
 
 namespace st {
 namespace {
@@ -73,25 +71,6 @@ __host__ __device__ inline TmaDim tma_dim(int len, int SL) {
   return d;
 }
 
-__device__ __forceinline__ uint64_t make_desc_sbo(uint32_t saddr, uint32_t sbo) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFF);
-  d |= (uint64_t)(128u >> 4) << 16;
-  d |= (uint64_t)((sbo >> 4) & 0x3FFF) << 32;
-  d |= (uint64_t)1 << 46;
-  return d;
-}
-
-template <int N>
-__device__ __forceinline__ void mma_ta(uint32_t dtmem, uint32_t atmem, uint64_t bd, uint32_t acc) {
-  constexpr uint32_t idesc = (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kM >> 4) << 24);
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(dtmem),
-      "r"(atmem), "l"(bd), "r"(idesc), "r"(acc));
-}
-
 // B operand: [parity][column set][hi, lo][8-column group], a column set being the columns that one
 // slot multiplies: the tile's 32 (SL 1) or 64 (SL 2) columns, or half of its 128 (SL 4).
 template <int SL>
@@ -125,119 +104,9 @@ __device__ __forceinline__ void issue_tile(uint32_t a_base, uint32_t bop, const 
   }
 }
 
-// S into tensor memory: variant (slot, piece) at columns variant * hK / 2, from the host image
-// [variant][hK / 16][128 rows][16 halves]; `nw` warps of the block share the work
-template <int SL>
-__device__ __forceinline__ void load_a(const uint4 *img, int hK, uint32_t a_base, int warp, int nw,
-                                       int lane) {
-  const int q = warp & 3, nq = (nw - q + 3) / 4, KS = hK >> 4, cnt = 2 * num_slots(SL) * KS;
-  const uint32_t lanes = (uint32_t)(q * 32) << 16;
-  // four pieces' loads in flight before the first store: one at a time, the latency of eight loads in
-  // a row was 4 of a 30 us launch
-  for (int i0 = warp >> 2; i0 < cnt; i0 += 4 * nq) {
-    uint4 c[4][2];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int i = i0 + k * nq;
-      if (i < cnt) {
-        const uint4 *p = img + ((size_t)i * kM + (size_t)(q * 32 + lane)) * 2;
-        c[k][0] = __ldg(p);
-        c[k][1] = __ldg(p + 1);
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int i = i0 + k * nq;
-      if (i < cnt) {
-        const uint32_t w[8] = {c[k][0].x, c[k][0].y, c[k][0].z, c[k][0].w,
-                               c[k][1].x, c[k][1].y, c[k][1].z, c[k][1].w};
-        const int v = i / KS, ks = i - v * KS;
-        tmem_st8(a_base + lanes + (uint32_t)(v * (hK >> 1) + ks * 8), w);
-      }
-    }
-  }
-  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-}
-
-// ---------------------------------------------------------------- tensor copies
-__device__ __forceinline__ void tma_load3(uint32_t dst, const CUtensorMap *map, int x, int y, int z,
-                                          uint32_t mbar) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, "
-      "%3, %4}], [%5];" ::"r"(dst),
-      "l"(map), "r"(x), "r"(y), "r"(z), "r"(mbar)
-      : "memory");
-}
-__device__ __forceinline__ void tma_store3(const CUtensorMap *map, uint32_t src, int x, int y,
-                                           int z) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(map),
-      "r"(x), "r"(y), "r"(z), "r"(src)
-      : "memory");
-}
-__device__ __forceinline__ void bulk_commit() {
-  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-}
-// this thread's stores have read their shared memory / are complete
-__device__ __forceinline__ void bulk_wait_read() {
-  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-}
-__device__ __forceinline__ void bulk_wait_done() {
-  asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-}
-
-__device__ __forceinline__ float4 lds4(uint32_t a) {
-  float4 v;
-  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-               : "r"(a));
-  return v;
-}
-__device__ __forceinline__ float lds1(uint32_t a) {
-  float v;
-  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ void sts4(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
-  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(x), "r"(y), "r"(z), "r"(w)
-               : "memory");
-}
-__device__ __forceinline__ void sts4f(uint32_t a, float x, float y, float z, float w) {
-  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(x), "f"(y), "f"(z), "f"(w)
-               : "memory");
-}
-__device__ __forceinline__ void sts2f(uint32_t a, float x, float y) {
-  asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(x), "f"(y) : "memory");
-}
-__device__ __forceinline__ void sts1f(uint32_t a, float x) {
-  asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(x) : "memory");
-}
-
 // ---------------------------------------------------------------- fold, scale, split
-// A build set is 128 threads.  Each thread holds four vectors of eight folded rows (one t-block):
-// strided lines: four adjacent columns of one t-block; x lines: four t-blocks of one line.
-//
-// Column scale: the power of two that brings the column's largest folded value m into [2^13, 2^14)
-// (1 for m = 0 or not finite), and 1 / (8 scale).
-__device__ __forceinline__ float scale_of(float m) {
-  const int E = (int)((__float_as_uint(m) >> 23) & 255u);  // m in [2^(E-127), 2^(E-126))
-  if (m == 0.f || E == 255) return 1.0f;
-  const int s = 267 - E;  // biased exponent of 2^(14 - (E - 126))
-  return __uint_as_float((uint32_t)(s > 254 ? 254 : s) << 23);
-}
-__device__ __forceinline__ float inv_scale(float s) {
-  return (1.0f / s) * (1.0f / kSScale);
-}
-
-// eight folded rows of one column and parity, times the scale, as the hi and lo pieces
-__device__ __forceinline__ void put_piece(uint32_t a, uint32_t ph, const float (&v)[8], float sc) {
-  uint32_t hi[4], lo[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) split_h2(v[2 * q] * sc, v[2 * q + 1] * sc, hi[q], lo[q]);
-  sts4(a, hi[0], hi[1], hi[2], hi[3]);
-  sts4(a + ph, lo[0], lo[1], lo[2], lo[3]);
-}
-
+// A build set is 128 threads (256 with two columns a thread).  Each thread holds vectors of eight folded
+// rows: strided lines, four (two) adjacent columns of one t-block; x lines, four t-blocks of one line.
 template <int NC>
 __device__ __forceinline__ void lds_cols(uint32_t a, float (&v)[NC]) {
   if constexpr (NC == 4) {
@@ -403,13 +272,7 @@ __device__ __forceinline__ bool build_xlines(uint32_t buf, uint32_t bop, uint32_
 // 16 values of one unit: the hi and lo halves of the accumulator summed
 template <int SL>
 __device__ __forceinline__ void tmem_unit16(uint32_t acc, int j, int k, float (&v)[16]) {
-  const uint32_t hi = acc + (SL == 1 ? 64u : 32u) * (uint32_t)j + 16u * (uint32_t)k;
-  uint32_t a[16], b[16];
-  tmem_ld16_async(hi, a);
-  tmem_ld16_async(hi + (SL == 1 ? 32u : 64u), b);
-  tmem_wait_ld();
-#pragma unroll
-  for (int c = 0; c < 16; ++c) v[c] = __uint_as_float(a[c]) + __uint_as_float(b[c]);
+  tmem_sum16(acc + (SL == 1 ? 64u : 32u) * (uint32_t)j + 16u * (uint32_t)k, SL == 1 ? 32u : 64u, v);
 }
 template <int SL>
 __device__ __forceinline__ void tmem_unit(uint32_t acc, int j, float (&v)[32]) {
@@ -539,7 +402,7 @@ __global__ void __launch_bounds__(kNTS, 1)
     for (unsigned tile = first; tile < ntiles && preloaded < (uint32_t)NB; tile += step)
       load(tile, (int)preloaded++);
   __syncwarp();
-  load_a<SL>(img, D.hK, tmem, warp, kNTS / 32, lane);
+  load_a_variants(img, 2 * num_slots(SL), D.hK, tmem, warp, kNTS / 32, lane);
   fence_before();
   __syncthreads();
   fence_after();
@@ -766,24 +629,6 @@ __device__ __forceinline__ void regs_inc() {
 }
 __device__ __forceinline__ void warpgroup_sync() { group_sync(3 + (threadIdx.x >> 7), 128); }
 
-// 1/p of row r and column factor tmu for one kind of symbol (0: theta, 1: BDF2, 2: P_theta); the
-// kinds are compiled apart so that the unrolled epilogue stays small
-template <int KIND>
-__device__ __forceinline__ float inv_sym_k(const SymRow &r, float omth, float tmu) {
-  if (KIND == 2) return 1.0f / (r.a + r.b * tmu);
-  float re, im;
-  if (KIND == 0) {
-    re = r.a + tmu * r.b;
-    im = (-1.0f + omth * tmu) * r.c;
-  } else {
-    re = r.a + tmu;
-    im = r.c;
-  }
-  float y;  // p is far from the subnormal range
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(re * re + im * im));
-  return y;
-}
-
 template <int SL>
 struct TimeSmem {
   // full, yfull, ofull, oempty [8 each]; b1full, b1empty, b2full, b2empty, a1full, a1empty, a2full,
@@ -858,7 +703,7 @@ __global__ void __launch_bounds__(kNTT, 1)
     for (unsigned tile = first; tile < ntiles && preloaded < (uint32_t)NB; tile += step)
       load(tile, (int)preloaded++);
   __syncwarp();
-  load_a<SL>(img, D.hK, tmem, warp, kNTT / 32, lane);
+  load_a_variants(img, 2 * num_slots(SL), D.hK, tmem, warp, kNTT / 32, lane);
   fence_before();
   __syncthreads();
   fence_after();
@@ -1095,40 +940,6 @@ __global__ void __launch_bounds__(kNTT, 1)
 // ---------------------------------------------------------------- host
 constexpr uint32_t kSmemMax = 227u * 1024u;
 
-typedef CUresult (*EncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
-                             const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
-                             const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
-                             CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeFn encode_fn() {
-  static const EncodeFn f = [] {
-    void *p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
-                                         &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess)
-      p = nullptr;
-    return reinterpret_cast<EncodeFn>(p);
-  }();
-  return f;
-}
-
-// float32 tensor [d2][d1][d0], rows s1 floats apart, planes s2 floats apart; boxes of 32 x b1 x 1
-// in 128-byte-swizzled rows.  Bases and strides are multiples of 16 bytes in the padded layout,
-// and every copy starts at a multiple of 32 columns.
-cudaError_t encode(CUtensorMap *m, const float *base, long long d0, long long d1, long long d2,
-                   long long s1, long long s2, int b1) {
-  const EncodeFn f = encode_fn();
-  if (!f) return cudaErrorNotSupported;
-  const cuuint64_t dims[3] = {(cuuint64_t)d0, (cuuint64_t)d1, (cuuint64_t)d2};
-  const cuuint64_t str[2] = {(cuuint64_t)s1 * 4u, (cuuint64_t)s2 * 4u};
-  const cuuint32_t box[3] = {32u, (cuuint32_t)b1, 1u}, es[3] = {1u, 1u, 1u};
-  const CUresult r = f(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float *>(base), dims, str,
-                       box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                       CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
-}
-
 int ring_of(uint32_t fixed, uint32_t rb) {
   int nb = (int)((kSmemMax - 1024u - fixed) / rb);
   return nb > kMaxRing ? kMaxRing : nb;
@@ -1150,15 +961,15 @@ cudaError_t launch_dst(const float *in, float *out, int len, long long cols, lon
   if (XL) {
     chunks = (len + 1) / 32;
     groups = (unsigned)planes;  // lines
-    e = encode(&mi, in, len + 1, planes, 1, len + 1, (long long)(len + 1) * planes, 32 * SL);
+    e = tma_encode(&mi, in, len + 1, planes, 1, len + 1, (long long)(len + 1) * planes, 32 * SL);
     m0 = m1 = mi;
   } else {
     chunks = (int)((cols + 31) / 32);
     groups = (unsigned)(planes * chunks);
-    e = encode(&mi, in, cols, len, planes, rs, ps, len);
+    e = tma_encode(&mi, in, cols, len, planes, rs, ps, len);
     if (e == cudaSuccess)
-      e = encode(&m0, out, cols, (len + 1) / 2, planes, 2 * rs, ps, D.h);
-    if (e == cudaSuccess) e = encode(&m1, out + rs, cols, len / 2, planes, 2 * rs, ps, D.h);
+      e = tma_encode(&m0, out, cols, (len + 1) / 2, planes, 2 * rs, ps, D.h);
+    if (e == cudaSuccess) e = tma_encode(&m1, out + rs, cols, len / 2, planes, 2 * rs, ps, D.h);
   }
   if (e != cudaSuccess) return e;
   auto kern = k_dst_tma<SL, XL>;
@@ -1197,9 +1008,9 @@ cudaError_t launch_time(float *data, const Geom &g, const Spec<float> &sp,
   if (smem < 116u * 1024u) smem = 116u * 1024u;
   const unsigned groups = (unsigned)((g.mp + 31) / 32);
   CUtensorMap mi, m0, m1;
-  cudaError_t e = encode(&mi, data, g.mp, g.n, 1, g.mp, g.Np, g.n);
-  if (e == cudaSuccess) e = encode(&m0, data, g.mp, (g.n + 1) / 2, 1, 2 * g.mp, g.Np, D.h);
-  if (e == cudaSuccess) e = encode(&m1, data + g.mp, g.mp, g.n / 2, 1, 2 * g.mp, g.Np, D.h);
+  cudaError_t e = tma_encode(&mi, data, g.mp, g.n, 1, g.mp, g.Np, g.n);
+  if (e == cudaSuccess) e = tma_encode(&m0, data, g.mp, (g.n + 1) / 2, 1, 2 * g.mp, g.Np, D.h);
+  if (e == cudaSuccess) e = tma_encode(&m1, data + g.mp, g.mp, g.n / 2, 1, 2 * g.mp, g.Np, D.h);
   if (e != cudaSuccess) return e;
   auto kern = sp.prec == ST_PREC_PTHETA ? k_time_tma<SL, 2>
               : sp.scheme == ST_THETA    ? k_time_tma<SL, 0>
@@ -1229,8 +1040,7 @@ size_t dst_tma_image_halves(int len) {
 // the slot's rows of the MMA, zeros elsewhere, hi and lo fp16 pieces: [slot][piece][K step][row][16].
 void dst_tma_build_image(int len, unsigned short *out) {
   const int SL = slots_for(len), h = (len + 1) / 2, hK = (h + 15) & ~15;
-  const double PI = 3.14159265358979323846;
-  const double sn = std::sqrt(2.0 / (len + 1));
+  const SinePieces S(len);
   const size_t piece = (size_t)kM * hK;
   for (size_t i = 0; i < dst_tma_image_halves(len); ++i) out[i] = 0;
   for (int s = 0; s < num_slots(SL); ++s) {
@@ -1239,15 +1049,14 @@ void dst_tma_build_image(int len, unsigned short *out) {
     for (int r = 0; r < h; ++r) {
       const int k = 2 * r + 1 + P;
       if (k > len) continue;
+      unsigned short *q = out + (size_t)(2 * s) * piece + (size_t)(row0 + r) * 16;
+      int a = 0;
       for (int t = 0; t < h; ++t) {
-        const long long a = (long long)k * (t + 1) % (2 * (len + 1));
-        const double v = kSScale * sn * std::sin(PI * (double)a / (len + 1));
-        const __half hi = __float2half_rn((float)v);
-        const __half lo = __float2half_rn((float)(v - (double)__half2float(hi)));
-        const __half_raw rh = hi, rl = lo;
-        const size_t off = ((size_t)(t >> 4) * kM + row0 + r) * 16 + (t & 15);
-        out[(size_t)(2 * s) * piece + off] = rh.x;
-        out[(size_t)(2 * s + 1) * piece + off] = rl.x;
+        a += k;
+        if (a >= S.period) a -= S.period;
+        const size_t off = (size_t)(t >> 4) * kM * 16 + (t & 15);
+        q[off] = S.hi[a];
+        q[piece + off] = S.lo[a];
       }
     }
   }

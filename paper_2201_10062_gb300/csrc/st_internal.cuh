@@ -341,8 +341,10 @@ struct PrecPlan {
   const unsigned short *sop_z;  // fp16 S_mz image for the tensor-core z-DST (3D mixed), or null
   const unsigned short *sop_x;  // fp16 S_mx image for the tensor-core x-DST of the last spatial
                                 // pass (mixed), or null
-  const unsigned short *sop_long;  // streamed S_n chunks for the tensor-core time kernel when
-                                   // 256 < n <= 512 (mixed), or null
+  // operand images of the axes of 257 to 512 points (mixed), or null, and the float32 vector (the
+  // stencil output's room, free once the Lanczos step has read it) their transforms go through
+  const unsigned short *sop_long, *sop_ly, *sop_lz;
+  float *fscratch;
   const unsigned char *sdig;  // integer-digit image of S_n for the float64-accurate tensor-core
                               // time kernel (float64 path, double-float engine), or null
   int sdig_e;                 // its scale: the digits are those of S_n 2^sdig_e
@@ -417,12 +419,17 @@ int time_tcd_build(int n, unsigned char *out);  // returns the scale exponent of
 cudaError_t launch_time_tcd(dd *data, dd *scratch, const Geom &g, const Spec<dd> &sp,
                             const unsigned char *img, int eS, State *S, int tmode,
                             double *partials, int gk, cudaStream_t st);
-bool time_tc_long_supported(int n);
-size_t time_tc_long_bytes(int n);
-void time_tc_long_build(int n, unsigned short *out);
-cudaError_t launch_time_tc_long(float *data, const Geom &g, const Spec<float> &sp,
-                                const unsigned short *A, State *S, int tmode, double *partials,
-                                int gk, cudaStream_t st);
+// axes of 257 to 512 points (st_dst_long.cu): out of place, for y, z and the time stage (there and back)
+bool dst_long_supported(int len);
+size_t dst_long_image_halves(int len);
+void dst_long_build_image(int len, unsigned short *out);
+cudaError_t launch_dst_long_y(const float *in, float *out, const Geom &g, const unsigned short *img,
+                              State *S, int gk, cudaStream_t st);
+cudaError_t launch_dst_long_z(const float *in, float *out, const Geom &g, const unsigned short *img,
+                              State *S, int gk, cudaStream_t st);
+cudaError_t launch_time_long(float *data, float *scratch, const Geom &g, const Spec<float> &sp,
+                             const unsigned short *img, State *S, int tmode, double *partials, int gk,
+                             cudaStream_t st);
 
 // energy mode of the time kernel's last block
 enum { TM_NONE = 0, TM_INIT = 1, TM_ITER = 2, TM_RESTART = 3 };

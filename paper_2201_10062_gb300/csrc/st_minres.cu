@@ -564,6 +564,16 @@ bool tc_z_ok(const Geom &g) {
          g.N >= (3LL << 18);
 }
 
+// axes of 257 to 512 points
+bool tc_long_ok(const Geom &g) { return dst_long_supported(g.n) && g.mp >= 32; }
+bool tc_ly_ok(const Geom &g) {
+  return g.dim >= 2 && g.px >= 32 && dst_long_supported(g.my) && g.N >= (3LL << 18);
+}
+bool tc_lz_ok(const Geom &g) {
+  return g.dim == 3 && (long long)g.px * g.my >= 32 && dst_long_supported(g.mz) &&
+         g.N >= (3LL << 18);
+}
+
 size_t workspace_bytes(const Geom &g, bool mixed, int cheb, int ugroup) {
   const size_t N = (size_t)g.N;
   const size_t Nv = mixed ? (size_t)g.Np : N;  // the mixed path's own vectors are padded
@@ -582,7 +592,9 @@ size_t workspace_bytes(const Geom &g, bool mixed, int cheb, int ugroup) {
   b += table_floats(g) * sizeof(dd) + 256;  // double-float copies of the spectral tables
   b += (faces_x(g) + faces_y(g) + faces_z(g)) * sizeof(df) + 256;  // df faces
   if (mixed && tc_time_ok(g)) b += dst_tma_image_halves(g.n) * 2;
-  if (mixed && !tc_time_ok(g) && time_tc_long_supported(g.n)) b += time_tc_long_bytes(g.n) + 256;
+  if (mixed && tc_long_ok(g)) b += dst_long_image_halves(g.n) * 2 + 256;
+  if (mixed && tc_ly_ok(g)) b += dst_long_image_halves(g.my) * 2 + 256;
+  if (mixed && tc_lz_ok(g)) b += dst_long_image_halves(g.mz) * 2 + 256;
   if (mixed && tc_y_ok(g)) b += dst_tma_image_halves(g.my) * 2 + 256;
   if (mixed && tc_z_ok(g)) b += dst_tma_image_halves(g.mz) * 2 + 256;
   if (mixed && tc_x_ok(g)) b += dst_tma_image_halves(g.mx) * 2 + 256;
@@ -814,10 +826,10 @@ int build_tables(st_handle *h) {
   if (use_tc && tc_time_ok(g)) {
     sop.resize(dst_tma_image_halves(n));
     dst_tma_build_image(n, sop.data());
-  } else if (use_tc && time_tc_long_supported(n)) {
-    // streamed chunks for 256 < n <= 512, in the same slot of the table allocation
-    sop.resize(time_tc_long_bytes(n) / 2);
-    time_tc_long_build(n, sop.data());
+  } else if (use_tc && tc_long_ok(g)) {
+    // 256 < n <= 512, in the same slot of the table allocation
+    sop.resize(dst_long_image_halves(n));
+    dst_long_build_image(n, sop.data());
     long_tc = true;
   }
   const size_t o_sop = (bytes_d + bytes_f + 255) / 256 * 256;
@@ -829,13 +841,20 @@ int build_tables(st_handle *h) {
   const size_t o_cdf = (o_sop + sop.size() * sizeof(unsigned short) + 255) / 256 * 256;
   // fp16 S_my / S_mz images for the tensor-core y- and z-DSTs (mixed precision, supported lengths)
   std::vector<unsigned short> sopy, sopz, sopx;
+  const bool long_y = use_tc && tc_ly_ok(g), long_z = use_tc && tc_lz_ok(g);
   if (use_tc && tc_y_ok(g)) {
     sopy.resize(dst_tma_image_halves(g.my));
     dst_tma_build_image(g.my, sopy.data());
+  } else if (long_y) {
+    sopy.resize(dst_long_image_halves(g.my));
+    dst_long_build_image(g.my, sopy.data());
   }
   if (use_tc && tc_z_ok(g)) {
     sopz.resize(dst_tma_image_halves(g.mz));
     dst_tma_build_image(g.mz, sopz.data());
+  } else if (long_z) {
+    sopz.resize(dst_long_image_halves(g.mz));
+    dst_long_build_image(g.mz, sopz.data());
   }
   // and S_mx for the tensor-core x-DST of the last spatial pass
   if (use_tc && tc_x_ok(g)) {
@@ -947,6 +966,11 @@ int build_tables(st_handle *h) {
                           : reinterpret_cast<const unsigned short *>((const char *)h->tables + o_sopy);
   pp.sop_z = sopz.empty() ? nullptr
                           : reinterpret_cast<const unsigned short *>((const char *)h->tables + o_sopz);
+  // a long axis' image serves its own kernels
+  pp.sop_ly = long_y ? pp.sop_y : nullptr;
+  pp.sop_lz = long_z ? pp.sop_z : nullptr;
+  if (long_y) pp.sop_y = nullptr;
+  if (long_z) pp.sop_z = nullptr;
   h->tc_time_img = pp.sop;
   h->tc_y_img = pp.sop_y;
   h->tc_z_img = pp.sop_z;
@@ -1358,6 +1382,7 @@ int st::setup_handle(const st_problem *prob, st_handle **out, int ugroup) {
   h->zscratch = (float *)h->Z[0];
   if (e == cudaSuccess) e = cudaMalloc(&h->q, Nv * sizeof(double));
   h->pp.tscratch = reinterpret_cast<dd *>(h->q);  // free during a preconditioner pass
+  h->pp.fscratch = reinterpret_cast<float *>(h->q);
   if (e == cudaSuccess && h->mixed) e = cudaMalloc(&h->Xdf, Nv * sizeof(df));
   h->partials_len = partials_needed(g);
   if (e == cudaSuccess) e = cudaMalloc(&h->partials, (size_t)h->partials_len * sizeof(double));

@@ -860,6 +860,28 @@ cudaError_t dst_z_pass(Src src, Tc *out, const Geom &g, const PrecPlan &pp, Stat
                                         pp.dst_shift, st);
 }
 
+// A y (axis 1) or z (axis 2) pass on *cur: in place, or for a long axis on the tensor cores from *cur to
+// *oth, which then trade places (a preconditioner pass transforms every axis twice, so the data ends
+// where it began).
+template <class Tc>
+cudaError_t yz_pass(int axis, Tc *&cur, Tc *&oth, const Geom &g, const PrecPlan &pp, State *S, int gk,
+                    cudaStream_t st) {
+  using Arr = SrcArray<Tc, Tc>;
+  if constexpr (sizeof(Tc) == sizeof(float)) {
+    const unsigned short *img = axis == 1 ? pp.sop_ly : pp.sop_lz;
+    if (img != nullptr) {
+      const cudaError_t e = axis == 1 ? launch_dst_long_y(cur, oth, g, img, S, gk, st)
+                                      : launch_dst_long_z(cur, oth, g, img, S, gk, st);
+      Tc *t = cur;
+      cur = oth;
+      oth = t;
+      return e;
+    }
+  }
+  return axis == 1 ? dst_y_pass<Tc>(Arr{cur}, cur, g, pp, S, gk, st)
+                   : dst_z_pass<Tc>(Arr{cur}, cur, g, pp, S, gk, st);
+}
+
 // The time DST alone (the P_theta paths with varying a): tensor cores in float32 when the plan has
 // the S_n image, else the FFMA/DFMA kernel.
 // in -> out (the same array, or one that does not overlap).
@@ -891,10 +913,11 @@ cudaError_t cheb_stages(const Geom &g, const PrecPlan &pp, Src src, Tc *zc, Stat
   const long long nx = (long long)g.n * g.my * g.mz;
   const Tc *twx = tw_of<Tc>(pp, true);
   cudaError_t e;
-  // the y (and z) passes of one half of the spatial transform, in place
-  auto yz_pass = [&](Tc *a) -> cudaError_t {
-    cudaError_t r = dst_y_pass<Tc>(Arr{a}, a, g, pp, S, gk, st);
-    if (r == cudaSuccess && g.dim == 3) r = dst_z_pass<Tc>(Arr{a}, a, g, pp, S, gk, st);
+  // the y (and z) passes of one half of the spatial transform; wc: where the data is
+  Tc *wc = W, *wo = reinterpret_cast<Tc *>(pp.fscratch);
+  auto yz = [&]() -> cudaError_t {
+    cudaError_t r = yz_pass<Tc>(1, wc, wo, g, pp, S, gk, st);
+    if (r == cudaSuccess && g.dim == 3) r = yz_pass<Tc>(2, wc, wo, g, pp, S, gk, st);
     return r;
   };
   prof_begin(KC_AUX, st);
@@ -908,16 +931,16 @@ cudaError_t cheb_stages(const Geom &g, const PrecPlan &pp, Src src, Tc *zc, Stat
   for (int j = 0; j < pp.cheb; ++j) {
     // the axes commute: x, y (z), then x with the scaling fused into its loads, then y (z); the
     // y and z passes take the tensor cores in float32 when the plan has the S_my / S_mz image
-    e = launch_dst<Tc, Arr, Tc, true>(Arr{j == 0 ? zc : R}, W, g.mx, pp.Lx, nx, g.mx, 0, 0, y.px,
+    e = launch_dst<Tc, Arr, Tc, true>(Arr{j == 0 ? zc : R}, wc, g.mx, pp.Lx, nx, g.mx, 0, 0, y.px,
                                       y.px, twx, S, gk, pp.dst_shift, st);
     if (e != cudaSuccess) return e;
-    if ((e = yz_pass(W)) != cudaSuccess) return e;
-    const SrcChebScale<Tc> sc{W, scoef + (size_t)j * g.n, sp.lh, sp.lht, sp.mux, sp.muy,
+    if ((e = yz()) != cudaSuccess) return e;
+    const SrcChebScale<Tc> sc{wc, scoef + (size_t)j * g.n, sp.lh, sp.lht, sp.mux, sp.muy,
                               (unsigned)y.mp, (unsigned)y.px};
-    e = launch_dst<Tc, SrcChebScale<Tc>, Tc, true>(sc, W, g.mx, pp.Lx, nx, g.mx, 0, 0, y.px, y.px,
+    e = launch_dst<Tc, SrcChebScale<Tc>, Tc, true>(sc, wc, g.mx, pp.Lx, nx, g.mx, 0, 0, y.px, y.px,
                                                    twx, S, gk, pp.dst_shift, st);
     if (e != cudaSuccess) return e;
-    if ((e = yz_pass(W)) != cudaSuccess) return e;
+    if ((e = yz()) != cudaSuccess) return e;  // back in W
     const Tc *aj = acoef + (size_t)j * g.n;
     if (j + 1 < pp.cheb) {
       const dim3 rb(kChebBX, kChebBY);
@@ -1037,21 +1060,23 @@ cudaError_t prec_stages(const Geom &g, const PrecPlan &pp, Src src, Tout *z, Sta
                                       lay<Tc>(g).px, tw_of<Tc>(pp, true), S, gk, pp.dst_shift,
                                       st);
   if (e != cudaSuccess) return e;
-  if (g.dim >= 2 && (e = dst_y_pass<Tc>(Inner{z}, zt, g, pp, S, gk, st)) != cudaSuccess) return e;
-  if (g.dim == 3 && (e = dst_z_pass<Tc>(Inner{z}, zt, g, pp, S, gk, st)) != cudaSuccess) return e;
+  // cur: where the data is (z, or the scratch vector between the two passes of a long axis)
+  Tc *cur = zt, *oth = reinterpret_cast<Tc *>(pp.fscratch);
+  if (g.dim >= 2 && (e = yz_pass<Tc>(1, cur, oth, g, pp, S, gk, st)) != cudaSuccess) return e;
+  if (g.dim == 3 && (e = yz_pass<Tc>(2, cur, oth, g, pp, S, gk, st)) != cudaSuccess) return e;
   if (sizeof(Tc) == sizeof(float) && pp.sop != nullptr)
-    e = launch_time_tma(reinterpret_cast<float *>(z), g, pp.spec_f, pp.sop, S, tmode, partials, gk,
+    e = launch_time_tma(reinterpret_cast<float *>(cur), g, pp.spec_f, pp.sop, S, tmode, partials, gk,
                         st);
   else if (sizeof(Tc) == sizeof(float) && pp.sop_long != nullptr)
-    e = launch_time_tc_long(reinterpret_cast<float *>(z), g, pp.spec_f, pp.sop_long, S, tmode,
-                            partials, gk, st);
+    e = launch_time_long(reinterpret_cast<float *>(cur), reinterpret_cast<float *>(oth), g, pp.spec_f,
+                         pp.sop_long, S, tmode, partials, gk, st);
   else
-    e = launch_time<Tc>(reinterpret_cast<Tc *>(z), g, spec_of<Tc>(pp), S, tmode, 0, partials, gk,
+    e = launch_time<Tc>(cur, g, spec_of<Tc>(pp), S, tmode, 0, partials, gk,
                         sizeof(Tc) == sizeof(float) ? pp.time_J_f : pp.time_J_d, st);
   if (e != cudaSuccess) return e;
   if (after_time && (e = cudaEventRecord(after_time, st)) != cudaSuccess) return e;
-  if (g.dim == 3 && (e = dst_z_pass<Tc>(Inner{z}, zt, g, pp, S, gk, st)) != cudaSuccess) return e;
-  if (g.dim >= 2 && (e = dst_y_pass<Tc>(Inner{z}, zt, g, pp, S, gk, st)) != cudaSuccess) return e;
+  if (g.dim == 3 && (e = yz_pass<Tc>(2, cur, oth, g, pp, S, gk, st)) != cudaSuccess) return e;
+  if (g.dim >= 2 && (e = yz_pass<Tc>(1, cur, oth, g, pp, S, gk, st)) != cudaSuccess) return e;
   // a caller's contiguous output: the last pass leaves the padding out
   if (user) {
     if (sizeof(Tc) == sizeof(float) && pp.sop_x != nullptr)

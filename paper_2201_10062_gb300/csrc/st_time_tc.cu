@@ -1,19 +1,18 @@
-// Time-axis DST-I on the 5th-generation tensor cores (tcgen05) for the axes that k_time_tma
-// (st_dst_tma.cu) does not take: float32-accurate for 256 < n <= 512 with S_n streamed from global
-// memory (k_time_tc_long), and, at the end of this file, float64-accurate with integer digits for
+// Float64-accurate time-axis DST-I on the 5th-generation tensor cores (tcgen05) with integer digits, for
 // the float64 path (k_time_tcd).
 //
 // The folded transform is two dense products per parity of the output index k:
 //   odd  k = 2r+1:  Y_k = sum_{t=1..h} S_{k,t} (x_t + x_{n+1-t})
-//   even k = 2r+2:  Y_k = sum_{t=1..h} S_{k,t} (x_t - x_{n+1-t}),     h = n/2,
-// i.e. D_P[r][j] = sum_t A_P[r][t] B_P[t][j] with A_P (h x h) fixed and B_P the folded data of a
-// tile of 32 spatial columns.  Every wait on an mbarrier is bounded; on timeout the block records
-// ST_ERR_TIMEOUT in the MINRES state and stops.  Before it releases its tensor memory it gives every
-// MMA batch whose commit it has not seen complete one more bounded wait: MMAs still in flight may
-// be writing that memory.  If that wait runs out as well, the block keeps it (it must not be given to
+//   even k = 2r+2:  Y_k = sum_{t=1..h} S_{k,t} (x_t - x_{n+1-t}),     h = ceil(n/2),
+// i.e. D_P[r][j] = sum_t A_P[r][t] B_P[t][j] with A_P fixed and B_P the folded data of a tile of 32
+// spatial columns.  Every wait on an mbarrier is bounded; on timeout the block records
+// ST_ERR_TIMEOUT in the MINRES state and stops.  Before it releases its tensor memory it gives every MMA
+// batch whose commit it has not seen complete one more bounded wait: MMAs still in flight may be
+// writing that memory.  If that wait runs out as well, the block keeps it (it must not be given to
 // another block while an MMA may write it) and sets State::tmem_held, which closes the device to
 // further calls on the host side.
 #include <cmath>
+#include <vector>
 #include <cstdlib>
 
 #include "st_tc.cuh"
@@ -21,331 +20,7 @@
 namespace st {
 namespace {
 
-constexpr int kNT = 512;         // 16 warps
 constexpr int kYS = kTN + 1;  // padded row of the parity-split Y tile (conflict-free row writes)
-
-// ------------------------------------------------------------------ long time axes (n > 256)
-// For 256 < n <= 512 the S_n operand (both parities, two 128-row M tiles each, K padded to 256,
-// hi and lo: 512 KB) does not fit in shared memory.  It is laid out in global memory as 16
-// chunks of 32 KB, chunk q = (P*2 + mt)*4 + kc holding rows mt*128.. of parity P and K range
-// kc*64.., each piece canonical K-major with K = 64, and one thread streams the chunks through a
-// two-slot ring with cp.async.bulk (mbarrier transaction counts), one chunk ahead of the MMAs.
-// The B operand holds both parities for K = 256 (zero beyond h); the four accumulators
-// (parity x M tile, 32 columns each) take 128 tensor-memory columns.
-constexpr int kKP2 = 256;                 // padded K of the long kernel
-constexpr uint32_t kChunk2 = 32768u;      // bytes per streamed A chunk (2 pieces x 128 x 64 fp16)
-constexpr uint32_t kPiece2 = kChunk2 / 2; // one piece of a chunk
-
-struct Tc2Smem {
-  uint32_t ring, bop, ytile, colscale, colinv1, colinv2, colmax, tmu, mbar, tmem, total;
-};
-
-__host__ __device__ inline Tc2Smem tc2_layout(int n) {
-  const int h = n / 2;
-  Tc2Smem L{};
-  uint32_t o = 0;
-  L.ring = o;
-  o += 2u * kChunk2;
-  L.bop = o;
-  o += 2u * 2u * kTN * kKP2 * 2u;  // [parity][piece][32][256] fp16
-  L.ytile = o;
-  o += 2u * h * kYS * 4u;
-  L.colscale = o;
-  o += kTN * 4u;
-  L.colinv1 = o;
-  o += kTN * 4u;
-  L.colinv2 = o;
-  o += kTN * 4u;
-  L.colmax = o;
-  o += kTN * 4u;
-  L.tmu = o;
-  o += kTN * 4u;
-  L.mbar = o;  // full[2], empty[2], done
-  o += 5 * 8;
-  L.tmem = o;
-  o += 8;
-  L.total = o;
-  return L;
-}
-
-// Fold, scale and split for K = 256 (h <= 256 folded rows): thread (column c, group g) handles
-// the t-blocks g and g + 16 of 8 rows each.  Same arithmetic as build_b.
-template <class Src>
-__device__ __forceinline__ void build_b_long(unsigned char *smem, const Tc2Smem &L,
-                                             uint32_t colinv_off, int n, Src src, int tid) {
-  const int h = n >> 1, hb = h >> 3;
-  unsigned int *colmax = reinterpret_cast<unsigned int *>(smem + L.colmax);
-  float *colscale = reinterpret_cast<float *>(smem + L.colscale);
-  float *colinv = reinterpret_cast<float *>(smem + colinv_off);
-  const int c = tid & (kTN - 1), g = tid >> 5;
-  if (tid < kTN) colmax[tid] = 0u;
-  float u[2][8], d[2][8];
-  float mx = 0.f;
-#pragma unroll
-  for (int it = 0; it < 2; ++it) {
-    const int tb = g + 16 * it;
-    if (tb < hb) {
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int t = tb * 8 + q;
-        const float a = src(t, c), b = src(n - 1 - t, c);
-        u[it][q] = a + b;
-        d[it][q] = a - b;
-        mx = fmaxf(mx, fmaxf(fabsf(u[it][q]), fabsf(d[it][q])));
-      }
-    }
-  }
-  __syncthreads();
-  atomicMax(&colmax[c], __float_as_uint(mx));
-  __syncthreads();
-  if (tid < kTN) {
-    const float m = __uint_as_float(colmax[tid]);
-    float s = 1.0f;
-    if (m > 0.f && isfinite(m)) {
-      int e;
-      frexpf(m, &e);
-      s = ldexpf(1.0f, 14 - e);
-    }
-    colscale[tid] = s;
-    colinv[tid] = 1.0f / (s * kSScale);
-  }
-  __syncthreads();
-  const float s = colscale[c];
-  unsigned char *bop = smem + L.bop;
-  const uint32_t piece = (uint32_t)kTN * kKP2 * 2u;
-#pragma unroll
-  for (int it = 0; it < 2; ++it) {
-    const int tb = g + 16 * it;
-    if (tb < hb) {
-      uint32_t uh[4], ul[4], dh[4], dl[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        split_h2(u[it][2 * q] * s, u[it][2 * q + 1] * s, uh[q], ul[q]);
-        split_h2(d[it][2 * q] * s, d[it][2 * q + 1] * s, dh[q], dl[q]);
-      }
-      const uint32_t off = canon_off(c, tb * 8, kKP2);
-      *reinterpret_cast<uint4 *>(bop + 0 * piece + off) = make_uint4(uh[0], uh[1], uh[2], uh[3]);
-      *reinterpret_cast<uint4 *>(bop + 1 * piece + off) = make_uint4(ul[0], ul[1], ul[2], ul[3]);
-      *reinterpret_cast<uint4 *>(bop + 2 * piece + off) = make_uint4(dh[0], dh[1], dh[2], dh[3]);
-      *reinterpret_cast<uint4 *>(bop + 3 * piece + off) = make_uint4(dl[0], dl[1], dl[2], dl[3]);
-    }
-  }
-}
-
-// Issued by one thread: one transform (16 streamed A chunks x 4 K steps x 3 products into the
-// four accumulators), then a commit to `done`, which tracks every MMA issued before it.  The ring
-// phases persist across calls.  Returns false if a wait ran out (the caller records the
-// timeout); *fills_drained is false if, after such a timeout, a bulk copy into the ring could
-// still be in flight.
-__device__ __forceinline__ bool stream_mmas(unsigned char *smem, const Tc2Smem &L,
-                                            const unsigned char *A_g, uint32_t tmem,
-                                            uint32_t *fph, uint32_t *eph, bool *fills_drained) {
-  const uint32_t full0 = smem_u32(smem + L.mbar), empty0 = full0 + 16, done = full0 + 32;
-  const uint32_t ring = smem_u32(smem + L.ring), bbase = smem_u32(smem + L.bop);
-  const uint32_t bpiece = (uint32_t)kTN * kKP2 * 2u;
-  auto fill = [&](int q, int slot) {
-    mbar_expect_tx(full0 + 8u * slot, kChunk2);
-    bulk_g2s(ring + (uint32_t)slot * kChunk2, A_g + (size_t)q * kChunk2, kChunk2,
-             full0 + 8u * slot);
-  };
-  bool ok = true;
-  int pending[2] = {0, 0};  // fills not yet waited for, per slot
-  fill(0, 0);
-  fill(1, 1);
-  pending[0] = pending[1] = 1;
-  for (int q = 0; q < 16; ++q) {
-    const int slot = q & 1;
-    if (!mbar_wait(full0 + 8u * slot, fph[slot])) {
-      ok = false;
-      break;
-    }
-    fph[slot] ^= 1u;
-    --pending[slot];
-    const int P = q >> 3, mt = (q >> 2) & 1, kc = q & 3;
-    const uint32_t d = tmem + (uint32_t)((P * 2 + mt) * kTN);
-    const uint32_t a_hi = ring + (uint32_t)slot * kChunk2, a_lo = a_hi + kPiece2;
-    const uint32_t b_hi = bbase + (2 * P) * bpiece, b_lo = b_hi + bpiece;
-#pragma unroll
-    for (int ks = 0; ks < 4; ++ks) {
-      const uint32_t aoff = (uint32_t)ks * 256u, boff = (uint32_t)(kc * 4 + ks) * 256u;
-      mma_f16(d, make_desc(a_hi + aoff, 64), make_desc(b_hi + boff, kKP2),
-              (kc > 0 || ks > 0) ? 1u : 0u);
-      mma_f16(d, make_desc(a_hi + aoff, 64), make_desc(b_lo + boff, kKP2), 1u);
-      mma_f16(d, make_desc(a_lo + aoff, 64), make_desc(b_hi + boff, kKP2), 1u);
-    }
-    mma_commit(empty0 + 8u * slot);
-    // chunk q-1 (other slot) is read by MMAs issued before; once they are done, load chunk q+1
-    if (q >= 1 && q + 1 < 16) {
-      const int other = slot ^ 1;
-      if (!mbar_wait(empty0 + 8u * other, eph[other])) {
-        ok = false;
-        break;
-      }
-      eph[other] ^= 1u;
-      fill(q + 1, other);
-      ++pending[other];
-    }
-  }
-  if (ok) {
-    // the commits of the last two chunks (slots 0 and 1) complete one more phase of each empty
-    // barrier: consume them so that the phases stay in step for the next transform
-    for (int sl = 0; sl < 2 && ok; ++sl) {
-      if (!mbar_wait(empty0 + 8u * sl, eph[sl])) ok = false;
-      eph[sl] ^= 1u;
-    }
-  } else {
-    // after a timeout: wait (bounded) for copies still in flight before the block moves on
-    for (int sl = 0; sl < 2; ++sl)
-      if (pending[sl] > 0 && !mbar_wait(full0 + 8u * sl, fph[sl])) *fills_drained = false;
-  }
-  mma_commit(done);
-  return ok;
-}
-
-__global__ void __launch_bounds__(kNT, 1)
-    k_time_tc_long(float *data, int n, long long m, int mx, int px, Spec<float> sp,
-                   const unsigned char *A_g, State *S, int tmode, double *__restrict__ partials,
-                   int gk) {
-  __shared__ double red[32];
-  if (gate_closed(S, gk)) return;
-  extern __shared__ __align__(1024) unsigned char smem[];
-  const int h = n >> 1;
-  const Tc2Smem L = tc2_layout(n);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + L.tmem);
-  const float *colinv1 = reinterpret_cast<const float *>(smem + L.colinv1);
-  const float *colinv2 = reinterpret_cast<const float *>(smem + L.colinv2);
-  float *ytile = reinterpret_cast<float *>(smem + L.ytile);
-  float *tmus = reinterpret_cast<float *>(smem + L.tmu);
-  const uint32_t full0 = smem_u32(smem + L.mbar), done = full0 + 32;
-  const long long ntiles = (m + kTN - 1) / kTN;
-  {  // B rows t >= h stay zero for the whole launch
-    uint4 *b = reinterpret_cast<uint4 *>(smem + L.bop);
-    const int cnt = (int)((2u * 2u * kTN * kKP2 * 2u) / 16u);
-    for (int i = tid; i < cnt; i += kNT) b[i] = make_uint4(0u, 0u, 0u, 0u);
-  }
-  if (tid == 0) {
-    for (int i = 0; i < 5; ++i)
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full0 + 8u * i) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 128;" ::"r"(
-                     smem_u32(tmem_slot))
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  fence_before();
-  __syncthreads();
-  fence_after();
-  const uint32_t tmem = *tmem_slot;
-  uint32_t fph[2] = {0u, 0u}, eph[2] = {0u, 0u}, dph = 0u;  // phases (used by thread 0)
-  bool ok = true;
-  bool out_done = false;      // a commit to `done` whose completion has not been seen
-  bool fills_drained = true;  // thread 0: no bulk copy into the ring left in flight
-  float esum = 0.f, ecomp = 0.f;
-  // accumulator view: TMEM lanes 32q.. (rows r = mt*128 + 32q + lane), parity P, columns 16ch..
-  const int qq = warp & 3, P = (warp >> 2) & 1, ch = warp >> 3;
-  const int c0 = ch * 16;
-  const uint32_t lanes = (uint32_t)(qq * 32) << 16;
-  SymRow sr[2];
-#pragma unroll
-  for (int mt = 0; mt < 2; ++mt) {
-    const int r = mt * 128 + (qq << 5) + lane;
-    sr[mt] = sym_row(sp, r < h ? (P == 0 ? 2 * r + 1 : 2 * r + 2) : 1);
-  }
-  auto ycell = [&](int t, int c) -> float { return ytile[((t & 1) * h + (t >> 1)) * kYS + c]; };
-  auto run_mmas = [&]() {
-    fence_async_smem();
-    __syncthreads();
-    fence_after();
-    bool w = true;
-    if (tid == 0) w = stream_mmas(smem, L, A_g, tmem, fph, eph, &fills_drained);
-    const bool d = __syncthreads_and(mbar_wait(done, dph) ? 1 : 0) != 0;
-    if (d) {
-      dph ^= 1u;
-    } else {
-      out_done = true;
-    }
-    ok = (__syncthreads_and((w && d) ? 1 : 0) != 0) && ok;
-    fence_after();
-  };
-  for (long long tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-    const long long j0 = tile * kTN;
-    const int je = (int)min((long long)kTN, m - j0);
-    if (tid < kTN) tmus[tid] = tmu_col(sp, j0 + tid, mx, px, m);
-    build_b_long(smem, L, L.colinv1, n,
-                 [&](int t, int c) -> float {
-                   return (c < je) ? data[(long long)t * m + j0 + c] : 0.f;
-                 },
-                 tid);
-    run_mmas();
-    if (!ok) break;  // uniform
-    // unscale, spectral scaling, energy; Y into the parity-split tile
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt) {
-      float v[16];
-      tmem_ld16(tmem + lanes + (uint32_t)((P * 2 + mt) * kTN + c0), v);
-      const int r = mt * 128 + (qq << 5) + lane;
-      if (r < h) {
-        float *yrow = ytile + (P * h + r) * kYS;
-        float rs = 0.f;
-#pragma unroll
-        for (int c = 0; c < 16; ++c) {
-          const float y = v[c] * colinv1[c0 + c];
-          const float yi = y * inv_sym(sp, sr[mt], tmus[c0 + c]);
-          if (c0 + c < je) rs = fmaf(y, yi, rs);
-          yrow[c0 + c] = yi;
-        }
-        const float term = rs - ecomp;
-        const float t = esum + term;
-        ecomp = (t - esum) - term;
-        esum = t;
-      }
-    }
-    fence_before();
-    __syncthreads();
-    fence_after();
-    build_b_long(smem, L, L.colinv2, n, [&](int t, int c) -> float { return ycell(t, c); }, tid);
-    run_mmas();
-    if (!ok) break;  // uniform
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt) {
-      float v[16];
-      tmem_ld16(tmem + lanes + (uint32_t)((P * 2 + mt) * kTN + c0), v);
-      const int r = mt * 128 + (qq << 5) + lane;
-      if (r < h) {
-        float *yrow = ytile + (P * h + r) * kYS;
-#pragma unroll
-        for (int c = 0; c < 16; ++c) yrow[c0 + c] = v[c] * colinv2[c0 + c];
-      }
-    }
-    fence_before();
-    __syncthreads();
-    fence_after();
-    for (int idx = tid; idx < n * kTN; idx += kNT) {
-      const int t = idx >> 5, c = idx & (kTN - 1);
-      if (c < je) data[(long long)t * m + j0 + c] = ycell(t, c);
-    }
-    __syncthreads();
-  }
-  // a bulk copy that may still land in the ring keeps the block from handing its resources back
-  // as well: it counts as an outstanding completion
-  const bool fills_ok = __syncthreads_and(fills_drained ? 1 : 0) != 0;
-  tc_release_cols<128>(ok, out_done, done, dph, false, 0u, 0u, tmem, S, fills_ok);
-  if (tmode != TM_NONE) {
-    const double e = (double)esum - (double)ecomp;
-    double tot;
-    if (last_block_reduce<kNT>(e, partials, &S->counter[CNT_TIME], gridDim.x, blockIdx.x, red,
-                               &tot) &&
-        tid == 0) {
-      if (tmode == TM_INIT || tmode == TM_RESTART)
-        minres_init_scalars_dev(S, tot);
-      else
-        minres_givens_dev(S, tot);
-    }
-  }
-}
 
 }  // namespace
 
@@ -360,63 +35,6 @@ int time_tc_grid() {
   return sms;
 }
 
-// ------------------------------------------------------------------ long time axes: host side
-bool time_tc_long_supported(int n) {
-  return n > 256 && n <= 512 && (n % 32) == 0 && tc2_layout(n).total + 1024u <= 227u * 1024u;
-}
-
-size_t time_tc_long_bytes(int) { return (size_t)16 * kChunk2; }
-
-// Host: the 16 streamed chunks of 8 S_n (rows of parity P, M tile mt, K range kc*64..), hi and
-// lo pieces, each canonical K-major with K = 64.  Rows beyond h or with k > n, and columns
-// t >= h, are zero.
-void time_tc_long_build(int n, unsigned short *out) {
-  const int h = n / 2;
-  const double PI = 3.14159265358979323846;
-  const double sn = std::sqrt(2.0 / (n + 1));
-  const size_t halves = kChunk2 / 2, piece = kPiece2 / 2;
-  for (size_t i = 0; i < 16 * halves; ++i) out[i] = 0;
-  for (int P = 0; P < 2; ++P)
-    for (int mt = 0; mt < 2; ++mt)
-      for (int kc = 0; kc < 4; ++kc) {
-        unsigned short *chunk = out + (size_t)((P * 2 + mt) * 4 + kc) * halves;
-        for (int rr = 0; rr < kM; ++rr) {
-          const int r = mt * kM + rr;
-          const int k = (P == 0) ? 2 * r + 1 : 2 * r + 2;
-          if (r >= h || k > n) continue;
-          for (int kk = 0; kk < 64; ++kk) {
-            const int t = kc * 64 + kk;
-            if (t >= h) continue;
-            const double v = kSScale * sn * std::sin(PI * (double)k * (t + 1) / (n + 1));
-            const __half hi = __float2half_rn((float)v);
-            const __half lo = __float2half_rn((float)(v - (double)__half2float(hi)));
-            const uint32_t off = canon_off(rr, kk, 64) / 2;
-            __half_raw rh = hi, rl = lo;
-            chunk[off] = rh.x;
-            chunk[piece + off] = rl.x;
-          }
-        }
-      }
-}
-
-cudaError_t launch_time_tc_long(float *data, const Geom &g, const Spec<float> &sp,
-                                const unsigned short *A, State *S, int tmode, double *partials,
-                                int gk, cudaStream_t st) {
-  const uint32_t smem_bytes = tc2_layout(g.n).total;
-  cudaError_t e = cudaFuncSetAttribute(k_time_tc_long,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem_bytes);
-  if (e != cudaSuccess) return e;
-  const long long ntiles = (g.mp + kTN - 1) / kTN;
-  int grid = time_tc_grid();
-  if (ntiles < grid) grid = (int)ntiles;
-  prof_begin(KC_TIME, st);
-  k_time_tc_long<<<grid, kNT, smem_bytes, st>>>(data, g.n, g.mp, g.mx, g.px, sp,
-                                                reinterpret_cast<const unsigned char *>(A), S,
-                                                tmode, partials, gk);
-  prof_end(st);
-  return cudaGetLastError();
-}
 // ------------------------------------------------------------------ float64-accurate time DST
 // The time stage of the float64 preconditioner (Sec. 3.1.1, steps 1-3 along time) on the tensor
 // cores, for double-float data.  An fp16 MMA with float32 accumulation is exact on integers as
@@ -886,13 +504,27 @@ int time_tcd_build(int n, unsigned char *out) {
   const int h = (n + 1) / 2, hK = tcd_hk(n);
   const double PI = 3.14159265358979323846;
   const double sn = std::sqrt(2.0 / (n + 1));
+  // S_{k,t} = sn sin(pi a / (n+1)) with a = k t mod 2 (n+1): the digits of these 2 (n+1) values.  The
+  // largest entry over k <= n, t <= h is taken from them as well.
+  const int period = 2 * (n + 1);
+  std::vector<double> val(period);
+  for (int a = 0; a < period; ++a) val[a] = sn * std::sin(PI * (double)a / (n + 1));
   double smax = 0.0;
   for (int k = 1; k <= n; ++k)
-    for (int t = 1; t <= h; ++t)
-      smax = std::fmax(smax, std::fabs(sn * std::sin(PI * (double)k * t / (n + 1))));
+    for (int t = 1, a = k; t <= h; ++t, a = (a + k) % period) smax = std::fmax(smax, std::fabs(val[a]));
   int E = 0;
   std::frexp(smax, &E);
   const int eS = 7 - E;  // smax 2^eS in [2^6, 2^7)
+  std::vector<unsigned short> dig((size_t)period * kDg);
+  for (int a = 0; a < period; ++a) {
+    double v = std::ldexp(val[a], eS);
+    for (int dg = 0; dg < kDg; ++dg) {
+      const double q = std::nearbyint(v);
+      v = (v - q) * 128.0;
+      const __half_raw raw = __float2half_rn((float)q);
+      dig[(size_t)a * kDg + dg] = raw.x;
+    }
+  }
   unsigned short *o = reinterpret_cast<unsigned short *>(out);
   const size_t piece = (size_t)kM * hK;  // halves
   for (size_t i = 0; i < time_tcd_bytes(n) / 2; ++i) o[i] = 0;
@@ -900,15 +532,13 @@ int time_tcd_build(int n, unsigned char *out) {
     for (int r = 0; r < h; ++r) {
       const int k = (P == 0) ? 2 * r + 1 : 2 * r + 2;
       if (k > n) continue;
+      int a = 0;
       for (int t = 0; t < h; ++t) {
-        double v = std::ldexp(sn * std::sin(PI * (double)k * (t + 1) / (n + 1)), eS);
-        for (int dg = 0; dg < kDg; ++dg) {
-          const double q = std::nearbyint(v);
-          v = (v - q) * 128.0;
-          const __half hq = __float2half_rn((float)q);
-          __half_raw raw = hq;
-          o[(size_t)(P * kDg + dg) * piece + canon_off(r, t, hK) / 2] = raw.x;
-        }
+        a += k;
+        if (a >= period) a -= period;
+        const size_t off = canon_off(r, t, hK) / 2;
+        for (int dg = 0; dg < kDg; ++dg)
+          o[(size_t)(P * kDg + dg) * piece + off] = dig[(size_t)a * kDg + dg];
       }
     }
   return eS;
