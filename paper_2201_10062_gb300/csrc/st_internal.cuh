@@ -22,7 +22,6 @@ struct Geom {
   const double *cy;     // [mz][my+1][mx] tau * a(y-face) / hy^2 (NULL in 1D)
   const df *cxd, *cyd;  // the same coefficients as double-float pairs (mixed-precision stencil)
   df th_d, omth_d;      // theta and 1 - theta as double-float pairs
-  int th_exact;         // theta in {0, 1/2, 1}: products with theta, 1 - theta are exact scalings
   int st_target;        // stencil launch: target number of blocks (0: default), set by autotune
   int mz;               // interior points along z: 1 unless 3D
   const double *cz;     // [mz+1][my][mx] tau * a(z-face) / hz^2 (NULL unless 3D)
@@ -161,7 +160,7 @@ __device__ inline double warp_sum(double v) {
 template <int NT>
 __device__ inline double block_sum(double v, double *red) {
   v = warp_sum(v);
-  const int lane = threadIdx.x & 31, wid = (threadIdx.x + threadIdx.y * blockDim.x) >> 5;
+  const int tid = threadIdx.x + threadIdx.y * blockDim.x, lane = tid & 31, wid = tid >> 5;
   __syncthreads();
   if (lane == 0) red[wid] = v;
   __syncthreads();

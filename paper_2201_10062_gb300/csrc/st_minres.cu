@@ -922,7 +922,6 @@ int build_tables(st_handle *h) {
   }
   h->g.th_d = df_of_double(h->g.theta);
   h->g.omth_d = df_of_double(1.0 - h->g.theta);
-  h->g.th_exact = (h->g.theta == 0.0 || h->g.theta == 0.5 || h->g.theta == 1.0) ? 1 : 0;
   PrecPlan &pp = h->pp;
   pp.pcr = (p.prec == ST_PREC_PTHETA && p.a_nodal != nullptr && g.dim == 1) ? 1 : 0;
   // every interval of zero width (a constant field): the steps after the first add exact zeros,
@@ -1533,7 +1532,7 @@ int st_autotune(st_handle *h, int reps) {
   cudaMemsetAsync(h->Z[0], 0, fp32 ? g.Np * sizeof(float) : g.N * sizeof(double), st);
   // 1. stencil: blocks per launch (time-chunk length)
   {
-    const int cand[] = {608, 1216, 2432, 4864};
+    const int cand[] = {0, 608, 1216, 2432, 4864};  // 0: the default rule
     State s{};
     s.active = 1;
     s.beta = 1.0;

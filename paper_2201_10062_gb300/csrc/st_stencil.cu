@@ -8,9 +8,11 @@
 // and Y only reverses the block order, so row k of T v is written to block n-1-k.
 // One thread owns one spatial node and walks a chunk of consecutive time levels (and their
 // mirror images), carrying neighbouring planes in registers so that each plane of v is read once.
+#include <algorithm>
 #include <type_traits>
 
 #include "st_internal.cuh"
+
 
 namespace st {
 
@@ -22,6 +24,7 @@ constexpr int kNT = 256;
 
 struct Tile {
   int kc, nchunk, gx, gy;
+  int bx;  // threads along x (double-float stencil)
 };
 
 Tile tile_for(const Geom &g) {
@@ -43,6 +46,45 @@ Tile tile_for(const Geom &g) {
   if (nchunk < 1) nchunk = 1;
   if (nchunk > half) nchunk = half;
   t.kc = (int)((half + nchunk - 1) / nchunk);
+  t.nchunk = (half + t.kc - 1) / t.kc;
+  return t;
+}
+
+// Weights of the double-float stencil: theta = 1/2, theta = 1, any other theta, BDF2
+enum StencilWeights { W_HALF, W_ONE, W_ANY, W_BDF2 };
+
+// Resident blocks of the double-float stencil on an SM.  A uniform coefficient leaves room for
+// three (80 registers; 63.6 -> 58.1 us at 255^2 x 256); with a coefficient per face, or 7 points,
+// three would spill (511^2 x 128, BDF2: 166 us with two, 182 with three).
+constexpr int df_blocks(int dim, bool uni) { return uni && dim < 3 ? 3 : 2; }
+
+// Double-float stencil: two x neighbours a thread, df_blocks blocks on each of 152 SMs.  Of the
+// chunk lengths the one with the least waves x (levels + 2) is taken: a chunk starts with two
+// extra planes, and a last wave that is nearly empty costs as much as a full one.
+Tile tile_df_for(const Geom &g) {
+  const int nb = df_blocks(g.dim, g.c_uniform);
+  Tile t;
+  t.bx = (g.dim == 1) ? kBX1 : std::min(kBX2, g.px / 2);
+  t.gx = (g.px / 2 + t.bx - 1) / t.bx;
+  t.gy = (g.my * g.mz + kNT / t.bx - 1) / (kNT / t.bx);
+  const int half = (g.n + 1) / 2;
+  const long long tiles = (long long)t.gx * t.gy;
+  if (g.st_target > 0) {
+    const long long nchunk = std::min<long long>(half, (g.st_target + tiles - 1) / tiles);
+    t.kc = (int)((half + nchunk - 1) / nchunk);
+  } else {
+    long long best = -1;
+    t.kc = half;
+    for (int kc = half; kc >= 1; --kc) {
+      const long long blocks = tiles * ((half + kc - 1) / kc);
+      if (blocks > 2432 && best >= 0) break;
+      const long long cost = ((blocks + 152 * nb - 1) / (152 * nb)) * (kc + 2);
+      if (best < 0 || cost < best) {
+        best = cost;
+        t.kc = kc;
+      }
+    }
+  }
   t.nchunk = (half + t.kc - 1) / t.kc;
   return t;
 }
@@ -242,56 +284,119 @@ __global__ void __launch_bounds__(kNT) k_stencil(Geom g, const Tz *__restrict__ 
 // added error-free, so the result carries ~46 significant bits with no float64 instruction per
 // element (GB300 runs float64 at 1/64 of the float32 rate).  Same mirrored-plane walk as the
 // float64 kernel; the dot <Y T z, z> is accumulated unscaled and scaled by 1/beta^2 at the end.
-struct acc_df {
-  float s, t;
-  __device__ __forceinline__ void add(float p, float e) {
-    float ss, err;
-    two_sum(s, p, ss, err);
-    s = ss;
-    t += err + e;
-  }
-  __device__ __forceinline__ void add(df a) { add(a.hi, a.lo); }
-  // add a float (no low-order part)
-  __device__ __forceinline__ void add1(float p) {
-    float ss, err;
-    two_sum(s, p, ss, err);
-    s = ss;
-    t += err;
-  }
-  __device__ __forceinline__ void add_prod(df a, df b) {
-    float p, e;
-    two_prod(a.hi, b.hi, p, e);
-    e = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, e));
-    add(p, e);
-  }
-  __device__ __forceinline__ void add_prod(df a, float b) {
-    float p, e;
-    two_prod(a.hi, b, p, e);
-    e = fmaf(a.lo, b, e);
-    add(p, e);
-  }
-  __device__ __forceinline__ df get() const { return df_from_sum(s, t); }
+// Two float32 values in one 64-bit register pair.  sm_100 and later issue add, sub, mul and fma on
+// such pairs as one instruction, each half rounded as the scalar instruction rounds it.
+struct f2 {
+  unsigned long long v;
 };
-
-__device__ __forceinline__ void face_term(acc_df &A, df c, float a, float b) {
-  float dh, dl;
-  two_sum(a, -b, dh, dl);
-  float p, e;
-  two_prod(c.hi, dh, p, e);
-  e = fmaf(c.hi, dl, fmaf(c.lo, dh, e));
-  A.add(p, e);
+__device__ __forceinline__ f2 pack2(float a, float b) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ f2 dup2(float a) { return pack2(a, a); }
+__device__ __forceinline__ void unpack2(f2 a, float &x, float &y) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a.v));
+}
+__device__ __forceinline__ f2 operator+(f2 a, f2 b) {
+  f2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ f2 operator-(f2 a, f2 b) {
+  f2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ f2 operator*(f2 a, f2 b) {
+  f2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+  f2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
 }
 
-// D3: the 3D grid (7-point stencil; planes mx*my apart), at three resident blocks per SM so that
-// its two extra planes stay in registers.  The 1D/2D instantiation carries no z terms.
+// Two double-float numbers, and a constant one with its high part negated besides: -(a b) is then
+// a product, and every difference below is a subtraction, so no sign is flipped on the way.
+struct df2 {
+  f2 hi, lo;
+};
+struct cf2 {
+  f2 hi, lo, nhi;
+};
+__device__ __forceinline__ cf2 cf2_of(df a, df b, float w = 1.f) {
+  return cf2{pack2(w * a.hi, w * b.hi), pack2(w * a.lo, w * b.lo), pack2(-w * a.hi, -w * b.hi)};
+}
+__device__ __forceinline__ df2 df2_from_sum(f2 s, f2 t) {
+  const f2 hi = s + t;
+  return df2{hi, t - (hi - s)};
+}
+
+// running double-float sums (see st_df.cuh), two at a time
+struct acc2 {
+  f2 s, t;
+  __device__ __forceinline__ f2 sum(f2 p) {  // s += p, returns the rounding error
+    const f2 ss = s + p, bb = ss - s;
+    const f2 err = (s - (ss - bb)) + (p - bb);
+    s = ss;
+    return err;
+  }
+  __device__ __forceinline__ f2 diff(f2 np) {  // s -= np, returns the rounding error
+    const f2 ss = s - np, bb = ss - s;
+    const f2 err = (s - (ss - bb)) - (np + bb);
+    s = ss;
+    return err;
+  }
+  __device__ __forceinline__ void add(df2 a) {
+    const f2 err = sum(a.hi);
+    t = t + (err + a.lo);
+  }
+  __device__ __forceinline__ void add1(f2 p) {
+    const f2 err = sum(p);
+    t = t + err;
+  }
+  __device__ __forceinline__ void sub1(f2 p) {
+    const f2 err = diff(p);
+    t = t + err;
+  }
+  // add c b
+  __device__ __forceinline__ void add_prod(cf2 c, df2 b) {
+    const f2 np = c.nhi * b.hi;
+    const f2 e = fma2(c.hi, b.lo, fma2(c.lo, b.hi, fma2(c.hi, b.hi, np)));
+    const f2 err = diff(np);
+    t = t + (err + e);
+  }
+  // add a b, nb = -b
+  __device__ __forceinline__ void add_prod(df2 a, f2 b, f2 nb) {
+    const f2 np = a.hi * nb;
+    const f2 e = fma2(a.lo, b, fma2(a.hi, b, np));
+    const f2 err = diff(np);
+    t = t + (err + e);
+  }
+  __device__ __forceinline__ df2 get() const { return df2_from_sum(s, t); }
+};
+
+// A thread owns two x neighbours (i even; the slot after a line's last node is its padding, whose
+// result is zero), and every double-float operation acts on both at once.
+// One node a thread with scalar instructions was bound by instruction issue: about 167 instructions
+// per unknown, 83% of the issue slots.  The pair takes 79 and shares the loads (8 bytes each but
+// for the two outer x neighbours), the addresses, which advance by a level instead of being formed
+// from k, and the loop; what bounds it now is latency (45% of the issue slots: waits for the loads
+// of the next level, the float32 pipe and dependent sums, ncu).  Before and now, us a launch:
+// 255^2 x 256 uniform, theta = 1/2: 86 and 58; 63^3 x 64 uniform: 105 and 73; 511^2 x 128 BDF2,
+// varying coefficient: 207 and 166; 255^2 x 128 varying, theta = 1: 60 and 49.
+// DIM 1, 2, 3: the 3-, 5- or 7-point stencil (planes px my apart in 3D).
 // UNI: every face coefficient has the same value c (a constant coefficient on a grid with equal
 // spacing along every axis, g.c_uniform): tau K z = c (f z_c - sum_f z_f) over the f faces of the
 // node, so the face terms reduce to one exactly summed difference (TwoSum chain over floats) and
 // one double-float product, in place of one product per face.
-template <bool D3, bool UNI>
-__global__ void __launch_bounds__(kNT, D3 ? 3 : 4) k_stencil_df(Geom g, const float *__restrict__ z,
-                                                    df *__restrict__ out, State *S,
-                                                    double *__restrict__ partials, int kc) {
+template <int DIM, bool UNI, int W>
+__global__ void __launch_bounds__(kNT, df_blocks(DIM, UNI)) k_stencil_df(Geom g, const float *__restrict__ z,
+                                                       df *__restrict__ out, State *S,
+                                                       double *__restrict__ partials, int kc) {
   __shared__ double red[32];
   if (!S->active) return;
   const bool lead = blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && flat_tid() == 0;
@@ -301,46 +406,61 @@ __global__ void __launch_bounds__(kNT, D3 ? 3 : 4) k_stencil_df(Geom g, const fl
   }
   // first iteration after a device-side restart: the restart pass is complete
   if (lead && S->restart) S->restart = 0;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  constexpr bool THETA = W != W_BDF2;
+  const int i = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   const int j = blockIdx.y * blockDim.y + threadIdx.y;  // row jz*my + jy
   // z and out are padded: px slots a line, m a level
-  const int mx = g.mx, my = g.my, dim = g.dim, n = g.n, px = g.px;
+  const int mx = g.mx, my = g.my, n = g.n, px = g.px;
   const long long m = g.mp, pl = (long long)px * my;
   const bool valid = (i < mx) && (j < my * g.mz);
   const int half = (n + 1) >> 1;
   const int k0 = blockIdx.z * kc;
   const int k1 = min(half, k0 + kc);
-  acc_df D{0.f, 0.f};
+  const f2 O = dup2(0.f), neg1 = dup2(-1.f);
+  acc2 D{O, O};
   if (valid) {
-    const int jz = D3 ? j / my : 0, jy = j - jz * my;
+    const int jz = DIM == 3 ? j / my : 0, jy = j - jz * my;
     const long long p = (long long)j * px + i;
-    const df zero_f{0.f, 0.f};
-    const Faces6<df> fc = UNI ? Faces6<df>{zero_f, zero_f, zero_f, zero_f, zero_f, zero_f}
-                              : faces_df_at(g, i, jy, jz);
-    const df cw = fc.w, ce = fc.e, cs = fc.s, cn = fc.n, cd = fc.d, cu = fc.u;
-    const df th = g.th_d, omth = g.omth_d;
-    const bool theta = (g.scheme == ST_THETA);
-    auto center = [&](int k) -> float { return __ldg(z + (long long)k * m + p); };
-    auto combine = [&](float c, float c1, float c2, df Kc, df K1) -> df {
-      acc_df A{0.f, 0.f};
-      if (theta) {
+    const bool two = i + 1 < mx;  // the second slot is a node
+    const bool hs = DIM >= 2 && jy > 0, hn = DIM >= 2 && jy < my - 1;
+    const bool hd = DIM == 3 && jz > 0, hu = DIM == 3 && jz < g.mz - 1;
+    cf2 cw, ce, cs, cn, cd, cu;
+    // theta = 1/2 scales the coefficients, an exact scaling
+    const float sc = W == W_HALF ? 0.5f : 1.f;
+    if (UNI) {
+      cw = cf2_of(g.c_uni, g.c_uni, sc);
+    } else {
+      const Faces6<df> a = faces_df_at(g, i, jy, jz), b = two ? faces_df_at(g, i + 1, jy, jz) : a;
+      cw = cf2_of(a.w, b.w, sc);
+      ce = cf2_of(a.e, b.e, sc);
+      cs = cf2_of(a.s, b.s, sc);
+      cn = cf2_of(a.n, b.n, sc);
+      cd = cf2_of(a.d, b.d, sc);
+      cu = cf2_of(a.u, b.u, sc);
+    }
+    const df2 zero{O, O};
+    auto center = [&](const float *b) -> f2 {
+      return f2{__ldg(reinterpret_cast<const unsigned long long *>(b))};
+    };
+    auto combine = [&](f2 c, f2 c1, f2 c2, df2 Kc, df2 K1) -> df2 {
+      acc2 A;
+      if (THETA) {
         // the exact difference c - c1 starts the sum
-        two_sum(c, -c1, A.s, A.t);
-        if (g.th_exact) {
-          // theta and 1 - theta are 0, 1/2 or 1: the products are exact scalings (the same
-          // values add_prod gives), and a zero weight adds nothing
-          A.add(th.hi * Kc.hi, th.hi * Kc.lo);
-          if (omth.hi != 0.f) A.add(omth.hi * K1.hi, omth.hi * K1.lo);
+        A.s = c;
+        A.t = A.diff(c1);
+        if (W == W_ANY) {
+          A.add_prod(cf2_of(g.th_d, g.th_d), Kc);
+          A.add_prod(cf2_of(g.omth_d, g.omth_d), K1);
         } else {
-          A.add_prod(th, Kc);
-          A.add_prod(omth, K1);
+          A.add(Kc);
+          if (W == W_HALF) A.add(K1);
         }
       } else {
-        float pp, e;
-        two_prod(1.5f, c, pp, e);
-        A.add(pp, e);
-        A.add1(-2.0f * c1);
-        A.add1(0.5f * c2);
+        const f2 h = dup2(1.5f), np = dup2(-1.5f) * c;
+        A.s = O - np;
+        A.t = fma2(h, c, np);
+        A.sub1(dup2(2.0f) * c1);
+        A.add1(dup2(0.5f) * c2);
         A.add(Kc);
       }
       return A.get();
@@ -348,135 +468,151 @@ __global__ void __launch_bounds__(kNT, D3 ? 3 : 4) k_stencil_df(Geom g, const fl
     // The loads of iteration kA + 1 (stencil points of both walks) are issued before the
     // arithmetic of iteration kA, so their latency overlaps it.
     struct P5 {
-      float c, w, e, s, n, d, u;
+      f2 c, s, n, d, u;
+      float w, e;  // west of the first node, east of the second
     };
-    auto load5 = [&](int k) -> P5 {
-      const float *b = z + (long long)k * m + p;
-      P5 r;
-      r.c = __ldg(b);
+    const P5 none{O, O, O, O, O, 0.f, 0.f};
+    auto load5 = [&](const float *b) -> P5 {
+      P5 r = none;
+      r.c = center(b);
       r.w = __ldg(b - 1);  // the padding slots on either side of a line hold the boundary's zeros
-      r.e = __ldg(b + 1);
-      r.s = (dim >= 2 && jy > 0) ? __ldg(b - px) : 0.f;
-      r.n = (dim >= 2 && jy < my - 1) ? __ldg(b + px) : 0.f;
-      r.d = (D3 && jz > 0) ? __ldg(b - pl) : 0.f;
-      r.u = (D3 && jz < g.mz - 1) ? __ldg(b + pl) : 0.f;
+      if (two) r.e = __ldg(b + 2);
+      if (hs) r.s = center(b - px);
+      if (hn) r.n = center(b + px);
+      if (hd) r.d = center(b - pl);
+      if (hu) r.u = center(b + pl);
       return r;
     };
+    auto face = [&](acc2 &A, cf2 a, f2 c, f2 q) {
+      const f2 dh = c - q, bb = dh - c;
+      const f2 dl = (c - (dh - bb)) - (q + bb);
+      A.add_prod(a, df2{dh, dl});
+    };
     // tau K at a plane: the face terms in a fixed order
-    auto stiff5 = [&](const P5 &q, float c) -> df {
+    auto stiff = [&](const P5 &q) -> df2 {
+      float c0, c1;
+      unpack2(q.c, c0, c1);
+      const f2 w = pack2(q.w, c0), e = pack2(c1, q.e);
       if (UNI) {
         // c_uni (f z_c - z_w - z_e - ...): f z_c is exact (f = 2, 4, or 4 + 2 in 3D)
-        acc_df A{(dim >= 2) ? 4.f * c : 2.f * c, 0.f};
-        if (D3) A.add1(2.f * c);
-        A.add1(-q.w);
-        A.add1(-q.e);
-        if (dim >= 2) {
-          A.add1(-q.s);
-          A.add1(-q.n);
+        acc2 A{dup2(DIM >= 2 ? 4.f : 2.f) * q.c, O};
+        if (DIM == 3) A.add1(dup2(2.f) * q.c);
+        A.sub1(w);
+        A.sub1(e);
+        if (DIM >= 2) {
+          A.sub1(q.s);
+          A.sub1(q.n);
         }
-        if (D3) {
-          A.add1(-q.d);
-          A.add1(-q.u);
+        if (DIM == 3) {
+          A.sub1(q.d);
+          A.sub1(q.u);
         }
-        return df_mul(g.c_uni, A.get());
+        const df2 x = A.get();
+        const f2 np = cw.nhi * x.hi;
+        const f2 r = fma2(cw.hi, x.lo, fma2(cw.lo, x.hi, fma2(cw.hi, x.hi, np)));
+        return df2{O - np, r};  // r is far below an ulp of the product: no normalisation
       }
-      acc_df A{0.f, 0.f};
-      face_term(A, cw, c, q.w);
-      face_term(A, ce, c, q.e);
-      if (dim >= 2) {
-        face_term(A, cs, c, q.s);
-        face_term(A, cn, c, q.n);
+      acc2 A{O, O};
+      face(A, cw, q.c, w);
+      face(A, ce, q.c, e);
+      if (DIM >= 2) {
+        face(A, cs, q.c, q.s);
+        face(A, cn, q.c, q.n);
       }
-      if (D3) {
-        face_term(A, cd, c, q.d);
-        face_term(A, cu, c, q.u);
+      if (DIM == 3) {
+        face(A, cd, q.c, q.d);
+        face(A, cu, q.c, q.u);
       }
       return A.get();
     };
-    auto stiff = [&](int k, float c) -> df { return stiff5(load5(k), c); };
-    const df zero{0.f, 0.f};
-    float a1 = 0.f, a2 = 0.f;
-    df aK1 = zero;
-    float b0 = 0.f, b1 = 0.f;
-    df bK0 = zero;
+    auto store = [&](df *o, df2 y) {
+      float h0, h1, l0, l1;
+      unpack2(y.hi, h0, h1);
+      unpack2(y.lo, l0, l1);
+      *reinterpret_cast<float4 *>(o) = make_float4(h0, l0, h1, l1);
+    };
+    // the padding slot's result is zero
+    auto masked = [&](df2 y) -> df2 {
+      float h0, h1, l0, l1;
+      unpack2(y.hi, h0, h1);
+      unpack2(y.lo, l0, l1);
+      return df2{pack2(h0, two ? h1 : 0.f), pack2(l0, two ? l1 : 0.f)};
+    };
+    f2 a1 = O, a2 = O, b0, b1 = O;
+    df2 aK1 = zero, bK0 = zero;
+    // planes kA = k0 (upwards) and kB = n - 1 - k0 (downwards), and the outputs of their rows
+    const float *zA = z + (long long)k0 * m + p, *zB = z + (long long)(n - 1 - k0) * m + p;
+    df *oA = out + (long long)(n - 1 - k0) * m + p, *oB = out + (long long)k0 * m + p;
     if (k0 > 0) {
-      a1 = center(k0 - 1);
-      if (theta) aK1 = stiff(k0 - 1, a1);
+      a1 = center(zA - m);
+      if (THETA) aK1 = stiff(load5(zA - m));
     }
-    if (!theta && k0 > 1) a2 = center(k0 - 2);
-    {
-      const int kb = n - 1 - k0;
-      b0 = center(kb);
-      if (theta) bK0 = stiff(kb, b0);
-      else if (kb > 0) b1 = center(kb - 1);
-    }
+    if (!THETA && k0 > 1) a2 = center(zA - 2 * m);
+    b0 = center(zB);
+    if (THETA) bK0 = stiff(load5(zB));
+    else if (n - 1 - k0 > 0) b1 = center(zB - m);
     // planes read by iteration kA: A-walk plane kA; mirrored walk plane kB - 1 (theta) or kB
     // plus the centre of kB - 2 (BDF2)
-    auto planes = [&](int kA, P5 &A, P5 &B, float &C) {
+    auto planes = [&](int kA, P5 &A, P5 &B, f2 &C) {
       const int kB = n - 1 - kA;
-      A = load5(kA);
-      B = P5{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      C = 0.f;
+      A = load5(zA);
+      B = none;
+      C = O;
       if (kB != kA) {
-        if (theta) {
-          if (kB > 0) B = load5(kB - 1);
+        if (THETA) {
+          B = load5(zB - m);
         } else {
-          B = load5(kB);
-          if (kB > 1) C = __ldg(z + (long long)(kB - 2) * m + p);
+          B = load5(zB);
+          if (kB > 1) C = center(zB - 2 * m);
         }
       }
+      zA += m;
+      zB -= m;
     };
-    P5 pA{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, pB = pA;
-    float pC = 0.f;
+    P5 pA = none, pB = none;
+    f2 pC = O;
     if (k0 < k1) planes(k0, pA, pB, pC);
-    for (int kA = k0; kA < k1; ++kA) {
-      P5 nA{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, nB = nA;
-      float nC = 0.f;
+    // Both walks' arithmetic is one straight piece of code (kB > kA, so kB > 0), so that their two
+    // dependent chains overlap; the middle plane of an odd n, its own mirror, follows the loop.
+    const int k2 = min(k1, n >> 1);
+    for (int kA = k0; kA < k2; ++kA) {
+      P5 nA = none, nB = none;
+      f2 nC = O;
       if (kA + 1 < k1) planes(kA + 1, nA, nB, nC);
-      const int kB = n - 1 - kA;
-      const float cA = pA.c;
-      const df KA = stiff5(pA, cA);
-      const df yA = combine(cA, a1, a2, KA, aK1);
-      if (theta) {
+      const f2 cA = pA.c;
+      const df2 KA = stiff(pA), KB = stiff(pB);
+      const df2 yA = masked(combine(cA, a1, a2, KA, aK1));
+      const df2 yB = masked(THETA ? combine(b0, pB.c, O, bK0, KB) : combine(b0, b1, pC, KB, zero));
+      D.add_prod(yA, b0, b0 * neg1);  // b0: z in plane kB, partner of yA
+      D.add_prod(yB, cA, cA * neg1);
+      store(oA, yA);
+      store(oB, yB);
+      oA -= m;
+      oB += m;
+      if (THETA) {
         aK1 = KA;
+        bK0 = KB;
+        b0 = pB.c;
       } else {
         a2 = a1;
+        b0 = b1;
+        b1 = pC;
       }
       a1 = cA;
-      const bool twin = (kB != kA);
-      const float zB = twin ? b0 : cA;
-      df yB = zero;
-      if (twin) {
-        if (theta) {
-          float nb = 0.f;
-          df nK = zero;
-          if (kB > 0) {
-            nb = pB.c;
-            nK = stiff5(pB, nb);
-          }
-          yB = combine(b0, nb, 0.f, bK0, nK);
-          b0 = nb;
-          bK0 = nK;
-        } else {
-          const df KB = stiff5(pB, b0);
-          const float nb2 = (kB > 1) ? pC : 0.f;
-          yB = combine(b0, b1, nb2, KB, zero);
-          b0 = b1;
-          b1 = nb2;
-        }
-      }
-      out[(long long)kB * m + p] = yA;
-      D.add_prod(yA, zB);
-      if (twin) {
-        out[(long long)kA * m + p] = yB;
-        D.add_prod(yB, cA);
-      }
       pA = nA;
       pB = nB;
       pC = nC;
     }
+    if (k2 < k1) {
+      const df2 y = masked(combine(pA.c, a1, a2, stiff(pA), aK1));
+      store(oA, y);
+      D.add_prod(y, pA.c, pA.c * neg1);
+    }
   }
-  const double acc = (double)D.s + (double)D.t;
+  float s0, s1, t0, t1;
+  unpack2(D.s, s0, s1);
+  unpack2(D.t, t0, t1);
+  const double acc = ((double)s0 + (double)s1) + ((double)t0 + (double)t1);
   const int nb = gridDim.x * gridDim.y * gridDim.z;
   const int bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
   double tot;
@@ -695,8 +831,8 @@ __global__ void k_grad_nodes(int dim, int mx, int my, int nchunk, const double *
 }  // namespace
 
 int stencil_blocks(const Geom &g) {
-  Tile t = tile_for(g);
-  return t.gx * t.gy * t.nchunk;
+  const Tile t = tile_for(g), d = tile_df_for(g);
+  return std::max(t.gx * t.gy * t.nchunk, d.gx * d.gy * d.nchunk);
 }
 
 template <class Tz>
@@ -725,21 +861,34 @@ cudaError_t launch_stencil(const Geom &g, int mode, const Tz *z, double *out, co
 
 cudaError_t launch_stencil_df(const Geom &g, const float *z, df *q, State *S, double *partials,
                               cudaStream_t st) {
-  Tile t = tile_for(g);
-  dim3 block = (g.dim == 1) ? dim3(kBX1, 1) : dim3(kBX2, kBY2);
-  dim3 grid(t.gx, t.gy, t.nchunk);
+  const Tile t = tile_df_for(g);
+  const dim3 block(t.bx, kNT / t.bx), grid(t.gx, t.gy, t.nchunk);
+  const double th = g.theta;
   prof_begin(KC_STENCIL, st);
-  if (g.dim == 3) {
-    if (g.c_uniform)
-      k_stencil_df<true, true><<<grid, block, 0, st>>>(g, z, q, S, partials, t.kc);
+  auto go = [&](auto dim, auto uni) {
+    constexpr int D = decltype(dim)::value;
+    constexpr bool U = decltype(uni)::value;
+    if (g.scheme != ST_THETA)
+      k_stencil_df<D, U, W_BDF2><<<grid, block, 0, st>>>(g, z, q, S, partials, t.kc);
+    else if (th == 0.5)
+      k_stencil_df<D, U, W_HALF><<<grid, block, 0, st>>>(g, z, q, S, partials, t.kc);
+    else if (th == 1.0)
+      k_stencil_df<D, U, W_ONE><<<grid, block, 0, st>>>(g, z, q, S, partials, t.kc);
     else
-      k_stencil_df<true, false><<<grid, block, 0, st>>>(g, z, q, S, partials, t.kc);
-  } else {
+      k_stencil_df<D, U, W_ANY><<<grid, block, 0, st>>>(g, z, q, S, partials, t.kc);
+  };
+  auto pick = [&](auto dim) {
     if (g.c_uniform)
-      k_stencil_df<false, true><<<grid, block, 0, st>>>(g, z, q, S, partials, t.kc);
+      go(dim, std::true_type{});
     else
-      k_stencil_df<false, false><<<grid, block, 0, st>>>(g, z, q, S, partials, t.kc);
-  }
+      go(dim, std::false_type{});
+  };
+  if (g.dim == 3)
+    pick(std::integral_constant<int, 3>{});
+  else if (g.dim == 2)
+    pick(std::integral_constant<int, 2>{});
+  else
+    pick(std::integral_constant<int, 1>{});
   prof_end(st);
   return cudaGetLastError();
 }
