@@ -335,7 +335,7 @@ struct DstSmem {
   static __host__ __device__ uint32_t total(const TmaDim &D, int NB) { return bop(D, NB) + 2u * D.bb + 1008u; }
 };
 
-// XL: `groups` is the number of lines, chunks = px / 32, and in0 serves loads and stores, unless `user`
+// XL: `groups` is the number of lines, chunks = px / 32, out0 takes the result, unless `user`
 // takes the lines without their padding (contiguous, not aligned: the store warp copies them); else
 // groups of 32 columns, `chunks` of them in a plane, and out0 / out1 take the odd and even outputs.
 template <int SL, bool XL>
@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(kNTS, 1)
         const uint32_t src = ring + (uint32_t)s * D.rb;
         if (XL) {
           for (int c = 0; c < chunks; ++c)
-            tma_store3(&in0, src + (uint32_t)c * (32u * SL * 128u), c * 32, (int)(tile * per), 0);
+            tma_store3(&out0, src + (uint32_t)c * (32u * SL * 128u), c * 32, (int)(tile * per), 0);
         } else {
           for (int g = 0; g < SL; ++g) {
             const unsigned gi = tile * per + g;
@@ -962,7 +962,9 @@ cudaError_t launch_dst(const float *in, float *out, int len, long long cols, lon
     chunks = (len + 1) / 32;
     groups = (unsigned)planes;  // lines
     e = tma_encode(&mi, in, len + 1, planes, 1, len + 1, (long long)(len + 1) * planes, 32 * SL);
-    m0 = m1 = mi;
+    if (e == cudaSuccess)
+      e = tma_encode(&m0, out, len + 1, planes, 1, len + 1, (long long)(len + 1) * planes, 32 * SL);
+    m1 = m0;
   } else {
     chunks = (int)((cols + 31) / 32);
     groups = (unsigned)(planes * chunks);
@@ -1062,9 +1064,9 @@ void dst_tma_build_image(int len, unsigned short *out) {
   }
 }
 
-cudaError_t launch_dst_tma_x(float *data, const Geom &g, const unsigned short *img, State *S,
-                             int gk, cudaStream_t st, float *user) {
-  return launch_dst_any<true>(data, data, g.mx, 0, (long long)g.n * g.my * g.mz, 0, 0, img, S, gk,
+cudaError_t launch_dst_tma_x(const float *in, float *out, const Geom &g, const unsigned short *img,
+                             State *S, int gk, cudaStream_t st, float *user) {
+  return launch_dst_any<true>(in, out, g.mx, 0, (long long)g.n * g.my * g.mz, 0, 0, img, S, gk,
                               KC_DSTX, st, user);
 }
 

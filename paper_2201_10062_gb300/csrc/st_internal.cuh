@@ -398,10 +398,10 @@ void dst_tma_build_image(int len, unsigned short *out);
 cudaError_t launch_time_tma(float *data, const Geom &g, const Spec<float> &sp,
                             const unsigned short *img, State *S, int tmode, double *partials,
                             int gk, cudaStream_t st);
-// one DST-I along x (in place, or into a caller's contiguous vector), y or z (in place), and along
+// one DST-I along x (in place, into another vector, or into a caller's contiguous one), y or z (in place), and along
 // time alone (in -> out)
-cudaError_t launch_dst_tma_x(float *data, const Geom &g, const unsigned short *img, State *S,
-                             int gk, cudaStream_t st, float *user = nullptr);
+cudaError_t launch_dst_tma_x(const float *in, float *out, const Geom &g, const unsigned short *img,
+                             State *S, int gk, cudaStream_t st, float *user = nullptr);
 cudaError_t launch_dst_tma_y(float *data, const Geom &g, const unsigned short *img, State *S,
                              int gk, cudaStream_t st);
 cudaError_t launch_dst_tma_z(float *data, const Geom &g, const unsigned short *img, State *S,

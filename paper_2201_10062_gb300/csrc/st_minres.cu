@@ -977,7 +977,7 @@ int build_tables(st_handle *h) {
   // for the FFT at 255^2 x 256); st_autotune times both, and ST_X_TENSOR_CORES=0 starts a handle
   // with the FFT.  The P_theta paths with varying a run their x passes through the Chebyshev and
   // PCR kernels.
-  h->tc_x_img = (sopx.empty() || pp.pcr || pp.cheb)
+  h->tc_x_img = (sopx.empty() || pp.pcr)
                     ? nullptr
                     : reinterpret_cast<const unsigned short *>((const char *)h->tables + o_sopx);
   {

@@ -17,6 +17,8 @@
 // accumulates <v, P^-1 v> = sum v~^2 / p for MINRES.
 #include <math.h>
 
+#include <algorithm>
+
 #include "st_fft.cuh"
 #include "st_internal.cuh"
 #include "st_symbol.cuh"
@@ -447,6 +449,35 @@ struct SrcChebScale {
   }
 };
 
+// w <- s_k / (lam_H,k + lam_Htheta,k tau mu) w (SrcChebScale's factor, in its order), where the x
+// passes around it take the tensor cores and cannot apply it as they load.  Four slots of a line a
+// thread; bound by L2 and memory, 8 bytes an unknown: the two tensor-core x passes and this one
+// take 44 us at 255^2 x 128 against 90 us for the two FFT passes.  The padding slot stays zero.
+__global__ void __launch_bounds__(kNT)
+    k_cheb_scale(float *__restrict__ w, unsigned quads, int n, unsigned lq, int mx,
+                 const float *__restrict__ s, const float *__restrict__ lh,
+                 const float *__restrict__ lht, const float *__restrict__ mux,
+                 const float *__restrict__ muy, const State *S, int gk) {
+  if (gate_closed(S, gk)) return;
+  const unsigned q = blockIdx.x * kNT + threadIdx.x;  // quad within a level
+  if (q >= quads) return;
+  const unsigned row = q >> lq, ix = (q - (row << lq)) * 4u;
+  const float my = muy[row];
+  const float m0 = mux[ix] + my, m1 = mux[ix + 1] + my, m2 = mux[ix + 2] + my;
+  const bool last = (int)ix + 3 >= mx;
+  const float m3 = last ? 0.f : mux[ix + 3] + my;
+  for (int k = blockIdx.y; k < n; k += gridDim.y) {
+    const float sk = s[k], a = lh[k], b = lht[k];
+    float4 *p = reinterpret_cast<float4 *>(w) + (size_t)k * quads + q;
+    float4 v = *p;
+    v.x = v.x * sk / (a + b * m0);
+    v.y = v.y * sk / (a + b * m1);
+    v.z = v.z * sk / (a + b * m2);
+    v.w = last ? 0.f : v.w * sk / (a + b * m3);
+    *p = v;
+  }
+}
+
 // Face coefficient tau a / h^2 in the transform type: float64 tables for float64, the leading
 // float of the double-float copy for float32 (no float64 conversion per element).
 template <class Tc>
@@ -825,7 +856,8 @@ template <class Tc, class Tout>
 cudaError_t dst_x_last_pass(Tout *z, const Geom &g, const PrecPlan &pp, State *S, int gk,
                             cudaStream_t st) {
   if (sizeof(Tc) == sizeof(float) && pp.sop_x != nullptr)
-    return launch_dst_tma_x(reinterpret_cast<float *>(z), g, pp.sop_x, S, gk, st);
+    return launch_dst_tma_x(reinterpret_cast<float *>(z), reinterpret_cast<float *>(z), g, pp.sop_x,
+                            S, gk, st);
   const long long nx = (long long)g.n * g.my * g.mz;
   const int px = lay<Tc>(g).px;
   return launch_dst<Tc, SrcArray<Tc, Tout>, Tout, true>(SrcArray<Tc, Tout>{z}, z, g.mx, pp.Lx,
@@ -931,14 +963,35 @@ cudaError_t cheb_stages(const Geom &g, const PrecPlan &pp, Src src, Tc *zc, Stat
   for (int j = 0; j < pp.cheb; ++j) {
     // the axes commute: x, y (z), then x with the scaling fused into its loads, then y (z); the
     // y and z passes take the tensor cores in float32 when the plan has the S_my / S_mz image
-    e = launch_dst<Tc, Arr, Tc, true>(Arr{j == 0 ? zc : R}, wc, g.mx, pp.Lx, nx, g.mx, 0, 0, y.px,
-                                      y.px, twx, S, gk, pp.dst_shift, st);
+    const bool xtc = sizeof(Tc) == sizeof(float) && pp.sop_x != nullptr && g.N >= (3LL << 18);
+    if (xtc)
+      e = launch_dst_tma_x(reinterpret_cast<const float *>(j == 0 ? zc : R),
+                           reinterpret_cast<float *>(wc), g, pp.sop_x, S, gk, st);
+    else
+      e = launch_dst<Tc, Arr, Tc, true>(Arr{j == 0 ? zc : R}, wc, g.mx, pp.Lx, nx, g.mx, 0, 0,
+                                        y.px, y.px, twx, S, gk, pp.dst_shift, st);
     if (e != cudaSuccess) return e;
     if ((e = yz()) != cudaSuccess) return e;
-    const SrcChebScale<Tc> sc{wc, scoef + (size_t)j * g.n, sp.lh, sp.lht, sp.mux, sp.muy,
+    if (xtc) {
+      const unsigned quads = (unsigned)(y.mp / 4);
+      unsigned lq = 0;
+      while ((4u << lq) < (unsigned)y.px) ++lq;
+      const Spec<float> &sf = pp.spec_f;
+      prof_begin(KC_AUX, st);
+      k_cheb_scale<<<dim3((quads + kNT - 1) / kNT, (unsigned)std::min(g.n, 4096)), kNT, 0, st>>>(
+          reinterpret_cast<float *>(wc), quads, g.n, lq, g.mx,
+          reinterpret_cast<const float *>(scoef) + (size_t)j * g.n, sf.lh, sf.lht, sf.mux, sf.muy,
+          S, gk);
+      prof_end(st);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      e = launch_dst_tma_x(reinterpret_cast<float *>(wc), reinterpret_cast<float *>(wc), g, pp.sop_x,
+                           S, gk, st);
+    } else {
+      const SrcChebScale<Tc> sc{wc, scoef + (size_t)j * g.n, sp.lh, sp.lht, sp.mux, sp.muy,
                               (unsigned)y.mp, (unsigned)y.px};
-    e = launch_dst<Tc, SrcChebScale<Tc>, Tc, true>(sc, wc, g.mx, pp.Lx, nx, g.mx, 0, 0, y.px, y.px,
-                                                   twx, S, gk, pp.dst_shift, st);
+      e = launch_dst<Tc, SrcChebScale<Tc>, Tc, true>(sc, wc, g.mx, pp.Lx, nx, g.mx, 0, 0, y.px, y.px,
+                                                     twx, S, gk, pp.dst_shift, st);
+    }
     if (e != cudaSuccess) return e;
     if ((e = yz()) != cudaSuccess) return e;  // back in W
     const Tc *aj = acoef + (size_t)j * g.n;
@@ -1080,8 +1133,8 @@ cudaError_t prec_stages(const Geom &g, const PrecPlan &pp, Src src, Tout *z, Sta
   // a caller's contiguous output: the last pass leaves the padding out
   if (user) {
     if (sizeof(Tc) == sizeof(float) && pp.sop_x != nullptr)
-      return launch_dst_tma_x(reinterpret_cast<float *>(z), g, pp.sop_x, S, gk, st,
-                              reinterpret_cast<float *>(user));
+      return launch_dst_tma_x(reinterpret_cast<float *>(z), reinterpret_cast<float *>(z), g, pp.sop_x,
+                              S, gk, st, reinterpret_cast<float *>(user));
     return launch_dst<Tc, SrcArray<Tc, Tout>, Tout, true>(SrcArray<Tc, Tout>{z}, user, g.mx, pp.Lx,
                                                           nx, g.mx, 0, 0, lay<Tc>(g).px, g.mx,
                                                           tw_of<Tc>(pp, true), S, gk,
