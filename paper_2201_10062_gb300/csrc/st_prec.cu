@@ -64,7 +64,7 @@ struct StockhamPasses {
 // and the fused Lanczos source (its loads held in registers ahead of the stores): two
 template <class Tc, class Src, class Tout, bool XL, int LOGL>
 __global__ void __launch_bounds__(kNTD, (sizeof(Tc) == 4 && !has_fetch<Src>::value) ? 3 : 2)
-    k_dst_space(Src src, Tout *out, int len, long long nlines, int mx, long long ld, long long m,
+    k_dst_space(Src src, Tout *out, int len, long long nlines, int mx, int ld, long long m,
                 int pin, int pout, const Tc *tw, int PB, const State *S, int gk) {
   if (gate_closed(S, gk)) return;
   src.prepare(S);
