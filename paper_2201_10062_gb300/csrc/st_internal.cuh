@@ -31,7 +31,9 @@ struct Geom {
   // float32 and double-float vectors of the mixed path are stored with one padding slot after each
   // x line: px = mx + 1 (a power of two) slots a line, mp = px*my*mz a time level, Np = n*mp in
   // all.  Lines, planes and levels then start on 16-byte boundaries (tensor copies need that),
-  // and the padding holds zeros: the Dirichlet values the stencil reads on either side of a line.
+  // and the padding of z holds zeros: the Dirichlet values the stencil reads on either side of a
+  // line.  The first pass of a preconditioner application writes them (the later ones carry a zero
+  // column along), so nothing of an earlier call's data can be left there.
   int px;
   long long mp, Np;
 };

@@ -1366,8 +1366,10 @@ int st::setup_handle(const st_problem *prob, st_handle **out, int ugroup) {
     if (e == cudaSuccess && !h->mixed) e = cudaMalloc(&h->Z[i], N * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&h->D[i], Nv * sizeof(double));
   }
-  // z vectors of a mixed handle, with those of the iterations a grouped update keeps pending; their
-  // padding stays zero from here on
+  // z vectors of a mixed handle, with those of the iterations a grouped update keeps pending.  The
+  // zeros are for the slots in front of the first one: the padding of a vector is written by the
+  // first pass of every preconditioner application (a vector's neighbour to the left, whose last
+  // slot the stencil reads, is the z of the iteration before)
   h->ugroup = h->mixed ? ugroup : 1;
   if (e == cudaSuccess && h->mixed) {
     const size_t zf = zslab_floats(g, ugroup);

@@ -37,7 +37,7 @@ constexpr int kNT = 256;
 
 // ------------------------------------------------------------------------------ spatial DST
 // XL = true: lines are rows (contiguous; line l starts at l*pin in the source and at l*pout in the
-// output: the line length len, or len + 1 in the padded layout).
+// output: the line length len, or len + 1 in the padded layout, whose last slot is set to zero).
 // XL = false: lines are columns of planes: line l = k*mx + i starts at k*m + i and its elements are
 // `ld` apart; columns i with i mod pin >= pout are left alone (the padding columns of z lines: the
 // two lines of a packed pair leave rounding in each other, and the padding stays exactly zero).  A block owns 2*PB consecutive lines (PB complex sequences, line
@@ -163,12 +163,15 @@ __global__ void __launch_bounds__(kNTD, (sizeof(Tc) == 4 && !has_fetch<Src>::val
   if (XL) {
     for (int idx = tid; idx < (PB << logH); idx += kNTD) {
       const int pp = idx >> logH, e = idx & (half - 1);
-      if (e >= len) continue;
+      if (e >= pout) continue;
       const cpx<Tc> Z = buf[pp * Ls + fft_pad<Tc>(e + 1)];
       const int la = 2 * pp, lb = la + 1;
       Tout *p = out + (line0 + la) * pout + e;
-      if (la < nl) p[0] = (Tout)(-Z.y * sc);
-      if (lb < nl) p[pout] = (Tout)(Z.x * sc);
+      // e = len is the padding slot of a padded line (half = len + 1).  It gets a zero on every
+      // pass: an earlier call on non-finite data may have left 0 x NaN there.
+      const bool pad = e == len;
+      if (la < nl) p[0] = pad ? Tout(0) : (Tout)(-Z.y * sc);
+      if (lb < nl) p[pout] = pad ? Tout(0) : (Tout)(Z.x * sc);
     }
   } else {
     const int pp = tid & (PB - 1), estep = kNTD >> logPB;
@@ -546,18 +549,23 @@ __global__ void __launch_bounds__(kChebBX * kChebBY)
 // the transform type (float64 arithmetic per element would bind a float32 pass to the slow
 // float64 pipe) and combined across threads in float64.  o is a separate array: rewriting z in
 // place inside this accumulating loop measured five times slower (213 against 43 us per
-// 255^2 x 128 float pass).
+// 255^2 x 128 float pass).  Slots e with (e & pmask) == pcol are padding: o gets a zero there, and
+// nothing of the other vectors' padding, which no step of the map writes, is used.
 template <class Tc>
 __global__ void __launch_bounds__(kNT)
-    k_cheb_final(long long N, long long m, const Tc *__restrict__ dprev,
-                 const Tc *__restrict__ w, const Tc *__restrict__ x, const Tc *__restrict__ z,
-                 Tc *__restrict__ o, const Tc *__restrict__ acoef, int first, State *S, int tmode,
-                 double *__restrict__ partials, int gk) {
+    k_cheb_final(long long N, long long m, unsigned pmask, unsigned pcol,
+                 const Tc *__restrict__ dprev, const Tc *__restrict__ w, const Tc *__restrict__ x,
+                 const Tc *__restrict__ z, Tc *__restrict__ o, const Tc *__restrict__ acoef,
+                 int first, State *S, int tmode, double *__restrict__ partials, int gk) {
   __shared__ double red[32];
   if (gate_closed(S, gk)) return;
   Tc esum = Tc(0), ecomp = Tc(0);
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < N;
        e += (long long)gridDim.x * blockDim.x) {
+    if (((unsigned)e & pmask) == pcol) {
+      o[e] = Tc(0);
+      continue;
+    }
     const unsigned k = (unsigned)e / (unsigned)m;
     const Tc d = first ? w[e] : acoef[k] * dprev[e] + w[e];
     const Tc xv = first ? d : x[e] + d;
@@ -582,17 +590,18 @@ __global__ void __launch_bounds__(kNT)
 }
 
 // z = source elements in the transform type (a conversion, or the fused Lanczos step), line by
-// line: pin slots a line in the source, pout in z.  The padding slots of z keep their zeros.
+// line: pin slots a line in the source, pout in z.  The padding slot of a z line is set to zero,
+// whatever an earlier call left there.
 template <class Tc, class Src>
 __global__ void k_copy_to(unsigned nlines, int mx, int pin, int pout, Src src, Tc *z,
                           const State *S, int gk) {
   if (gate_closed(S, gk)) return;
   src.prepare(S);
-  const unsigned total = nlines * (unsigned)mx;  // = N < 2^31
+  const unsigned total = nlines * (unsigned)pout;  // at most 4/3 N < 3 2^30 (mx >= 3)
   for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += gridDim.x * blockDim.x) {
-    const unsigned l = e / (unsigned)mx, i = e - l * (unsigned)mx;
-    z[(long long)l * pout + i] = src((long long)l * pin + i);
+    const unsigned l = e / (unsigned)pout, i = e - l * (unsigned)pout;
+    z[e] = (int)i < mx ? src((long long)l * pin + i) : Tc(0);
   }
 }
 
@@ -1006,8 +1015,11 @@ cudaError_t cheb_stages(const Geom &g, const PrecPlan &pp, Src src, Tc *zc, Stat
       cur ^= 1;
     } else {
       prof_begin(KC_TIME, st);
-      k_cheb_final<Tc><<<kChebBlocks, kNT, 0, st>>>(N, y.mp, Dd[cur], W, X, zc, R, aj,
-                                                    j == 0 ? 1 : 0, S, tmode, partials, gk);
+      // padded lines have px = mx + 1 slots, a power of two; others have no slot to skip
+      const bool padded = y.px != g.mx;
+      k_cheb_final<Tc><<<kChebBlocks, kNT, 0, st>>>(
+          N, y.mp, padded ? (unsigned)g.mx : 0u, padded ? (unsigned)g.mx : 1u, Dd[cur], W, X, zc, R,
+          aj, j == 0 ? 1 : 0, S, tmode, partials, gk);
       prof_end(st);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
