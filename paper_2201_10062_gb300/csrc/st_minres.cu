@@ -930,8 +930,6 @@ int build_tables(st_handle *h) {
   if (cheb) {
     const size_t cb = cheb_coef_bytes(g, cheb);
     ST_TRY(cudaMalloc(&h->cheb, cb + 5 * (size_t)g.N * sizeof(double)));
-    // the scratch vectors' padding slots hold zeros
-    ST_TRY(cudaMemset((char *)h->cheb + cb, 0, 5 * (size_t)g.N * sizeof(double)));
     const size_t cnt = (size_t)cheb * n;
     std::vector<float> af(cnt), sf(cnt);
     for (size_t i = 0; i < cnt; ++i) {
@@ -1730,9 +1728,6 @@ int st_apply_prec(st_handle *h, const double *v_dev, double *z_dev) {
   ST_ENTER(h);
   ST_TRY((launch_prec<double, double, double>(h->g, h->pp, v_dev, z_dev, h->S, TM_NONE,
                                               h->partials, h->stream)));
-  // the float64 pass used the Chebyshev scratch unpadded: the mixed path wants its padding zero
-  if (h->mixed && h->pp.cheb)
-    ST_TRY(cudaMemsetAsync(h->pp.cheb_work, 0, 5 * (size_t)h->g.N * sizeof(double), h->stream));
   return ST_OK;
 }
 
@@ -1740,13 +1735,8 @@ int st_apply_prec_f32(st_handle *h, const double *v_dev, float *z_dev) {
   if (!h || !v_dev || !z_dev) return ST_ERR_ARG;
   ProfScope prof_scope(h);
   ST_ENTER(h);
-  // the passes work on a padded vector of the handle (Z[0], free between solves); on a float64
-  // handle, whose vectors are not padded, its slots (and the Chebyshev scratch) are zeroed first
-  if (!h->mixed) {
-    ST_TRY(cudaMemsetAsync(h->zscratch, 0, (size_t)h->g.Np * sizeof(float), h->stream));
-    if (h->pp.cheb)
-      ST_TRY(cudaMemsetAsync(h->pp.cheb_work, 0, 5 * (size_t)h->g.N * sizeof(double), h->stream));
-  }
+  // the passes work on a padded vector of the handle (Z[0], free between solves; N float64 slots of a
+  // float64 handle hold Np <= 4/3 N float32 ones)
   ST_TRY(launch_prec_user(h->g, h->pp, v_dev, h->zscratch, z_dev, h->S, h->partials, h->stream));
   return ST_OK;
 }
