@@ -152,6 +152,13 @@ __device__ __forceinline__ dd inv_sym_dd(const Spec<dd> &sp, const SymRowDD &r, 
   return rsqrt_dd(dd_fma(re, re, im * im));
 }
 
+// max(a, b), NaN if either is one
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
 // The seven 7-bit digits of x 2^e (|x 2^e| < 2^7, double-float): X = 2^42 x 2^e rounded to an
 // integer, held as H 2^21 + Lo with 0 <= Lo < 2^21 (32-bit parts: no float64 conversion), is
 // d_0 2^42 + sum_k d_k 2^(42-7k) with d_0 = H >> 21 (signed) and d_k the 7-bit fields below.
@@ -327,7 +334,7 @@ __global__ void __launch_bounds__(kNTG, 1)
                 const dd x2 = ld_dd(in + (long long)tm * m + j0 + bc);
                 f[it][q] = P == 0 ? x1 + x2 : x1 - x2;
               }
-              mxv = fmaxf(mxv, fabsf(f[it][q].hi));
+              mxv = max_nan(mxv, fabsf(f[it][q].hi));
             }
           }
         }
@@ -335,14 +342,17 @@ __global__ void __launch_bounds__(kNTG, 1)
         group_sync(kBarB, kBuildW * 32);
         float cm = 0.f;
 #pragma unroll
-        for (int k = 0; k < kBuildW; ++k) cm = fmaxf(cm, part[k * kTN + bc]);
+        for (int k = 0; k < kBuildW; ++k) cm = max_nan(cm, part[k * kTN + bc]);
+        // digits hold no NaN or infinity: a column with one gets the factor NaN, which the drain
+        // multiplies the whole column of the result by
+        const bool fin = isfinite(cm);
         int e = 0;
-        if (cm > 0.f && isfinite(cm)) {
+        if (cm > 0.f && fin) {
           int E;
           frexpf(cm, &E);
           e = 7 - E;  // cm 2^e in [2^6, 2^7)
         }
-        if (bw == 0) cdown[b * kTN + bc] = pow2f(-(eS + e));
+        if (bw == 0) cdown[b * kTN + bc] = fin ? pow2f(-(eS + e)) : __int_as_float(0x7fc00000);
         const float up21 = pow2f(e + 21);
         unsigned char *bb = smem + L.bdig + (uint32_t)b * bbytes;
 #pragma unroll

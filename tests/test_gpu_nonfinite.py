@@ -128,3 +128,20 @@ def test_batch_after_one_bad_instance(pkg):
             for u, r in zip(outs, ref):
                 assert torch.equal(u, r)
     b.close()
+
+
+@pytest.mark.parametrize("n", [129, 200, 224, 256])
+@pytest.mark.parametrize("bad", BAD[:2])
+def test_float64_digit_stage_keeps_nonfinite_values(pkg, n, bad):
+    """The float64 path's time stage on integer digits, which have no NaN and no infinity: as through
+    the CUDA-core stages, one of them reaches the whole result, and ends a solve with a breakdown."""
+    spec = _spec(pkg, 2, 63, 31, 1, n, "PH", "fp64")
+    v = _data(spec)
+    s = pkg.Solver(spec)
+    ref = s.st_apply_prec(v)
+    assert not torch.isfinite(s.st_apply_prec(_with(v, bad))).any()
+    assert torch.equal(s.st_apply_prec(v), ref)
+    with pytest.raises(pkg.SolverError) as e:
+        s.st_solve(_with(v, bad), tol=1e-8, maxit=40)
+    assert e.value.code == pkg.ST_ERR_BREAKDOWN
+    s.close()
