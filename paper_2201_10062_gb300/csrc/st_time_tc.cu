@@ -350,7 +350,9 @@ __global__ void __launch_bounds__(kNTG, 1)
         if (cm > 0.f && fin) {
           int E;
           frexpf(cm, &E);
-          e = 7 - E;  // cm 2^e in [2^6, 2^7)
+          // cm 2^e in [2^6, 2^7); below 2^-100 the digits end at 2^-148, where float32 itself does,
+          // and 2^(e + 21) stays finite
+          e = min(7 - E, 106);
         }
         if (bw == 0) cdown[b * kTN + bc] = fin ? pow2f(-(eS + e)) : __int_as_float(0x7fc00000);
         const float up21 = pow2f(e + 21);
