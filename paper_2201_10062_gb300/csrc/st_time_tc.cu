@@ -41,12 +41,13 @@ int time_tc_grid() {
 // long as every partial sum stays below 2^24, so both operands are cut into integer digits:
 //   S^ = S 2^eS = sum_i S_i 2^-7i,   X^ = X 2^ec = sum_j B_j 2^-7j,   i, j = 0..6,
 // with |S_i|, |B_j| <= 2^7 (one scale for S, one per column c of X and parity).  S's digits are
-// rounded ones taken in float64 on the host; X's are the 7-bit fields of the folded double-float
-// value as a 64-bit fixed-point integer (2^42 X^, rounded), the top one signed.  One product
+// rounded ones taken in float64 on the host; X's are those of the folded double-float value as a
+// 64-bit fixed-point integer (2^42 X^, rounded), in -64..63 below the top one.  One product
 // S_i B_j over K = h <= 128 folded rows is at most 2^21 in magnitude, and the at most seven
 // products of a digit group g = i + j sum below 2^24, so each group accumulates exactly in
 // float32.  The groups g <= 6 are kept (28 products per parity); the dropped ones and the
-// digits' remainders are below 2^-41 of the column's largest entry.  The groups are summed in
+// digits' remainders are below 2^-41 of the column's largest entry, and of no sign: measured against
+// float64 the stage is the more accurate one.  The groups are summed in
 // double-float (sum_g acc_g 2^-7g, TwoSum) and unscaled by 2^-(eS + ec).
 //
 // With S's digits read from shared memory each MMA (M = 128, N = 32) costs about ten times one
@@ -161,22 +162,38 @@ __device__ __forceinline__ float max_nan(float a, float b) {
 
 // The seven 7-bit digits of x 2^e (|x 2^e| < 2^7, double-float): X = 2^42 x 2^e rounded to an
 // integer, held as H 2^21 + Lo with 0 <= Lo < 2^21 (32-bit parts: no float64 conversion), is
-// d_0 2^42 + sum_k d_k 2^(42-7k) with d_0 = H >> 21 (signed) and d_k the 7-bit fields below.
-__device__ __forceinline__ void digits7(dd x, float up21, int (&d)[kDg]) {
+// sum_k d_k 2^(42-7k) with d_0 signed and -64 <= d_k < 64 below it: half of every lower digit's
+// range is added to X first, and the 7-bit fields of the sum are d_k + 64.  Balanced, the products that
+// the digit groups leave out have no mean.  (With d_k in 0..127 they left the same error in every
+// column, which the transforms along space gather in a few nodes: at 127 x 63 x 191 a largest error
+// of 5.2e-13 of the largest entry, now 2.0e-14; the double-float kernel's is 5.9e-14.)
+// Returned are the fields d_0 + 128 and d_k + 64: 0..256 and 0..127.
+__device__ __forceinline__ void digits7(dd x, float up21, uint32_t (&d)[kDg]) {
+  constexpr int kMid = (64 << 14) | (64 << 7) | 64;
   const float xh = x.hi * up21, xl = x.lo * up21;  // exact: powers of two
   int H = __float2int_rn(xh);                      // |H| <= 2^28; exact when |xh| >= 2^24
   const float r = xh - (float)H;                   // exact, |r| <= 1/2
   int Lo = __float2int_rn((r + xl) * 2097152.0f);  // (r + xl) 2^21; the rounding is below 1
+  Lo += kMid;
   const int carry = Lo >> 21;                      // floor(Lo / 2^21)
-  Lo -= carry * 2097152;
-  H += carry;
-  d[0] = H >> 21;
-  d[1] = (H >> 14) & 127;
-  d[2] = (H >> 7) & 127;
-  d[3] = H & 127;
-  d[4] = (Lo >> 14) & 127;
-  d[5] = (Lo >> 7) & 127;
-  d[6] = Lo & 127;
+  const uint32_t L = (uint32_t)Lo;
+  const uint32_t U = (uint32_t)H + (uint32_t)carry + (uint32_t)kMid + (128u << 21);
+  d[0] = (U >> 21) & 511u;  // 9 bits: a column that is not finite stays within half's integers too
+  d[1] = (U >> 14) & 127u;
+  d[2] = (U >> 7) & 127u;
+  d[3] = U & 127u;
+  d[4] = (L >> 14) & 127u;
+  d[5] = (L >> 7) & 127u;
+  d[6] = L & 127u;
+}
+
+// two fields as halves, their offset taken off: half 0x6400 | f is 1024 + f for f < 1024
+__device__ __forceinline__ uint32_t digit_pair(uint32_t f0, uint32_t f1, bool top) {
+  const uint32_t v = f0 | (f1 << 16) | 0x64006400u;
+  const uint32_t o = top ? 0x64806480u : 0x64406440u;  // 1024 + 128, 1024 + 64
+  const __half2 r = __hsub2(*reinterpret_cast<const __half2 *>(&v),
+                            *reinterpret_cast<const __half2 *>(&o));
+  return *reinterpret_cast<const uint32_t *>(&r);
 }
 
 // scaled: out = (S_n x)/p per column with <in, P^-1 in> into the MINRES state (tmode);
@@ -361,7 +378,7 @@ __global__ void __launch_bounds__(kNTG, 1)
         for (int it = 0; it < 2; ++it) {
           const int tb = bw + kBuildW * it;
           if (tb >= hb) continue;
-          int dq[8][kDg];
+          uint32_t dq[8][kDg];
 #pragma unroll
           for (int q = 0; q < 8; ++q) digits7(f[it][q], up21, dq[q]);
           const uint32_t off = canon_off(bc, tb * 8, hK);
@@ -369,10 +386,8 @@ __global__ void __launch_bounds__(kNTG, 1)
           for (int dg = 0; dg < kDg; ++dg) {
             uint32_t pk[4];
 #pragma unroll
-            for (int q2 = 0; q2 < 4; ++q2) {
-              const __half2 hv = __floats2half2_rn((float)dq[2 * q2][dg], (float)dq[2 * q2 + 1][dg]);
-              pk[q2] = *reinterpret_cast<const uint32_t *>(&hv);
-            }
+            for (int q2 = 0; q2 < 4; ++q2)
+              pk[q2] = digit_pair(dq[2 * q2][dg], dq[2 * q2 + 1][dg], dg == 0);
             *reinterpret_cast<uint4 *>(bb + (uint32_t)dg * bop + off) =
                 make_uint4(pk[0], pk[1], pk[2], pk[3]);
           }
