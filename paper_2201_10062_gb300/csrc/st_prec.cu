@@ -37,7 +37,8 @@ constexpr int kNT = 256;
 
 // ------------------------------------------------------------------------------ spatial DST
 // XL = true: lines are rows (contiguous; line l starts at l*pin in the source and at l*pout in the
-// output: the line length len, or len + 1 in the padded layout, whose last slot is set to zero).
+// output: the line length len, or len + 1 in the padded layout, whose last slot is set to zero in an
+// output that is not the source).
 // XL = false: lines are columns of planes: line l = k*mx + i starts at k*m + i and its elements are
 // `ld` apart; columns i with i mod pin >= pout are left alone (the padding columns of z lines: the
 // two lines of a packed pair leave rounding in each other, and the padding stays exactly zero).  A block owns 2*PB consecutive lines (PB complex sequences, line
@@ -59,6 +60,34 @@ struct StockhamPasses {
     }
   }
 };
+
+// a source in the transform type and the output's layout whose output is another vector
+template <class Tc>
+struct SrcOther : SrcArray<Tc, Tc> {};
+
+// Sources whose output is another vector than the one they read: the first pass of an application
+// (from the Lanczos vectors or a caller's float64 one), and SrcOther.
+template <class Src>
+struct new_out {
+  static constexpr bool value = false;
+};
+template <class Tc, class Tv>
+struct new_out<SrcLanczos<Tc, Tv>> {
+  static constexpr bool value = sizeof(Tc) == sizeof(float);
+};
+template <>
+struct new_out<SrcArray<float, df>> {
+  static constexpr bool value = true;
+};
+template <>
+struct new_out<SrcArray<float, double>> {
+  static constexpr bool value = true;
+};
+template <class Tc>
+struct new_out<SrcOther<Tc>> {
+  static constexpr bool value = sizeof(Tc) == sizeof(float);
+};
+
 
 // float32 transforms: three 512-thread blocks per SM (at most 40 registers); float64, double-float
 // and the fused Lanczos source (its loads held in registers ahead of the stores): two
@@ -85,6 +114,13 @@ __global__ void __launch_bounds__(kNTD, (sizeof(Tc) == 4 && !has_fetch<Src>::val
   for (int pp = tid; pp < PB; pp += kNTD) {
     buf[pp * Ls + fft_pad<Tc>(0)] = cpx<Tc>{Tc(0), Tc(0)};
     buf[pp * Ls + fft_pad<Tc>(len + 1)] = cpx<Tc>{Tc(0), Tc(0)};
+  }
+  // The padding slots of a vector that the pass does not read: an earlier call on non-finite data
+  // may have left 0 x NaN there.  (As values of the write loop below they cost 8 us of 99 at 255^2 x
+  // 256, here 1; compiled into the in-place pass, where they are zero already, 14 of 137 at 511^2 x 128.)
+  if constexpr (XL && new_out<Src>::value) {
+    if (pout > len)
+      for (int l = tid; l < nl; l += kNTD) out[(line0 + l) * pout + len] = Tout(0);
   }
   // one work item per (sequence, element): both lines of the pair, stored as one complex value
   // at e+1 and its negative at L-1-e (odd extension).  Index maps avoid divisions: len + 1 =
@@ -163,15 +199,12 @@ __global__ void __launch_bounds__(kNTD, (sizeof(Tc) == 4 && !has_fetch<Src>::val
   if (XL) {
     for (int idx = tid; idx < (PB << logH); idx += kNTD) {
       const int pp = idx >> logH, e = idx & (half - 1);
-      if (e >= pout) continue;
+      if (e >= len) continue;
       const cpx<Tc> Z = buf[pp * Ls + fft_pad<Tc>(e + 1)];
       const int la = 2 * pp, lb = la + 1;
       Tout *p = out + (line0 + la) * pout + e;
-      // e = len is the padding slot of a padded line (half = len + 1).  It gets a zero on every
-      // pass: an earlier call on non-finite data may have left 0 x NaN there.
-      const bool pad = e == len;
-      if (la < nl) p[0] = pad ? Tout(0) : (Tout)(-Z.y * sc);
-      if (lb < nl) p[pout] = pad ? Tout(0) : (Tout)(Z.x * sc);
+      if (la < nl) p[0] = (Tout)(-Z.y * sc);
+      if (lb < nl) p[pout] = (Tout)(Z.x * sc);
     }
   } else {
     const int pp = tid & (PB - 1), estep = kNTD >> logPB;
@@ -562,13 +595,10 @@ __global__ void __launch_bounds__(kNT)
   Tc esum = Tc(0), ecomp = Tc(0);
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < N;
        e += (long long)gridDim.x * blockDim.x) {
-    if (((unsigned)e & pmask) == pcol) {
-      o[e] = Tc(0);
-      continue;
-    }
+    const bool pad = ((unsigned)e & pmask) == pcol;
     const unsigned k = (unsigned)e / (unsigned)m;
     const Tc d = first ? w[e] : acoef[k] * dprev[e] + w[e];
-    const Tc xv = first ? d : x[e] + d;
+    const Tc xv = pad ? Tc(0) : first ? d : x[e] + d;
     const Tc term = z[e] * xv - ecomp;
     const Tc t = esum + term;
     ecomp = (t - esum) - term;
@@ -977,8 +1007,9 @@ cudaError_t cheb_stages(const Geom &g, const PrecPlan &pp, Src src, Tc *zc, Stat
       e = launch_dst_tma_x(reinterpret_cast<const float *>(j == 0 ? zc : R),
                            reinterpret_cast<float *>(wc), g, pp.sop_x, S, gk, st);
     else
-      e = launch_dst<Tc, Arr, Tc, true>(Arr{j == 0 ? zc : R}, wc, g.mx, pp.Lx, nx, g.mx, 0, 0,
-                                        y.px, y.px, twx, S, gk, pp.dst_shift, st);
+      e = launch_dst<Tc, SrcOther<Tc>, Tc, true>(SrcOther<Tc>{{j == 0 ? zc : R}}, wc, g.mx, pp.Lx, nx,
+                                                 g.mx, 0, 0, y.px, y.px, twx, S, gk, pp.dst_shift,
+                                                 st);
     if (e != cudaSuccess) return e;
     if ((e = yz()) != cudaSuccess) return e;
     if (xtc) {

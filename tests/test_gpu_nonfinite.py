@@ -34,7 +34,7 @@ CASES = [(1, 31, 1, 1, 40, "PH"), (1, 1023, 1, 1, 300, "PH"), (2, 7, 15, 1, 9, "
          (2, 255, 63, 1, 33, "PH"), (2, 255, 127, 1, 64, "PH"), (2, 31, 511, 1, 60, "PH"),
          (2, 127, 31, 1, 300, "PH"), (3, 15, 31, 31, 64, "PH"), (1, 255, 1, 1, 64, "Ptheta"),
          (2, 31, 31, 1, 20, "Ptheta"), (2, 127, 127, 1, 64, "Ptheta"),
-         (2, 255, 63, 1, 60, "Ptheta"), (3, 63, 31, 15, 30, "Ptheta")]
+         (2, 255, 63, 1, 60, "Ptheta"), (2, 511, 63, 1, 30, "Ptheta"), (3, 63, 31, 15, 30, "Ptheta")]
 
 
 def _spec(pkg, dim, mx, my, mz, n, prec, precision="mixed"):
