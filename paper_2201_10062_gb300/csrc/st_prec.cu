@@ -89,10 +89,11 @@ struct new_out<SrcOther<Tc>> {
 };
 
 
-// float32 transforms: three 512-thread blocks per SM (at most 40 registers); float64, double-float
-// and the fused Lanczos source (its loads held in registers ahead of the stores): two
+// float32 transforms: three 512-thread blocks per SM (at most 40 registers), or four where the write
+// of the padding would take more than 32; float64, double-float and the fused Lanczos source (its
+// loads held in registers ahead of the stores): two
 template <class Tc, class Src, class Tout, bool XL, int LOGL>
-__global__ void __launch_bounds__(kNTD, (sizeof(Tc) == 4 && !has_fetch<Src>::value) ? 3 : 2)
+__global__ void __launch_bounds__(kNTD, has_fetch<Src>::value || sizeof(Tc) != 4 ? 2 : new_out<Src>::value ? 4 : 3)
     k_dst_space(Src src, Tout *out, int len, long long nlines, int mx, int ld, long long m,
                 int pin, int pout, const Tc *tw, int PB, const State *S, int gk) {
   if (gate_closed(S, gk)) return;
@@ -116,12 +117,14 @@ __global__ void __launch_bounds__(kNTD, (sizeof(Tc) == 4 && !has_fetch<Src>::val
     buf[pp * Ls + fft_pad<Tc>(len + 1)] = cpx<Tc>{Tc(0), Tc(0)};
   }
   // The padding slots of a vector that the pass does not read: an earlier call on non-finite data
-  // may have left 0 x NaN there.  (As values of the write loop below they cost 8 us of 99 at 255^2 x
-  // 256, here 1; compiled into the in-place pass, where they are zero already, 14 of 137 at 511^2 x 128.)
-  if constexpr (XL && new_out<Src>::value) {
-    if (pout > len)
-      for (int l = tid; l < nl; l += kNTD) out[(line0 + l) * pout + len] = Tout(0);
-  }
+  // may have left 0 x NaN there.  The Lanczos pass writes them here (at the end they make it spill,
+  // and as values of its write loop they cost 8 us of 99 at 255^2 x 256), the others at the end (here
+  // they take 38 registers in place of 32, three blocks an SM in place of four: 107 -> 113 us at 511 x
+  // 127 x 365).  The in-place pass has no code for them (14 us of 137 at 511^2 x 128).
+  auto zero_padding = [&]() {
+    if (pout > len && tid < nl) out[(line0 + tid) * pout + len] = Tout(0);
+  };
+  if constexpr (XL && new_out<Src>::value && has_fetch<Src>::value) zero_padding();
   // one work item per (sequence, element): both lines of the pair, stored as one complex value
   // at e+1 and its negative at L-1-e (odd extension).  Index maps avoid divisions: len + 1 =
   // L/2 and PB are powers of two.
@@ -206,6 +209,7 @@ __global__ void __launch_bounds__(kNTD, (sizeof(Tc) == 4 && !has_fetch<Src>::val
       if (la < nl) p[0] = (Tout)(-Z.y * sc);
       if (lb < nl) p[pout] = (Tout)(Z.x * sc);
     }
+    if constexpr (new_out<Src>::value && !has_fetch<Src>::value) zero_padding();
   } else {
     const int pp = tid & (PB - 1), estep = kNTD >> logPB;
     const int la = 2 * pp, lb = la + 1;
