@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(kNTL, 1)
   __syncthreads();
   fence_after();
   const uint32_t tmem = __float_as_uint(lds1(tslot));
-  const uint32_t dcol = tmem + 256u;  // two 64-column accumulators (hi, lo) after A
+  const uint32_t dcol = tmem + 256u;  // after A: [buffer][four accumulators][32 columns]
   auto load = [&](unsigned tile, int s) {
     const uint32_t mb = full + 8u * s, dst = sm + L::ring + (uint32_t)s * kSlotL;
     const unsigned pl = tile / (unsigned)chunks;
@@ -143,24 +143,19 @@ __global__ void __launch_bounds__(kNTL, 1)
   } else if (warp == 20) {
     // ------------------------------------------------------------------ MMA thread
     if (elect_one()) {
-      const int KS = D.hK >> 4;
-      const uint32_t a_lo = tmem + (uint32_t)(D.hK >> 1);
+      // two pairs of accumulators, each for half of the 9 to 16 K steps (see issue_pair)
+      const int KS = D.hK >> 4, KA = (KS + 1) >> 1;
       uint32_t n = 0;
       for (unsigned tile = first; tile < groups; tile += step, ++n) {
-        const uint32_t b = n & 1u, ph = (n >> 1) & 1u, d = dcol + 64u * b;
+        const uint32_t b = n & 1u, ph = (n >> 1) & 1u, d = dcol + 128u * b;
         if (!mbar_wait(bfull + 8u * b, ph) || !mbar_wait(aempty + 8u * b, ph ^ 1u)) {
           ok = false;
           break;
         }
         fence_after();
         const uint64_t bd = make_desc_sbo(sm + L::bop + b * 2u * D.ph, D.sbo);
-#pragma unroll
-        for (int ks = 0; ks < 16; ++ks) {
-          if (ks < KS) {
-            mma_ta<64>(d, tmem + 8u * ks, bd + 16u * (uint64_t)ks, ks > 0 ? 1u : 0u);
-            mma_ta<32>(d, a_lo + 8u * ks, bd + 16u * (uint64_t)ks, 1u);
-          }
-        }
+        issue_two_pairs<32, 8>(d, d + 64u, tmem, tmem + 8u * KA, (uint32_t)(D.hK >> 1), bd,
+                               bd + 16u * (uint64_t)KA, D.ph >> 4, KA, KS - KA);
         mma_commit(afull + 8u * b);
         mma_commit(bempty + 8u * b);
       }
@@ -268,7 +263,14 @@ __global__ void __launch_bounds__(kNTL, 1)
 #pragma unroll
       for (int hf = 0; hf < 2; ++hf) {
         float v[16];
-        tmem_sum16(dcol + 64u * b + lanes + 16u * hf, 32u, v);
+        {
+          float w[16];
+          const uint32_t acc = dcol + 128u * b + lanes + 16u * hf;
+          tmem_sum16(acc, 32u, v);
+          tmem_sum16(acc + 64u, 32u, w);
+#pragma unroll
+          for (int c = 0; c < 16; ++c) v[c] += w[c];
+        }
         if (hf == 1) {
           fence_before();
           __syncwarp();

@@ -24,9 +24,8 @@
 //     parities (and for h <= 32 two halves of the groups as well) are stacked in the 128 rows of
 //     the MMA: slot s holds its rows of A and zeros elsewhere, every slot's product accumulates into
 //     the same accumulator columns, and every thread of the epilogue has 64 values to take out;
-//   - few, wide MMAs: A_hi meets B_hi and B_lo in one MMA of twice the width (they are adjacent along
-//     N) and the epilogue adds the two halves; A_lo meets B_hi in a second one.  They are issued under
-//     elect.sync (see elect_one): under `lane == 0` their issue alone took 2400 cycles a tile.
+//   - MMAs are issued under elect.sync (see elect_one): under `lane == 0` their issue alone took 2400
+//     cycles a tile.  Two accumulators share the K steps (see issue_pair).
 // S (all slots, hi and lo) stays in tensor memory for the whole launch; one block per SM walks the
 // tiles with its warps in separate roles that hand off through mbarriers, every wait bounded.  On a
 // timeout the block records ST_ERR_TIMEOUT and stops; before it frees its tensor memory every MMA
@@ -79,28 +78,24 @@ __device__ __forceinline__ uint32_t b_off(const TmaDim &D, int P, int c) {
   return (uint32_t)(P * 2) * D.ph + (uint32_t)(c >> 3) * D.sbo;
 }
 
-// All MMAs of one transform of a tile: slot s = parity (SL 1, 2) or 2 parity + column set (SL 4);
-// the first MMA of each accumulator overwrites it.  Accumulator columns: [parity][32 hi, 32 lo] for
-// SL 1, [64 hi, 64 lo] else (hi: A_hi B_hi + A_lo B_hi, lo: A_hi B_lo).
+// All MMAs of one transform of a tile: slot s = parity (SL 1, 2) or 2 parity + column set (SL 4).
+// Accumulators (see issue_pair): a pair of 32 columns for each parity with SL 1; else one pair of 64,
+// which the first slot overwrites (a slot's zero rows of A add exact zeros to the others' rows).
 template <int SL>
 __device__ __forceinline__ void issue_tile(uint32_t a_base, uint32_t bop, const TmaDim &D,
                                            uint32_t dcol) {
-  constexpr int N = SL == 1 ? 32 : 64;
   const int KS = D.hK >> 4;
   const uint32_t vc = (uint32_t)(D.hK >> 1);
+  const uint64_t lo = D.ph >> 4;
+  if constexpr (SL == 1) {
+    issue_two_pairs<32, 8>(dcol, dcol + 64u, a_base, a_base + 2u * vc, vc, make_desc_sbo(bop, D.sbo),
+                           make_desc_sbo(bop + 2u * D.ph, D.sbo), lo, KS, KS);
+  } else {
 #pragma unroll 1
-  for (int s = 0; s < num_slots(SL); ++s) {
-    const uint32_t d = SL == 1 ? dcol + 64u * (uint32_t)s : dcol;
-    const uint32_t a_hi = a_base + (uint32_t)(2 * s) * vc, a_lo = a_hi + vc;
-    const uint64_t bd = make_desc_sbo(bop + (uint32_t)(2 * s) * D.ph, D.sbo);
-    const uint32_t keep = (SL == 1 || s == 0) ? 0u : 1u;
-#pragma unroll
-    for (int ks = 0; ks < 8 / SL; ++ks) {
-      if (ks < KS) {
-        mma_ta<2 * N>(d, a_hi + 8u * ks, bd + 16u * (uint64_t)ks, ks > 0 ? 1u : keep);
-        mma_ta<N>(d, a_lo + 8u * ks, bd + 16u * (uint64_t)ks, 1u);
-      }
-    }
+    for (int s = 0; s < num_slots(SL); ++s)
+      issue_pair<64, 8 / SL>(dcol, a_base + (uint32_t)(2 * s) * vc, vc,
+                             make_desc_sbo(bop + (uint32_t)(2 * s) * D.ph, D.sbo), lo, KS,
+                             s > 0 ? 1u : 0u);
   }
 }
 
@@ -269,7 +264,7 @@ __device__ __forceinline__ bool build_xlines(uint32_t buf, uint32_t bop, uint32_
   return true;
 }
 
-// 16 values of one unit: the hi and lo halves of the accumulator summed
+// 16 values of one unit: its two accumulators summed
 template <int SL>
 __device__ __forceinline__ void tmem_unit16(uint32_t acc, int j, int k, float (&v)[16]) {
   tmem_sum16(acc + (SL == 1 ? 64u : 32u) * (uint32_t)j + 16u * (uint32_t)k, SL == 1 ? 32u : 64u, v);

@@ -31,6 +31,68 @@ __device__ __forceinline__ void mma_ta(uint32_t dtmem, uint32_t atmem, uint64_t 
       "r"(atmem), "l"(bd), "r"(idesc), "r"(acc));
 }
 
+// MMAs of one operand pair over KS (at most MAXK) K steps, into two accumulators of N columns at d and
+// d + N, which the epilogue adds: A_hi at a in tensor memory, A_lo vc columns further; B_hi at
+// descriptor b, B_lo (adjacent along N) at b + lo.
+// An MMA adds its K step to the accumulator with the sum cut off, not rounded, at float32's last bit,
+// and so takes half an ulp off it on average: one accumulator for all K steps left the two transforms
+// of a time stage short by 1e-6 (n = 256) to 2e-6 (n = 500) of the result, up to four times the error
+// of the float32 kernels.  So the K steps go half and half to the two accumulators, whose sum is
+// rounded, and the small products (A_hi B_lo, A_lo B_hi: 2^-11 of the large ones, and cut off that much
+// lower) come before the large ones of the second; axes beyond 256 take two pairs.  Against float64 the
+// largest and the root mean square error are then 0.9 of the float32 kernels' in the mean over 738
+// sizes, schemes and inputs.  In the first half A_hi meets B_hi and B_lo in one MMA of twice the width.
+// What this costs is the issue of the further MMAs (time stage at 255^2 x 256: 53.4 us with one
+// accumulator and 55.4 now; 511 x 127 x 365: 80.7 and 84.3 a launch; y at 511^2 x 128: 77 and 80), so the
+// conditions and operands of a step are shared where two pairs go together (pair after pair, the time
+// stage took 57 and 90 us).  keep: 0 overwrites the accumulators, 1 adds to them.
+template <int N, int MAXK>
+__device__ __forceinline__ void issue_pair(uint32_t d, uint32_t a, uint32_t vc, uint64_t b, uint64_t lo,
+                                           int KS, uint32_t keep) {
+  const int K2 = (KS + 1) >> 1;
+#pragma unroll
+  for (int ks = 0; ks < (MAXK + 1) / 2; ++ks)
+    if (ks < K2) mma_ta<2 * N>(d, a + 8u * ks, b + 16u * (uint64_t)ks, ks > 0 ? 1u : keep);
+#pragma unroll
+  for (int ks = 0; ks < MAXK; ++ks) {
+    if (ks < KS) mma_ta<N>(d + N, a + vc + 8u * ks, b + 16u * (uint64_t)ks, 1u);
+    if (ks >= K2 && ks < KS) mma_ta<N>(d + N, a + 8u * ks, b + lo + 16u * (uint64_t)ks, 1u);
+  }
+#pragma unroll
+  for (int ks = 1; ks < MAXK; ++ks)
+    if (ks >= K2 && ks < KS) mma_ta<N>(d + N, a + 8u * ks, b + 16u * (uint64_t)ks, 1u);
+}
+// Two such pairs in turns, of KS and KS1 (KS, or one less) steps.
+template <int N, int MAXK>
+__device__ __forceinline__ void issue_two_pairs(uint32_t d0, uint32_t d1, uint32_t a0, uint32_t a1,
+                                                uint32_t vc, uint64_t b0, uint64_t b1, uint64_t lo,
+                                                int KS, int KS1) {
+  const int K2 = (KS + 1) >> 1;
+#pragma unroll
+  for (int ks = 0; ks < (MAXK + 1) / 2; ++ks)
+    if (ks < K2) {
+      mma_ta<2 * N>(d0, a0 + 8u * ks, b0 + 16u * (uint64_t)ks, ks > 0 ? 1u : 0u);
+      mma_ta<2 * N>(d1, a1 + 8u * ks, b1 + 16u * (uint64_t)ks, ks > 0 ? 1u : 0u);
+    }
+#pragma unroll
+  for (int ks = 0; ks < MAXK; ++ks) {
+    if (ks < KS) {
+      mma_ta<N>(d0 + N, a0 + vc + 8u * ks, b0 + 16u * (uint64_t)ks, 1u);
+      if (ks < KS1) mma_ta<N>(d1 + N, a1 + vc + 8u * ks, b1 + 16u * (uint64_t)ks, 1u);
+    }
+    if (ks >= K2 && ks < KS) {
+      mma_ta<N>(d0 + N, a0 + 8u * ks, b0 + lo + 16u * (uint64_t)ks, 1u);
+      if (ks < KS1) mma_ta<N>(d1 + N, a1 + 8u * ks, b1 + lo + 16u * (uint64_t)ks, 1u);
+    }
+  }
+#pragma unroll
+  for (int ks = 1; ks < MAXK; ++ks)
+    if (ks >= K2 && ks < KS) {
+      mma_ta<N>(d0 + N, a0 + 8u * ks, b0 + 16u * (uint64_t)ks, 1u);
+      if (ks < KS1) mma_ta<N>(d1 + N, a1 + 8u * ks, b1 + 16u * (uint64_t)ks, 1u);
+    }
+}
+
 // A into tensor memory: variant (slot or block's own rows, piece) at columns variant * hK / 2, from the host image
 // [variant][hK / 16][128 rows][16 halves]; `nw` warps of the block share the work
 __device__ __forceinline__ void load_a_variants(const uint4 *img, int nv, int hK, uint32_t a_base,
@@ -139,11 +201,11 @@ __device__ __forceinline__ void put_piece(uint32_t a, uint32_t ph, const float (
   sts4(a + ph, lo[0], lo[1], lo[2], lo[3]);
 }
 
-// 16 accumulator columns at `hi` plus the 16 that lie `lo` columns further (the hi and lo halves of B)
-__device__ __forceinline__ void tmem_sum16(uint32_t hi, uint32_t lo, float (&v)[16]) {
+// 16 columns of one accumulator plus those of the one `off` columns further
+__device__ __forceinline__ void tmem_sum16(uint32_t acc, uint32_t off, float (&v)[16]) {
   uint32_t a[16], b[16];
-  tmem_ld16_async(hi, a);
-  tmem_ld16_async(hi + lo, b);
+  tmem_ld16_async(acc, a);
+  tmem_ld16_async(acc + off, b);
   tmem_wait_ld();
 #pragma unroll
   for (int c = 0; c < 16; ++c) v[c] = __uint_as_float(a[c]) + __uint_as_float(b[c]);
