@@ -38,15 +38,15 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, int K) {
   return d;
 }
 
-// instruction descriptor, kind::f16: D f32, A f16, B f16, both K-major, N = 32, M = 128
-constexpr uint32_t kIdesc = (1u << 4) | ((uint32_t)(kTN >> 3) << 17) | ((uint32_t)(kM >> 4) << 24);
-
-__device__ __forceinline__ void mma_f16(uint32_t dtmem, uint64_t ad, uint64_t bd, uint32_t acc) {
+// kind::f16, D f32, A (tensor memory) and B (shared memory) f16, both K-major, M = 128
+template <int N>
+__device__ __forceinline__ void mma_ta(uint32_t dtmem, uint32_t atmem, uint64_t bd, uint32_t acc) {
+  constexpr uint32_t idesc = (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kM >> 4) << 24);
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(dtmem),
-      "l"(ad), "l"(bd), "r"(kIdesc), "r"(acc));
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(dtmem),
+      "r"(atmem), "l"(bd), "r"(idesc), "r"(acc));
 }
 
 __device__ __forceinline__ void mma_commit(uint32_t mbar) {
@@ -196,30 +196,6 @@ __device__ __forceinline__ SymRow sym_row(const Spec<float> &sp, int k) {
   return r;
 }
 
-// 1/p: theta:  re = (1 - cos x) + tmu (th + (1-th) cos x), im = (-1 + (1-th) tmu) sin x;
-// BDF2: re = (1 - cos x)^2 + tmu, im = -sin x (2 - cos x);  P_theta: 1/(lam_H + lam_Htheta tmu)
-__device__ __forceinline__ float inv_sym(const Spec<float> &sp, const SymRow &r, float tmu) {
-  if (sp.prec == ST_PREC_PTHETA) return 1.0f / (r.a + r.b * tmu);
-  float re, im;
-  if (sp.scheme == ST_THETA) {
-    re = r.a + tmu * r.b;
-    im = (-1.0f + (1.0f - sp.theta) * tmu) * r.c;
-  } else {
-    re = r.a + tmu;
-    im = r.c;
-  }
-  return rsqrtf(re * re + im * im);
-}
-
-__device__ __forceinline__ void mma_f16_ta(uint32_t dtmem, uint32_t atmem, uint64_t bd,
-                                           uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(dtmem),
-      "r"(atmem), "l"(bd), "r"(kIdesc), "r"(acc));
-}
-
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
   asm volatile(
       "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr),
@@ -249,14 +225,6 @@ __device__ __forceinline__ bool group_sync_and(bool v, int id, int nthreads) {
 __device__ __forceinline__ void mbar_expect_tx(uint32_t mbar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(bytes)
                : "memory");
-}
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes,
-                                         uint32_t mbar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
-          "r"(dst),
-      "l"(src), "r"(bytes), "r"(mbar)
-      : "memory");
 }
 
 // tau mu_j of padded column j (x fastest, px = mx + 1 slots a row, m columns in all): the padding

@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(kNTG, 1)
               const uint64_t bd = bdesc + (uint64_t)(((uint32_t)(g - i) * bop) >> 4);
 #pragma unroll 8
               for (int ks = 0; ks < ksteps; ++ks) {
-                mma_f16_ta(d, at + (uint32_t)ks * 8u, bd + (uint64_t)(16 * ks), acc);
+                mma_ta<kTN>(d, at + (uint32_t)ks * 8u, bd + (uint64_t)(16 * ks), acc);
                 acc = 1u;
               }
             }

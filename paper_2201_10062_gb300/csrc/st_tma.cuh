@@ -21,16 +21,6 @@ __device__ __forceinline__ uint64_t make_desc_sbo(uint32_t saddr, uint32_t sbo) 
   return d;
 }
 
-template <int N>
-__device__ __forceinline__ void mma_ta(uint32_t dtmem, uint32_t atmem, uint64_t bd, uint32_t acc) {
-  constexpr uint32_t idesc = (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kM >> 4) << 24);
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(dtmem),
-      "r"(atmem), "l"(bd), "r"(idesc), "r"(acc));
-}
-
 // MMAs of one operand pair over KS (at most MAXK) K steps, into two accumulators of N columns at d and
 // d + N, which the epilogue adds: A_hi at a in tensor memory, A_lo vc columns further; B_hi at
 // descriptor b, B_lo (adjacent along N) at b + lo.
@@ -211,8 +201,11 @@ __device__ __forceinline__ void tmem_sum16(uint32_t acc, uint32_t off, float (&v
   for (int c = 0; c < 16; ++c) v[c] = __uint_as_float(a[c]) + __uint_as_float(b[c]);
 }
 
-// 1/p of row r and column factor tmu for one kind of symbol (0: theta, 1: BDF2, 2: P_theta); the
-// kinds are compiled apart so that the unrolled epilogue stays small
+// 1/p of row r and column factor tmu for one kind of symbol; the kinds are compiled apart so that the
+// unrolled epilogue stays small.
+// 0, theta:  re = (1 - cos x) + tmu (th + (1-th) cos x), im = (-1 + (1-th) tmu) sin x;
+// 1, BDF2:   re = (1 - cos x)^2 + tmu, im = -sin x (2 - cos x);
+// 2, P_theta: 1/(lam_H + lam_Htheta tmu)
 template <int KIND>
 __device__ __forceinline__ float inv_sym_k(const SymRow &r, float omth, float tmu) {
   if (KIND == 2) return 1.0f / (r.a + r.b * tmu);
