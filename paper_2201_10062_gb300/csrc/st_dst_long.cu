@@ -327,6 +327,21 @@ __global__ void __launch_bounds__(kNTL, 1)
   }
 }
 
+// Operand image of 8 S_len: [parity][half of the rows][hi, lo][K step][128 rows][16], zeros past the axis.  A
+// block per K step and quarter, a thread per row.
+__global__ void __launch_bounds__(kM) k_image_long(const __grid_constant__ SinePieces S, int len, uint4 *img) {
+  const int KS = gridDim.x, ks = blockIdx.x, p = blockIdx.y, row = threadIdx.x;
+  const int h = (len + 1) >> 1, r = (p & 1) * 128 + row;
+  uint4 hi[2], lo[2];
+  image_row(S, len, h, r < h ? 2 * r + 1 + (p >> 1) : len + 1, ks * 16, hi, lo);
+  uint4 *q = img + ((size_t)(2 * p * KS + ks) * kM + row) * 2;
+  q[0] = hi[0];
+  q[1] = hi[1];
+  q += (size_t)KS * kM * 2;
+  q[0] = lo[0];
+  q[1] = lo[1];
+}
+
 template <int KIND>
 cudaError_t launch_long(const float *in, float *out, int len, long long cols, long long planes,
                         long long rs, long long ps, const unsigned short *img, const Geom &g,
@@ -362,26 +377,9 @@ size_t dst_long_image_halves(int len) {
   return (size_t)4 * 2 * kM * (((len + 1) / 2 + 15) & ~15);
 }
 
-// Host: 8 S_len, [parity][half of the rows][hi, lo][K step][128 rows][16], zeros past the axis.
-void dst_long_build_image(int len, unsigned short *out) {
-  const int h = (len + 1) / 2, hK = (h + 15) & ~15;
-  const SinePieces S(len);
-  const size_t piece = (size_t)kM * hK;
-  for (size_t i = 0; i < dst_long_image_halves(len); ++i) out[i] = 0;
-  for (int P = 0; P < 2; ++P)
-    for (int r = 0; r < h; ++r) {
-      const int k = 2 * r + 1 + P;
-      if (k > len) continue;
-      unsigned short *q = out + (size_t)(2 * P + (r >> 7)) * 2 * piece + (size_t)(r & 127) * 16;
-      int a = 0;
-      for (int t = 0; t < h; ++t) {
-        a += k;
-        if (a >= S.period) a -= S.period;
-        const size_t off = (size_t)(t >> 4) * kM * 16 + (t & 15);
-        q[off] = S.hi[a];
-        q[piece + off] = S.lo[a];
-      }
-    }
+cudaError_t dst_long_build_image(int len, unsigned short *img) {
+  k_image_long<<<dim3(long_dim(len).hK >> 4, 4), kM>>>(SinePieces(len), len, (uint4 *)img);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_dst_long_y(const float *in, float *out, const Geom &g, const unsigned short *img,

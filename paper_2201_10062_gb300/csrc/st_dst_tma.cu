@@ -932,6 +932,23 @@ __global__ void __launch_bounds__(kNTT, 1)
   }
 }
 
+// Operand image of 8 S_len: rows of each slot (odd k = 2r + 1 for parity 0, even k = 2r + 2 for parity 1)
+// in the slot's rows of the MMA, zeros elsewhere, hi and lo fp16 pieces: [slot][piece][K step][row][16].
+// A block per K step and slot, a thread per row.
+__global__ void __launch_bounds__(kM) k_image_tma(const __grid_constant__ SinePieces S, int len, int SL,
+                                                  uint4 *img) {
+  const int h = (len + 1) >> 1, KS = gridDim.x, ks = blockIdx.x, s = blockIdx.y, row = threadIdx.x;
+  const int P = SL == 4 ? s >> 1 : s, r = row - (SL == 1 ? 0 : s * (kM / SL));
+  uint4 hi[2], lo[2];
+  image_row(S, len, h, r >= 0 && r < h ? 2 * r + 1 + P : len + 1, ks * 16, hi, lo);
+  uint4 *q = img + ((size_t)(2 * s * KS + ks) * kM + row) * 2;
+  q[0] = hi[0];
+  q[1] = hi[1];
+  q += (size_t)KS * kM * 2;
+  q[0] = lo[0];
+  q[1] = lo[1];
+}
+
 // ---------------------------------------------------------------- host
 constexpr uint32_t kSmemMax = 227u * 1024u;
 
@@ -1033,30 +1050,10 @@ size_t dst_tma_image_halves(int len) {
   return (size_t)2 * num_slots(SL) * kM * hK;
 }
 
-// Host: 8 S_len, rows of each slot (odd k = 2r + 1 for parity 0, even k = 2r + 2 for parity 1) in
-// the slot's rows of the MMA, zeros elsewhere, hi and lo fp16 pieces: [slot][piece][K step][row][16].
-void dst_tma_build_image(int len, unsigned short *out) {
-  const int SL = slots_for(len), h = (len + 1) / 2, hK = (h + 15) & ~15;
-  const SinePieces S(len);
-  const size_t piece = (size_t)kM * hK;
-  for (size_t i = 0; i < dst_tma_image_halves(len); ++i) out[i] = 0;
-  for (int s = 0; s < num_slots(SL); ++s) {
-    const int P = SL == 4 ? s >> 1 : s;
-    const int row0 = SL == 1 ? 0 : s * (kM / SL);
-    for (int r = 0; r < h; ++r) {
-      const int k = 2 * r + 1 + P;
-      if (k > len) continue;
-      unsigned short *q = out + (size_t)(2 * s) * piece + (size_t)(row0 + r) * 16;
-      int a = 0;
-      for (int t = 0; t < h; ++t) {
-        a += k;
-        if (a >= S.period) a -= S.period;
-        const size_t off = (size_t)(t >> 4) * kM * 16 + (t & 15);
-        q[off] = S.hi[a];
-        q[piece + off] = S.lo[a];
-      }
-    }
-  }
+cudaError_t dst_tma_build_image(int len, unsigned short *img) {
+  const int SL = slots_for(len), hK = ((len + 1) / 2 + 15) & ~15;
+  k_image_tma<<<dim3(hK >> 4, num_slots(SL)), kM>>>(SinePieces(len), len, SL, (uint4 *)img);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_dst_tma_x(const float *in, float *out, const Geom &g, const unsigned short *img,

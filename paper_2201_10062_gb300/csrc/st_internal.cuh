@@ -392,10 +392,10 @@ bool device_closed(int dev);
 
 // Tensor-core DSTs on padded float32 vectors (st_dst_tma.cu).  dst_tma_supported: the axis length
 // has a tile shape (16..256); images: the fp16 operand image of S_len the kernels load into tensor
-// memory, in halves, and its host builder.
+// memory, in halves, and the launch that fills it (device memory, default stream).
 bool dst_tma_supported(int len);
 size_t dst_tma_image_halves(int len);
-void dst_tma_build_image(int len, unsigned short *out);
+cudaError_t dst_tma_build_image(int len, unsigned short *img);
 // time DST, 1/p scaling with <v, P^-1 v> (and the MINRES scalar step of tmode), time DST, in place
 cudaError_t launch_time_tma(float *data, const Geom &g, const Spec<float> &sp,
                             const unsigned short *img, State *S, int tmode, double *partials,
@@ -415,7 +415,8 @@ int time_tc_grid();
 // data, exact float32 accumulation per digit group; k_time_tcd)
 bool time_tcd_supported(int n);
 size_t time_tcd_bytes(int n);
-int time_tcd_build(int n, unsigned char *out);  // returns the scale exponent of the digits
+// fills the image (device memory, default stream), returns the scale exponent of the digits
+int time_tcd_build(int n, unsigned char *img, cudaError_t *err);
 // scratch: an N-vector of double-floats that overlaps neither data nor anything the stage reads
 cudaError_t launch_time_tcd(dd *data, dd *scratch, const Geom &g, const Spec<dd> &sp,
                             const unsigned char *img, int eS, State *S, int tmode,
@@ -423,7 +424,7 @@ cudaError_t launch_time_tcd(dd *data, dd *scratch, const Geom &g, const Spec<dd>
 // axes of 257 to 512 points (st_dst_long.cu): out of place, for y, z and the time stage (there and back)
 bool dst_long_supported(int len);
 size_t dst_long_image_halves(int len);
-void dst_long_build_image(int len, unsigned short *out);
+cudaError_t dst_long_build_image(int len, unsigned short *img);
 cudaError_t launch_dst_long_y(const float *in, float *out, const Geom &g, const unsigned short *img,
                               State *S, int gk, cudaStream_t st);
 cudaError_t launch_dst_long_z(const float *in, float *out, const Geom &g, const unsigned short *img,

@@ -818,89 +818,67 @@ int build_tables(st_handle *h) {
   for (size_t i = o_mux; i < nd; ++i) hf[i - o_mux] = (float)hd[i];
   const size_t bytes_d = nd * sizeof(double);
   const size_t bytes_f = hf.size() * sizeof(float);
-  // fp16 S_n image for the tensor-core time kernel (mixed precision, supported n)
-  std::vector<unsigned short> sop;
+  // Operand images of the tensor-core transforms (mixed precision, supported lengths), in halves; kernels
+  // fill them below.  The time axis: n up to 256, or 257 to 512 (which the P_theta paths with varying a
+  // do not use).
   const char *no_tc = std::getenv("ST_DISABLE_TENSOR_CORES");
-  const bool use_tc = p.precision == ST_MIXED && !(no_tc && no_tc[0] == '1');
-  bool long_tc = false;
-  if (use_tc && tc_time_ok(g)) {
-    sop.resize(dst_tma_image_halves(n));
-    dst_tma_build_image(n, sop.data());
-  } else if (use_tc && tc_long_ok(g)) {
-    // 256 < n <= 512, in the same slot of the table allocation
-    sop.resize(dst_long_image_halves(n));
-    dst_long_build_image(n, sop.data());
-    long_tc = true;
-  }
+  const bool tc_off = no_tc && no_tc[0] == '1';
+  const bool use_tc = p.precision == ST_MIXED && !tc_off;
+  const bool pcr = p.prec == ST_PREC_PTHETA && p.a_nodal != nullptr && g.dim == 1;
+  const bool long_tc = use_tc && tc_long_ok(g) && !pcr && !cheb;
+  const size_t sop = use_tc && tc_time_ok(g) ? dst_tma_image_halves(n)
+                     : long_tc               ? dst_long_image_halves(n)
+                                             : 0;
   const size_t o_sop = (bytes_d + bytes_f + 255) / 256 * 256;
   // double-float copies of the face coefficients
   std::vector<df> cdf(cx.size() + cy.size() + cz.size());
   for (size_t i = 0; i < cx.size(); ++i) cdf[i] = df_of_double(cx[i]);
   for (size_t i = 0; i < cy.size(); ++i) cdf[cx.size() + i] = df_of_double(cy[i]);
   for (size_t i = 0; i < cz.size(); ++i) cdf[cx.size() + cy.size() + i] = df_of_double(cz[i]);
-  const size_t o_cdf = (o_sop + sop.size() * sizeof(unsigned short) + 255) / 256 * 256;
-  // fp16 S_my / S_mz images for the tensor-core y- and z-DSTs (mixed precision, supported lengths)
-  std::vector<unsigned short> sopy, sopz, sopx;
+  const size_t o_cdf = (o_sop + sop * sizeof(unsigned short) + 255) / 256 * 256;
   const bool long_y = use_tc && tc_ly_ok(g), long_z = use_tc && tc_lz_ok(g);
-  if (use_tc && tc_y_ok(g)) {
-    sopy.resize(dst_tma_image_halves(g.my));
-    dst_tma_build_image(g.my, sopy.data());
-  } else if (long_y) {
-    sopy.resize(dst_long_image_halves(g.my));
-    dst_long_build_image(g.my, sopy.data());
-  }
-  if (use_tc && tc_z_ok(g)) {
-    sopz.resize(dst_tma_image_halves(g.mz));
-    dst_tma_build_image(g.mz, sopz.data());
-  } else if (long_z) {
-    sopz.resize(dst_long_image_halves(g.mz));
-    dst_long_build_image(g.mz, sopz.data());
-  }
-  // and S_mx for the tensor-core x-DST of the last spatial pass
-  if (use_tc && tc_x_ok(g)) {
-    sopx.resize(dst_tma_image_halves(g.mx));
-    dst_tma_build_image(g.mx, sopx.data());
-  }
+  const size_t sopy = use_tc && tc_y_ok(g) ? dst_tma_image_halves(g.my)
+                      : long_y             ? dst_long_image_halves(g.my)
+                                           : 0;
+  const size_t sopz = use_tc && tc_z_ok(g) ? dst_tma_image_halves(g.mz)
+                      : long_z             ? dst_long_image_halves(g.mz)
+                                           : 0;
+  const size_t sopx = use_tc && tc_x_ok(g) ? dst_tma_image_halves(g.mx) : 0;
   const size_t o_sopy = (o_cdf + cdf.size() * sizeof(df) + 255) / 256 * 256;
-  const size_t o_sopz = (o_sopy + sopy.size() * sizeof(unsigned short) + 255) / 256 * 256;
-  const size_t o_sopx = (o_sopz + sopz.size() * sizeof(unsigned short) + 255) / 256 * 256;
+  const size_t o_sopz = (o_sopy + sopy * sizeof(unsigned short) + 255) / 256 * 256;
+  const size_t o_sopx = (o_sopz + sopz * sizeof(unsigned short) + 255) / 256 * 256;
   // double-float copies of the spectral tables and twiddles for the float64 preconditioner's
   // double-float engine (each value split exactly: hi the nearest float, lo the rest)
   std::vector<dd> hdd(nd - o_mux);
   for (size_t i = o_mux; i < nd; ++i) hdd[i - o_mux] = dd(hd[i]);
-  const size_t o_dd = (o_sopx + sopx.size() * sizeof(unsigned short) + 255) / 256 * 256;
+  const size_t o_dd = (o_sopx + sopx * sizeof(unsigned short) + 255) / 256 * 256;
   // integer-digit image of S_n for the float64 path's tensor-core time stage (double-float
   // engine, P_H / P-hat and constant-coefficient P_theta)
-  std::vector<unsigned char> sdig;
+  const bool sdig = p.precision == ST_FP64 && time_tcd_supported(n) && !tc_off && !pcr && !cheb;
   int sdig_e = 0;
-  if (p.precision == ST_FP64 && time_tcd_supported(n) && !(no_tc && no_tc[0] == '1')) {
-    sdig.resize(time_tcd_bytes(n));
-    sdig_e = time_tcd_build(n, sdig.data());
-  }
   const size_t o_dig = (o_dd + hdd.size() * sizeof(dd) + 255) / 256 * 256;
-  const size_t bytes = o_dig + sdig.size();
+  const size_t bytes = o_dig + (sdig ? time_tcd_bytes(n) : 0);
   ST_TRY(cudaMalloc(&h->tables, bytes));
   ST_TRY(cudaMemcpy(h->tables, hd.data(), bytes_d, cudaMemcpyHostToDevice));
   ST_TRY(cudaMemcpy((char *)h->tables + bytes_d, hf.data(), bytes_f, cudaMemcpyHostToDevice));
-  if (!sop.empty())
-    ST_TRY(cudaMemcpy((char *)h->tables + o_sop, sop.data(), sop.size() * sizeof(unsigned short),
-                      cudaMemcpyHostToDevice));
+  auto image = [&](size_t halves, bool lng, int len, size_t off) -> cudaError_t {
+    unsigned short *q = reinterpret_cast<unsigned short *>((char *)h->tables + off);
+    if (halves == 0) return cudaSuccess;
+    return lng ? dst_long_build_image(len, q) : dst_tma_build_image(len, q);
+  };
+  ST_TRY(image(sop, long_tc, n, o_sop));
+  ST_TRY(image(sopy, long_y, g.my, o_sopy));
+  ST_TRY(image(sopz, long_z, g.mz, o_sopz));
+  ST_TRY(image(sopx, false, g.mx, o_sopx));
   ST_TRY(cudaMemcpy((char *)h->tables + o_cdf, cdf.data(), cdf.size() * sizeof(df),
                     cudaMemcpyHostToDevice));
-  if (!sopy.empty())
-    ST_TRY(cudaMemcpy((char *)h->tables + o_sopy, sopy.data(),
-                      sopy.size() * sizeof(unsigned short), cudaMemcpyHostToDevice));
-  if (!sopz.empty())
-    ST_TRY(cudaMemcpy((char *)h->tables + o_sopz, sopz.data(),
-                      sopz.size() * sizeof(unsigned short), cudaMemcpyHostToDevice));
-  if (!sopx.empty())
-    ST_TRY(cudaMemcpy((char *)h->tables + o_sopx, sopx.data(),
-                      sopx.size() * sizeof(unsigned short), cudaMemcpyHostToDevice));
   ST_TRY(cudaMemcpy((char *)h->tables + o_dd, hdd.data(), hdd.size() * sizeof(dd),
                     cudaMemcpyHostToDevice));
-  if (!sdig.empty())
-    ST_TRY(cudaMemcpy((char *)h->tables + o_dig, sdig.data(), sdig.size(),
-                      cudaMemcpyHostToDevice));
+  if (sdig) {
+    cudaError_t e = cudaSuccess;
+    sdig_e = time_tcd_build(n, (unsigned char *)h->tables + o_dig, &e);
+    ST_TRY(e);
+  }
   const double *D = (const double *)h->tables;
   const float *F = (const float *)((const char *)h->tables + bytes_d) - o_mux;
   h->g.cx = D + o_cx;
@@ -951,17 +929,17 @@ int build_tables(st_handle *h) {
     pp.cheb_work = cbase + cb;
   }
   const unsigned short *sop_img =
-      (sop.empty() || pp.pcr || pp.cheb) ? nullptr
+      (sop == 0 || pp.pcr || pp.cheb) ? nullptr
                               : reinterpret_cast<const unsigned short *>((const char *)h->tables + o_sop);
   // the P_theta paths with varying a transform time alone (no scaling) on the tensor cores
-  pp.sop_t1 = (!sop.empty() && !long_tc && (pp.pcr || pp.cheb))
+  pp.sop_t1 = (sop != 0 && !long_tc && (pp.pcr || pp.cheb))
                   ? reinterpret_cast<const unsigned short *>((const char *)h->tables + o_sop)
                   : nullptr;
   pp.sop = long_tc ? nullptr : sop_img;
   pp.sop_long = long_tc ? sop_img : nullptr;
-  pp.sop_y = sopy.empty() ? nullptr
+  pp.sop_y = sopy == 0 ? nullptr
                           : reinterpret_cast<const unsigned short *>((const char *)h->tables + o_sopy);
-  pp.sop_z = sopz.empty() ? nullptr
+  pp.sop_z = sopz == 0 ? nullptr
                           : reinterpret_cast<const unsigned short *>((const char *)h->tables + o_sopz);
   // a long axis' image serves its own kernels
   pp.sop_ly = long_y ? pp.sop_y : nullptr;
@@ -975,7 +953,7 @@ int build_tables(st_handle *h) {
   // for the FFT at 255^2 x 256); st_autotune times both, and ST_X_TENSOR_CORES=0 starts a handle
   // with the FFT.  The P_theta paths with varying a run their x passes through the Chebyshev and
   // PCR kernels.
-  h->tc_x_img = (sopx.empty() || pp.pcr)
+  h->tc_x_img = (sopx == 0 || pp.pcr)
                     ? nullptr
                     : reinterpret_cast<const unsigned short *>((const char *)h->tables + o_sopx);
   {
@@ -1001,7 +979,7 @@ int build_tables(st_handle *h) {
   pp.twx_dd = DD + o_twx;
   pp.twy_dd = DD + o_twy;
   pp.twz_dd = DD + o_twz;
-  pp.sdig = sdig.empty() ? nullptr : (const unsigned char *)h->tables + o_dig;
+  pp.sdig = sdig ? (const unsigned char *)h->tables + o_dig : nullptr;
   pp.sdig_e = sdig_e;
   h->tc_dig_img = pp.sdig;
   // the float64 P_H / P-hat preconditioner runs its transforms in double-float unless

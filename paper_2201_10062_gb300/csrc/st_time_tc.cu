@@ -506,6 +506,31 @@ __global__ void __launch_bounds__(kNTG, 1)
   }
 }
 
+// The digits of sqrt(2/(n+1)) sin(pi a/(n+1)) 2^eS for a = 0 .. 2 n + 1
+struct SineDigits {
+  short d[kDg][2 * 257];
+};
+
+// The digit image of S_n for k_time_tcd: piece (parity P, digit i) at index P * 7 + i, the rows r of
+// parity P (k = 2r+1 or 2r+2) by K = hK folded columns, canonical K-major fp16; the digits of S 2^eS
+// (integers, |.| <= 2^7) were taken in float64, where they are exact.  A block per digit, parity and
+// eight rows, a thread per row and eight columns (filled by the host and copied, the image took 0.2 to
+// 0.5 ms of a handle's set-up).
+__global__ void k_image_digits(const __grid_constant__ SineDigits S, int n, uint4 *img) {
+  const int h = (n + 1) >> 1, hK = 8 * blockDim.y, dg = blockIdx.x, P = blockIdx.y;
+  const int r = 8 * blockIdx.z + threadIdx.x, t0 = 8 * threadIdx.y, k = 2 * r + 1 + P;
+  uint32_t w[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int a = (int)((unsigned)(k * (t0 + j + 1)) % (unsigned)(2 * (n + 1)));
+    const int v = r < h && k <= n && t0 + j < h ? S.d[dg][a] : 0;
+    const __half_raw x = __int2half_rn(v);
+    w[j] = x.x;
+  }
+  img[((size_t)(P * kDg + dg) * kM * hK * 2 + canon_off(r, t0, hK)) / 16] =
+      make_uint4(w[0] | w[1] << 16, w[2] | w[3] << 16, w[4] | w[5] << 16, w[6] | w[7] << 16);
+}
+
 }  // namespace
 
 // Multiples of 32 up to 256, and every n from 129 to 256 (ceil(n/2) folded rows, padded to the MMA K
@@ -523,51 +548,31 @@ bool time_tcd_supported(int n) {
 
 size_t time_tcd_bytes(int n) { return (size_t)2 * kDg * kM * (size_t)tcd_hk(n) * 2; }
 
-// Host: the digit image of S_n for k_time_tcd: piece (parity P, digit i) at index P * 7 + i, the
-// rows r of parity P (k = 2r+1 or 2r+2) by K = hK folded columns, canonical K-major fp16; the
-// digits of S 2^eS (integers, |.| <= 2^7) are taken in float64, where they are exact.
-// Returns eS.
-int time_tcd_build(int n, unsigned char *out) {
-  const int h = (n + 1) / 2, hK = tcd_hk(n);
+int time_tcd_build(int n, unsigned char *img, cudaError_t *err) {
   const double PI = 3.14159265358979323846;
   const double sn = std::sqrt(2.0 / (n + 1));
-  // S_{k,t} = sn sin(pi a / (n+1)) with a = k t mod 2 (n+1): the digits of these 2 (n+1) values.  The
-  // largest entry over k <= n, t <= h is taken from them as well.
+  // S_{k,t} = sn sin(pi a / (n+1)) with a = k t mod 2 (n+1), and every a = 1..n occurs (t = 1)
   const int period = 2 * (n + 1);
   std::vector<double> val(period);
-  for (int a = 0; a < period; ++a) val[a] = sn * std::sin(PI * (double)a / (n + 1));
   double smax = 0.0;
-  for (int k = 1; k <= n; ++k)
-    for (int t = 1, a = k; t <= h; ++t, a = (a + k) % period) smax = std::fmax(smax, std::fabs(val[a]));
+  for (int a = 0; a < period; ++a) {
+    val[a] = sn * std::sin(PI * (double)a / (n + 1));
+    smax = std::fmax(smax, std::fabs(val[a]));
+  }
   int E = 0;
   std::frexp(smax, &E);
   const int eS = 7 - E;  // smax 2^eS in [2^6, 2^7)
-  std::vector<unsigned short> dig((size_t)period * kDg);
+  SineDigits S;
   for (int a = 0; a < period; ++a) {
     double v = std::ldexp(val[a], eS);
     for (int dg = 0; dg < kDg; ++dg) {
       const double q = std::nearbyint(v);
       v = (v - q) * 128.0;
-      const __half_raw raw = __float2half_rn((float)q);
-      dig[(size_t)a * kDg + dg] = raw.x;
+      S.d[dg][a] = (short)q;
     }
   }
-  unsigned short *o = reinterpret_cast<unsigned short *>(out);
-  const size_t piece = (size_t)kM * hK;  // halves
-  for (size_t i = 0; i < time_tcd_bytes(n) / 2; ++i) o[i] = 0;
-  for (int P = 0; P < 2; ++P)
-    for (int r = 0; r < h; ++r) {
-      const int k = (P == 0) ? 2 * r + 1 : 2 * r + 2;
-      if (k > n) continue;
-      int a = 0;
-      for (int t = 0; t < h; ++t) {
-        a += k;
-        if (a >= period) a -= period;
-        const size_t off = canon_off(r, t, hK) / 2;
-        for (int dg = 0; dg < kDg; ++dg)
-          o[(size_t)(P * kDg + dg) * piece + off] = dig[(size_t)a * kDg + dg];
-      }
-    }
+  k_image_digits<<<dim3(kDg, 2, kM / 8), dim3(8, tcd_hk(n) >> 3)>>>(S, n, (uint4 *)img);
+  *err = cudaGetLastError();
   return eS;
 }
 

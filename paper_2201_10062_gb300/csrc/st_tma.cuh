@@ -5,7 +5,6 @@
 #include <cuda.h>
 
 #include <cmath>
-#include <vector>
 
 #include "st_tc.cuh"
 
@@ -223,23 +222,48 @@ __device__ __forceinline__ float inv_sym_k(const SymRow &r, float omth, float tm
 }
 
 // ---------------------------------------------------------------- host
-// The hi and lo fp16 pieces of 8 sqrt(2/(len+1)) sin(pi a/(len+1)) for a = 0 .. 2 (len+1) - 1: every entry
-// of the operand images is one of these (S_{k,t} has a = k t mod 2 (len+1)).
+// The hi (low half) and lo fp16 pieces of 8 sqrt(2/(len+1)) sin(pi a/(len+1)) for a = 0 .. len: every
+// entry of the operand images is one of these or its negative (S_{k,t} has a = k t mod 2 (len+1)).  They
+// go to the kernels that fill the images as an argument: filled by the host and copied, the images of
+// a handle took 0.1 to 0.3 ms of its set-up.
 struct SinePieces {
-  std::vector<unsigned short> hi, lo;
-  int period;
-  explicit SinePieces(int len) : hi(2 * (len + 1)), lo(2 * (len + 1)), period(2 * (len + 1)) {
+  uint32_t v[513];
+  explicit SinePieces(int len) {
     const double PI = 3.14159265358979323846, sn = std::sqrt(2.0 / (len + 1));
-    for (int a = 0; a < period; ++a) {
-      const double v = kSScale * sn * std::sin(PI * (double)a / (len + 1));
-      const __half h = __float2half_rn((float)v);
-      const __half l = __float2half_rn((float)(v - (double)__half2float(h)));
+    for (int a = 0; a <= len; ++a) {
+      const double x = kSScale * sn * std::sin(PI * (double)a / (len + 1));
+      const __half h = __float2half_rn((float)x);
+      const __half l = __float2half_rn((float)(x - (double)__half2float(h)));
       const __half_raw rh = h, rl = l;
-      hi[a] = rh.x;
-      lo[a] = rl.x;
+      v[a] = (uint32_t)rh.x | (uint32_t)rl.x << 16;
     }
   }
 };
+
+// Pieces of row k, folded columns t0 .. t0 + 15 (0-based; zeros from h on, and for k past len): the 16
+// halves of hi and of lo as they stand in an image.
+__device__ __forceinline__ void image_row(const SinePieces &S, int len, int h, int k, int t0, uint4 (&hi)[2],
+                                          uint4 (&lo)[2]) {
+  uint32_t w[16];
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    const int t = t0 + j;
+    int a = (int)((unsigned)(k * (t + 1)) % (unsigned)(2 * (len + 1)));
+    uint32_t flip = 0u;
+    if (a > len) {
+      a -= len + 1;
+      flip = 0x80008000u;
+    }
+    w[j] = k <= len && t < h ? S.v[a] ^ flip : 0u;
+  }
+  auto lo2 = [&](int j) { return __byte_perm(w[j], w[j + 1], 0x5410); };
+  auto hi2 = [&](int j) { return __byte_perm(w[j], w[j + 1], 0x7632); };
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    hi[q] = make_uint4(lo2(8 * q), lo2(8 * q + 2), lo2(8 * q + 4), lo2(8 * q + 6));
+    lo[q] = make_uint4(hi2(8 * q), hi2(8 * q + 2), hi2(8 * q + 4), hi2(8 * q + 6));
+  }
+}
 
 typedef CUresult (*EncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
                              const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
