@@ -1449,18 +1449,23 @@ struct Knobs {
   int tc_dd;                // 1: the double-float engine's time stage runs on the tensor cores
 };
 std::mutex g_tune_mu;
-std::map<std::tuple<int, int, int, int, int, int, int>, Knobs> g_tune_cache;
+std::map<std::tuple<int, int, int, int, int, int, int, int>, Knobs> g_tune_cache;
 }  // namespace
 
 int st_autotune(st_handle *h, int reps) {
   if (!h || reps < 1 || reps > 100) return ST_ERR_ARG;
   ST_ENTER(h);
   const bool fp32 = h->mixed;
+  // What selects the code that is timed: the shape, the engines and images of the handle, and what the
+  // stencil is compiled for (one coefficient or one a face, the weights of the time scheme).
+  const int weights = h->g.scheme != ST_THETA ? 3 : h->g.theta == 0.5 ? 0 : h->g.theta == 1.0 ? 1 : 2;
   const auto key = std::make_tuple(h->g.dim, h->g.mx, h->g.my, h->g.mz, h->g.n, (int)fp32,
                                    (h->tc_time_img ? 1 : 0) + (h->pp.pcr ? 2 : 0) +
                                        (h->pp.cheb ? 4 : 0) + (h->tc_y_img ? 8 : 0) +
                                        (h->tc_z_img ? 16 : 0) + (h->tc_dig_img ? 32 : 0) +
-                                       (h->tc_x_img ? 64 : 0));
+                                       (h->tc_x_img ? 64 : 0) + (h->pp.sop_long ? 128 : 0) +
+                                       (h->pp.sop_ly ? 256 : 0) + (h->pp.sop_lz ? 512 : 0),
+                                   2 * weights + (h->g.c_uniform ? 1 : 0));
   auto apply_engines = [&](const Knobs &k) {
     h->pp.sop = k.tc_time ? h->tc_time_img : nullptr;
     h->pp.sop_y = k.tc_y ? h->tc_y_img : nullptr;
