@@ -40,7 +40,7 @@ constexpr int kNT = 256;
 // output: the line length len, or len + 1 in the padded layout, whose last slot is set to zero in an
 // output that is not the source).
 // XL = false: lines are columns of planes: line l = k*mx + i starts at k*m + i and its elements are
-// `ld` apart; columns i with i mod pin >= pout are left alone (the padding columns of z lines: the
+// `ld` apart; columns i with i mod pin >= pout (pin a power of two then) are left alone (the padding columns of z lines: the
 // two lines of a packed pair leave rounding in each other, and the padding stays exactly zero).  A block owns 2*PB consecutive lines (PB complex sequences, line
 // 2p in the real part and line 2p+1 in the imaginary part), loads them coalesced into shared
 // memory as odd extensions, runs in-place Stockham passes and writes the sine coefficients.
@@ -180,12 +180,12 @@ __global__ void __launch_bounds__(kNTD, has_fetch<Src>::value || sizeof(Tc) != 4
     if (la < nl) {
       const int l = (int)line0 + la;
       const int k = l / mx, i = l - k * mx;
-      if (pin == pout || i % pin < pout) ia = (long long)k * m + i;
+      if (pin == pout || (i & (pin - 1)) < pout) ia = (long long)k * m + i;
     }
     if (lb < nl) {
       const int l = (int)line0 + lb;
       const int k = l / mx, i = l - k * mx;
-      if (pin == pout || i % pin < pout) ib = (long long)k * m + i;
+      if (pin == pout || (i & (pin - 1)) < pout) ib = (long long)k * m + i;
     }
     cpx<Tc> *bq = buf + pp * Ls;
     for (int e = tid >> logPB; e < len; e += estep) {
@@ -217,12 +217,12 @@ __global__ void __launch_bounds__(kNTD, has_fetch<Src>::value || sizeof(Tc) != 4
     if (la < nl) {
       const int l = (int)line0 + la;
       const int k = l / mx, i = l - k * mx;
-      if (pin == pout || i % pin < pout) pa = out + (long long)k * m + i;
+      if (pin == pout || (i & (pin - 1)) < pout) pa = out + (long long)k * m + i;
     }
     if (lb < nl) {
       const int l = (int)line0 + lb;
       const int k = l / mx, i = l - k * mx;
-      if (pin == pout || i % pin < pout) pb = out + (long long)k * m + i;
+      if (pin == pout || (i & (pin - 1)) < pout) pb = out + (long long)k * m + i;
     }
     const cpx<Tc> *bq = buf + pp * Ls;
     for (int e = tid >> logPB; e < len; e += estep) {
