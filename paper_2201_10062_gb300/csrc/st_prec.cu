@@ -315,7 +315,8 @@ __device__ void time_dst_tile(Tc *X, Tc *Y, const Tc *sintab, int n, int J) {
 template <class Tc, int KT, int JT>
 __global__ void __launch_bounds__(kNT)
     k_time(const Tc *data, Tc *out, int n, long long m, int mx, int px, int J, Spec<Tc> sp,
-           State *S, int tmode, int tkind, double *__restrict__ partials, int gk) {
+           State *S, int tmode, int tkind, double *__restrict__ partials, int gk, int ox,
+           long long mo) {
   __shared__ double red[32];
   if (gate_closed(S, gk)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -369,7 +370,13 @@ __global__ void __launch_bounds__(kNT)
   } else {
     for (int idx = tid; idx < n * J; idx += kNT) {
       const int t = idx / J, c = idx - t * J;
-      if (c < Je) out[(long long)t * m + j0 + c] = Y[idx];
+      if (c >= Je) continue;
+      if (ox == px) {
+        out[(long long)t * m + j0 + c] = Y[idx];
+      } else {  // into a contiguous vector (mo a level) without the padding
+        const unsigned j = (unsigned)j0 + (unsigned)c, jy = j / (unsigned)px, jx = j - jy * (unsigned)px;
+        if (jx < (unsigned)mx) out[(long long)t * mo + (long long)jy * mx + jx] = Y[idx];
+      }
     }
   }
   if (tmode != TM_NONE) {
@@ -794,7 +801,7 @@ int time_J(int n) {
 template <class Tc>
 cudaError_t launch_time(Tc *data, const Geom &g, const Spec<Tc> &sp, State *S, int tmode,
                         int tkind, double *partials, int gk, int Jover, cudaStream_t st,
-                        Tc *out = nullptr) {
+                        Tc *out = nullptr, bool contiguous = false) {
   const int J = Jover > 0 ? Jover : time_J<Tc>(g.n);
   const size_t sm = time_smem<Tc>(g.n, J);
   const Lay y = lay<Tc>(g);
@@ -805,7 +812,8 @@ cudaError_t launch_time(Tc *data, const Geom &g, const Spec<Tc> &sp, State *S, i
   if (e != cudaSuccess) return e;
   prof_begin(KC_TIME, st);
   kern<<<(unsigned)blocks, kNT, sm, st>>>(data, out ? out : data, g.n, y.mp, g.mx, y.px, J, sp, S, tmode,
-                                          tkind, partials, gk);
+                                          tkind, partials, gk, contiguous ? g.mx : y.px,
+                                          g.m);
   prof_end(st);
   return cudaGetLastError();
 }
@@ -959,14 +967,23 @@ cudaError_t yz_pass(int axis, Tc *&cur, Tc *&oth, const Geom &g, const PrecPlan 
 
 // The time DST alone (the P_theta paths with varying a): tensor cores in float32 when the plan has
 // the S_n image, else the FFMA/DFMA kernel.
-// in -> out (the same array, or one that does not overlap).
+// in -> out (the same array, or one that does not overlap), or to a caller's contiguous `user` where it
+// is given: the FFMA kernel writes it, the tensor cores' result is copied there.
 template <class Tc>
 cudaError_t time_single(Tc *in, Tc *out, const Geom &g, const PrecPlan &pp, State *S,
-                        double *partials, int gk, int Jo, cudaStream_t st) {
-  if (sizeof(Tc) == sizeof(float) && pp.sop_t1 != nullptr)
-    return launch_time_tma_single(reinterpret_cast<const float *>(in),
-                                  reinterpret_cast<float *>(out), g, pp.sop_t1, S, gk, st);
-  return launch_time<Tc>(in, g, spec_of<Tc>(pp), S, TM_NONE, 1, partials, gk, Jo, st, out);
+                        double *partials, int gk, int Jo, cudaStream_t st, Tc *user = nullptr) {
+  if constexpr (sizeof(Tc) == sizeof(float)) {
+    if (pp.sop_t1 != nullptr) {
+      const cudaError_t e = launch_time_tma_single(in, out, g, pp.sop_t1, S, gk, st);
+      if (e != cudaSuccess || !user) return e;
+      prof_begin(KC_AUX, st);
+      k_unpad<<<152 * 8, kNT, 0, st>>>((unsigned)((long long)g.n * g.my * g.mz), g.mx, g.px, out, user);
+      prof_end(st);
+      return cudaGetLastError();
+    }
+  }
+  return launch_time<Tc>(in, g, spec_of<Tc>(pp), S, TM_NONE, 1, partials, gk, Jo, st,
+                         user ? user : out, user != nullptr);
 }
 
 // P_theta with a varying 2D/3D coefficient: time DST, pp.cheb Chebyshev steps per frequency, time
@@ -974,7 +991,7 @@ cudaError_t time_single(Tc *in, Tc *out, const Geom &g, const PrecPlan &pp, Stat
 // last step leaves its iterate in R, from which the inverse time DST writes zc).
 template <class Tc, class Src>
 cudaError_t cheb_stages(const Geom &g, const PrecPlan &pp, Src src, Tc *zc, State *S, int tmode,
-                        double *partials, cudaStream_t st, cudaEvent_t after_time) {
+                        double *partials, cudaStream_t st, cudaEvent_t after_time, Tc *user) {
   using Arr = SrcArray<Tc, Tc>;
   const int gk = gate_kind_of(tmode);
   const Spec<Tc> &sp = spec_of<Tc>(pp);
@@ -1060,7 +1077,7 @@ cudaError_t cheb_stages(const Geom &g, const PrecPlan &pp, Src src, Tc *zc, Stat
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if (after_time && (e = cudaEventRecord(after_time, st)) != cudaSuccess) return e;
-  return time_single<Tc>(R, zc, g, pp, S, partials, gk, Jo, st);
+  return time_single<Tc>(R, zc, g, pp, S, partials, gk, Jo, st, user);
 }
 
 // The same source with double-float as its transform type.
@@ -1130,7 +1147,7 @@ cudaError_t prec_stages(const Geom &g, const PrecPlan &pp, Src src, Tout *z, Sta
   }
   if (pp.cheb)
     return cheb_stages<Tc>(g, pp, src, reinterpret_cast<Tc *>(z), S, tmode, partials, st,
-                           after_time);
+                           after_time, reinterpret_cast<Tc *>(user));
   if (pp.pcr) {
     // P_theta with a varying 1D coefficient: time DST, tridiagonal solves, time DST
     Tc *zc = reinterpret_cast<Tc *>(z);
@@ -1152,7 +1169,7 @@ cudaError_t prec_stages(const Geom &g, const PrecPlan &pp, Src src, Tout *z, Sta
     prof_end(st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (after_time && (e = cudaEventRecord(after_time, st)) != cudaSuccess) return e;
-    return time_single<Tc>(zc, zc, g, pp, S, partials, gk, Jo, st);
+    return time_single<Tc>(zc, zc, g, pp, S, partials, gk, Jo, st, reinterpret_cast<Tc *>(user));
   }
   const long long nx = (long long)g.n * g.my * g.mz;
   Tc *zt = reinterpret_cast<Tc *>(z);
@@ -1196,19 +1213,12 @@ cudaError_t launch_prec(const Geom &g, const PrecPlan &pp, const Tin *v, Tout *z
   return prec_stages<Tc>(g, pp, SrcArray<Tc, Tin>{v}, z, S, tmode, partials, st);
 }
 
-// z = P^-1 v in float32 into a caller's contiguous vector, by way of the padded scratch: the last x
-// pass writes it, or (the P_theta paths that end with a time transform) a copy.
+// z = P^-1 v in float32 into a caller's contiguous vector, by way of the padded scratch: the last pass
+// leaves the padding out.
 cudaError_t launch_prec_user(const Geom &g, const PrecPlan &pp, const double *v, float *scratch,
                              float *out, State *S, double *partials, cudaStream_t st) {
-  const bool direct = !pp.cheb && !pp.pcr;
-  cudaError_t e = prec_stages<float>(g, pp, SrcArray<float, double>{v}, scratch, S, TM_NONE,
-                                     partials, st, nullptr, direct ? out : nullptr);
-  if (e != cudaSuccess || direct) return e;
-  prof_begin(KC_AUX, st);
-  k_unpad<<<152 * 8, kNT, 0, st>>>((unsigned)((long long)g.n * g.my * g.mz), g.mx, g.px, scratch,
-                                   out);
-  prof_end(st);
-  return cudaGetLastError();
+  return prec_stages<float>(g, pp, SrcArray<float, double>{v}, scratch, S, TM_NONE, partials, st,
+                            nullptr, out);
 }
 
 // One MINRES iteration's preconditioner pass with the Lanczos step fused into its first stage:
