@@ -539,11 +539,9 @@ size_t cheb_coef_bytes(const Geom &g, int deg) {
 // left of a line; 256 bytes keep the vectors aligned)
 constexpr size_t kZGuard = 64;
 
-// The z vectors of a mixed handle: one allocation for the whole ring.  Each takes Np slots; the
-// padding of a full ring is counted whatever the group, so every further pending z costs N floats.
+// The z vectors of a mixed handle: one allocation for the whole ring, Np slots each.
 size_t zslab_floats(const Geom &g, int ugroup) {
-  return kZGuard + (size_t)(ugroup + 1) * (size_t)g.N +
-         (size_t)(kUpdRing + 1) * (size_t)(g.Np - g.N);
+  return kZGuard + (size_t)(ugroup + 1) * (size_t)g.Np;
 }
 
 // The axes of a mixed handle that the tensor-core transforms take (st_dst_tma.cu): 32-column tiles
@@ -580,7 +578,11 @@ size_t workspace_bytes(const Geom &g, bool mixed, int cheb, int ugroup) {
   size_t b = 0;
   if (cheb) b += cheb_coef_bytes(g, cheb) + 5 * N * sizeof(double);
   b += 2 * Nv * sizeof(double);                            // V
-  b += mixed ? zslab_floats(g, ugroup) * sizeof(float) : 2 * N * sizeof(double);  // Z
+  // Z: the padding of a full ring is counted whatever the group, so that every further pending z adds N
+  // floats (an upper bound for the smaller groups)
+  b += mixed ? zslab_floats(g, ugroup) * sizeof(float) +
+                   (size_t)(kUpdRing - ugroup) * (size_t)(g.Np - g.N) * sizeof(float)
+             : 2 * N * sizeof(double);
   b += 2 * Nv * sizeof(double);                            // D
   b += Nv * sizeof(double);                                // q
   if (mixed) b += Nv * sizeof(df);                         // x accumulator
