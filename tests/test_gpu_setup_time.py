@@ -19,7 +19,8 @@ def _setup(P, spec):
     return best
 
 
-# 1.35: the rest of the set-up is 0.3 ms here, a 400 KB image filled and copied by the host 0.35 ms
+# 0.2 ms: filled and copied by the host an image took 0.28 to 0.46 ms; a launch and a larger table
+# allocation are below 0.1
 @pytest.mark.parametrize("mx,n,precision", [(255, 200, "fp64"), (255, 255, "fp64"), (63, 300, "mixed")])
 def test_setup_with_and_without_tensor_cores(monkeypatch, mx, n, precision):
     import paper_2201_10062_gb300 as P
@@ -30,4 +31,4 @@ def test_setup_with_and_without_tensor_cores(monkeypatch, mx, n, precision):
     spec = P.ProblemSpec(1, mx, 1, n, 1.0, "theta", 0.5, None, "PH", precision)
     on = _setup(P, spec)
     monkeypatch.setenv("ST_DISABLE_TENSOR_CORES", "1")
-    assert on <= 1.35 * _setup(P, spec)
+    assert on <= _setup(P, spec) + 2e-4
