@@ -11,7 +11,9 @@
 // pieces (hi + lo, 22 bits); hi*hi + hi*lo + lo*hi accumulate in float32 in tensor memory.  Columns
 // of B are scaled by a power of two so that fp16 keeps its range; S is scaled by 8.
 //
-// What bounds these passes is not the MMAs but the instructions and the latency around them, so:
+// What bounds these passes is the latency of a tile's way through the roles (ncu, 255^2 x 256: issue
+// slots 51% busy in the time stage and 31% in a y or x pass, tensor pipe 20%, DRAM 14% and 30%; the
+// stalls are waits for tensor memory and for the role before).  So:
 //   - a tile is loaded by one thread with a few tensor copies (128-byte-swizzled boxes of 32
 //     floats), two or more tiles ahead, into a ring of buffers; its result is written back into
 //     the buffer it came from and leaves by tensor copies as well.  No thread computes a global
@@ -24,8 +26,8 @@
 //     parities (and for h <= 32 two halves of the groups as well) are stacked in the 128 rows of
 //     the MMA: slot s holds its rows of A and zeros elsewhere, every slot's product accumulates into
 //     the same accumulator columns, and every thread of the epilogue has 64 values to take out;
-//   - MMAs are issued under elect.sync (see elect_one): under `lane == 0` their issue alone took 2400
-//     cycles a tile.  Two accumulators share the K steps (see issue_pair).
+//   - MMAs are issued under elect.sync (see elect_one); two accumulators share the K steps (see
+//     issue_pair).
 // S (all slots, hi and lo) stays in tensor memory for the whole launch; one block per SM walks the
 // tiles with its warps in separate roles that hand off through mbarriers, every wait bounded.  On a
 // timeout the block records ST_ERR_TIMEOUT and stops; before it frees its tensor memory every MMA
@@ -607,7 +609,8 @@ __global__ void __launch_bounds__(kNTS, 1)
 // buffer; one unit each), epilogue 2 (the result into the buffer), two of build 1, two of build 2, and
 // one for the MMA threads of the two transforms, the loads and the stores.  The builds hold 32 folded
 // values a thread and take their registers from the other groups (kRegs*; their sum stays within the
-// 8 x 64 of the launch), as with equal shares they spill.
+// 8 x 64 of the launch), as with equal shares they spill more (now 4 to 64 bytes, in most of the nine
+// instantiations).
 constexpr int kNTT = 32 * 32, kMiscWarpT = 28, kLoadWarpT = 30, kStoreWarpT = 31;
 constexpr int kRegsLaunch = 64, kRegsEpi = 56, kRegsBuild = 72, kRegsMisc = 56;
 static_assert(3 * kRegsEpi + 4 * kRegsBuild + kRegsMisc <= 8 * kRegsLaunch, "register split");

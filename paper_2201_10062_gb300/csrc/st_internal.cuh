@@ -340,8 +340,8 @@ struct PrecPlan {
   const unsigned short *sop;  // fp16 S_n operand image for the tensor-core time kernel, or null
   const unsigned short *sop_y;  // fp16 S_my image for the tensor-core y-DST (2D/3D mixed), or null
   const unsigned short *sop_z;  // fp16 S_mz image for the tensor-core z-DST (3D mixed), or null
-  const unsigned short *sop_x;  // fp16 S_mx image for the tensor-core x-DST of the last spatial
-                                // pass (mixed), or null
+  const unsigned short *sop_x;  // fp16 S_mx image for the tensor-core x-DST (mixed: the last spatial
+                                // pass, and both of the P_theta inner map), or null
   // operand images of the axes of 257 to 512 points (mixed), or null, and the float32 vector (the
   // stencil output's room, free once the Lanczos step has read it) their transforms go through
   const unsigned short *sop_long, *sop_ly, *sop_lz;

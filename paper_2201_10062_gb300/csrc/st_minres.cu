@@ -951,10 +951,10 @@ int build_tables(st_handle *h) {
   h->tc_time_img = pp.sop;
   h->tc_y_img = pp.sop_y;
   h->tc_z_img = pp.sop_z;
-  // The last x pass runs on the tensor cores where mx + 1 allows (41.8 against 61.1 us per pass
-  // for the FFT at 255^2 x 256); st_autotune times both, and ST_X_TENSOR_CORES=0 starts a handle
-  // with the FFT.  The P_theta paths with varying a run their x passes through the Chebyshev and
-  // PCR kernels.
+  // The last x pass runs on the tensor cores where mx + 1 allows (27 against 61 us per pass for the FFT
+  // at 255^2 x 256; below 2^21 unknowns the FFT is 1 to 3 us faster); st_autotune times both, and
+  // ST_X_TENSOR_CORES=0 starts a handle with the FFT.  So do the x passes of the P_theta inner map in 2D
+  // and 3D; the 1D one (PCR) has none.
   h->tc_x_img = (sopx == 0 || pp.pcr)
                     ? nullptr
                     : reinterpret_cast<const unsigned short *>((const char *)h->tables + o_sopx);

@@ -489,7 +489,8 @@ struct SrcChebScale {
   unsigned m, mx;
   __device__ __forceinline__ void prepare(const State *) {}
   __device__ __forceinline__ Tc operator()(long long i) const {
-    const unsigned e = (unsigned)i;  // N < 2^31 for every accepted size
+    // N < 2^31 for every accepted size, and padded Np <= 4/3 N < 2^32: unsigned, not int
+    const unsigned e = (unsigned)i;
     const unsigned k = e / m, r = e - k * m;
     const unsigned jy = r / mx, ix = r - jy * mx;
     return w[i] * s[k] / (lh[k] + lht[k] * (mux[ix] + muy[jy]));
@@ -887,8 +888,8 @@ const float *cheb_s_of<float>(const PrecPlan &pp) {
 
 constexpr int kChebBlocks = 152 * 8;
 
-// Spatial DST-I along y (lines mx apart, planes of mx*my, n*mz of them) or z (lines mx*my apart,
-// planes of m, n of them), from src into out: the tensor cores in float32 when the plan has the
+// Spatial DST-I along y (elements one x line apart, n*mz planes) or z (elements one plane of x lines
+// apart, n levels; px slots a line in the padded layout), from src into out: the tensor cores in float32 when the plan has the
 // S_len image, else the shared-memory FFT.  Tensor-core passes work in place (src must be out).
 template <class Tc, class Src>
 cudaError_t dst_y_pass(Src src, Tc *out, const Geom &g, const PrecPlan &pp, State *S, int gk,

@@ -510,7 +510,7 @@ __global__ void __launch_bounds__(kNT, df_blocks(DIM, UNI)) k_stencil_df(Geom g,
         const df2 x = A.get();
         const f2 np = cw.nhi * x.hi;
         const f2 r = fma2(cw.hi, x.lo, fma2(cw.lo, x.hi, fma2(cw.hi, x.hi, np)));
-        return df2{O - np, r};  // r is far below an ulp of the product: no normalisation
+        return df2{O - np, r};  // r is an ulp of the product or so: the sums it enters take it as it is
       }
       acc2 A{O, O};
       face(A, cw, q.c, w);

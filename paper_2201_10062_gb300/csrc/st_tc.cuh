@@ -56,9 +56,8 @@ __device__ __forceinline__ void mma_commit(uint32_t mbar) {
 }
 
 // one lane of a converged warp.  The compiler knows a region under elect.sync to run in a single
-// thread and keeps MMA operands in uniform registers: one tcgen05.mma of N = 32 then issues every 16
-// cycles (the tensor pipe's own rate), against 45 under `lane == 0`, where each operand is moved
-// there first.
+// thread, and a tcgen05.mma then takes fewer instructions to issue than under `lane == 0`
+// (k_time_tcd at 255^2 x 256: 763 against 617 us a time stage).
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
   asm volatile(
