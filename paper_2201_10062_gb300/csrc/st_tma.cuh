@@ -29,8 +29,8 @@ __device__ __forceinline__ uint64_t make_desc_sbo(uint32_t saddr, uint32_t sbo) 
 // of the float32 kernels.  So the K steps go half and half to the two accumulators, whose sum is
 // rounded, and the small products (A_hi B_lo, A_lo B_hi: 2^-11 of the large ones, and cut off that much
 // lower) come before the large ones of the second; axes beyond 256 take two pairs.  Against float64 the
-// largest and the root mean square error are then 0.9 of the float32 kernels' in the mean over 738
-// sizes, schemes and inputs.  In the first half A_hi meets B_hi and B_lo in one MMA of twice the width.
+// root mean square and the largest error are then 0.95 of the float32 kernels' in the geometric mean
+// over 510 sizes, schemes and inputs.  In the first half A_hi meets B_hi and B_lo in one MMA of twice the width.
 // What this costs is the issue of the further MMAs (time stage at 255^2 x 256: 53.4 us with one
 // accumulator and 55.4 now; 511 x 127 x 365: 80.7 and 84.3 a launch; y at 511^2 x 128: 77 and 80), so the
 // conditions and operands of a step are shared where two pairs go together (pair after pair, the time
